@@ -92,96 +92,264 @@ __device__ __forceinline__ void conv_epilogue4(const ConvArgs &a, int b, int y, 
 }
 
 // ---- CUDA-core implicit-GEMM convolution ---------------------------------------------------------
-// CTA tile: 8x8 output pixels x 64 output channels; K slices of 16 channels of one tap.
-// 256 threads, each 4 pixels x 4 channels, FP32 accumulation.
-template <typename T>
-__global__ void __launch_bounds__(256) conv_simt_kernel(ConvArgs a) {
-  __shared__ __align__(16) float As[16][68];
-  __shared__ __align__(16) float Bs[16][68];
-  const int tilesX = (a.Wb + 7) >> 3, tilesY = (a.Hb + 7) >> 3;
-  int t = blockIdx.x;
-  const int tx = t % tilesX;
-  t /= tilesX;
-  const int ty = t % tilesY;
-  const int b = t / tilesY;
-  const int n0 = blockIdx.y * 64;
-  const int tid = threadIdx.x;
-  const int tp = tid & 15, tc = tid >> 4;
-  const int lp = tid >> 2, lc = (tid & 3) * 4;
-  const int py = ty * 8 + (lp >> 3), px = tx * 8 + (lp & 7);
-  const int bn = tid >> 2, bk = (tid & 3) * 4;
-  float acc[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; i++)
-#pragma unroll
-    for (int j = 0; j < 4; j++) acc[i][j] = 0.f;
+// CTA tile: BM output pixels x BN output channels, TM x TN per thread; K slices of BK channels of
+// one tap, double-buffered in shared memory, the next slice in flight to registers while one is
+// multiplied (one barrier per slice). Every output is one chain of FP32 FMAs in tap, channel, then
+// phase-2 order whatever the tile, so all tiles give the same bits.
+//
+// Bound: the FP32 FMA pipe (128 lanes per SM and clock) and, close behind, the shared-memory
+// reads: a 16-byte read returns 512 bytes to a warp's registers at 128 bytes per clock, broadcast
+// or not, so one K step of a warp costs TM + TN clocks of reads against TM TN / 4 of FMAs: 8 : 4 at
+// 4 x 4 per thread, 16 : 16 at 8 x 8, 24 : 32 at 8 x 16. The FMAs are packed pairs (fma.rn.f32x2:
+// two IEEE FMAs per lane, adjacent channels of one pixel), which frees the issue slots for the
+// rest. Pixels are a run of a rectangle in row-major order (the launch's tile list, or the flat
+// buffer), so only a rectangle's last tile is partly idle. Measured against the 8 x 8 pixel x 64
+// channel tile with 4 x 4 per thread it replaced: 64 -> 64 channels at 16 x 368 x 368: 4,330 ->
+// 3,040 us; 256 -> 256 with a phase 2 of 256 at 16 x 92 x 92: 5,150 -> 3,080 us (58 TFLOP/s);
+// 512 -> 512 at 94 x 126: 1,675 -> 1,055 us; at 4 x 4 pixels: 199 -> 78 us.
+//
+// Slice layout: As[k][px ^ SW (k/4 % Q)], Bs[k][ch ^ SW (k/4 % Q)], Q = BK / 4 channel quads,
+// SW = 32 / Q. 32 / Q pixels x Q quads make one warp's load instruction (4 BK contiguous bytes per
+// pixel); the XOR puts the quads of the transposing stores on different banks, and leaves
+// 4-element groups whole for the 16-byte reads. It moves elements within groups of 32, so BM and
+// BN are multiples of 32.
+__device__ __forceinline__ void fma2(unsigned long long &d, unsigned long long a,
+                                     unsigned long long b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ unsigned long long dup2(float v) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(v));
+  return r;
+}
 
-  auto mac = [&]() {
-#pragma unroll
-    for (int k = 0; k < 16; k++) {
-      float4 av = *reinterpret_cast<const float4 *>(&As[k][tp * 4]);
-      float4 bv = *reinterpret_cast<const float4 *>(&Bs[k][tc * 4]);
-      float ar[4] = {av.x, av.y, av.z, av.w}, br[4] = {bv.x, bv.y, bv.z, bv.w};
-#pragma unroll
-      for (int i = 0; i < 4; i++)
-#pragma unroll
-        for (int j = 0; j < 4; j++) acc[i][j] = fmaf(ar[i], br[j], acc[i][j]);
+template <typename T, int BM, int BN, int TM, int TN, int BK, int MINB>
+__global__ void __launch_bounds__((BM / TM) * (BN / TN), MINB) conv_simt_kernel(ConvArgs a) {
+  constexpr int NT = (BM / TM) * (BN / TN);           // threads
+  constexpr int Q = BK / 4, SW = 32 / Q;              // channel quads of a slice, swizzle step
+  constexpr int LA = BM * Q / NT, LB = BN * Q / NT;   // quads each thread loads per slice
+  // a warp covers (8 TM) pixels x (4 TN) channels; a thread's pixels and channels come in groups
+  // of 4, 32 pixels / 16 channels apart
+  constexpr int WN = BN / (4 * TN);                   // warps along the channels
+  constexpr int PG = TM < 4 ? TM : 4;                 // pixels per group
+  constexpr int GM = TM / PG, GN = TN / 4;
+  static_assert(LA * NT == BM * Q && LB * NT == BN * Q && BM % (8 * TM) == 0 &&
+                BN % (4 * TN) == 0 && BM % 32 == 0 && BN % 32 == 0 && 32 % Q == 0,
+                "convolution tile");
+  __shared__ __align__(16) float As[2][BK][BM];
+  __shared__ __align__(16) float Bs[2][BK][BN];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int n0 = blockIdx.y * BN;
+  // this CTA's run of pixels: entry {block, first pixel, y0 << 16 | x0, height << 16 | width} of
+  // the tile list, or pixels blockIdx.x BM .. of the whole buffer
+  int rb = 0, q0 = blockIdx.x * BM, ry = 0, rx = 0, rh = a.B * a.Hb, rw = a.Wb;
+  if (a.tiles) {
+    const int4 e = a.tiles[blockIdx.x];
+    rb = e.x;
+    q0 = e.y;
+    ry = (int)((unsigned)e.z >> 16);
+    rx = e.z & 0xffff;
+    rh = (int)((unsigned)e.w >> 16);
+    rw = e.w & 0xffff;
+  }
+  const int rn = rh * rw;
+  // pixel p of the run -> (block, y, x); false past the rectangle. (Without a list the rectangle
+  // is all B blocks' rows, Hb per block.)
+  auto pixel = [&](int p, int &b, int &y, int &x) -> bool {
+    const int q = q0 + p;
+    if (q >= rn) return false;
+    y = q / rw;
+    x = rx + q - y * rw;
+    y += ry;
+    b = rb;
+    if (!a.tiles) {
+      b = y / a.Hb;
+      y -= b * a.Hb;
     }
+    return true;
+  };
+  const int lc = (tid % Q) * 4;   // first channel of the quads this thread loads
+  int ly[LA], lx[LA], lo[LA];     // their pixels
+#pragma unroll
+  for (int i = 0; i < LA; i++) {
+    int b = 0, y = 0, x = 0;
+    const bool in = pixel(tid / Q + i * (NT / Q), b, y, x);
+    ly[i] = in ? y : -4;   // out of the buffer under every tap
+    lx[i] = x;
+    lo[i] = (b * a.Hb + y) * a.Wb + x;
+  }
+  const T *A = reinterpret_cast<const T *>(a.A), *A2 = reinterpret_cast<const T *>(a.A2);
+  const T *Wt = reinterpret_cast<const T *>(a.Wt), *W2 = reinterpret_cast<const T *>(a.W2);
+  const int n_main = a.taps * (a.cin / BK), n_slices = n_main + a.k2 / BK;
+
+  float va[LA][4], vb[LB][4];   // the slice in flight
+  // slices are loaded in order: the main phase tap by tap, channels ascending, then phase 2
+  int ls = 0, tap = 0, c = lc, dy = -1, dx = -1;
+  const T *wrow = Wt + (size_t)(n0 + tid / Q) * a.taps * a.cin;
+  auto load = [&]() {
+    if (ls < n_main) {
+#pragma unroll
+      for (int i = 0; i < LA; i++) {
+        const int y = ly[i] + dy, x = lx[i] + dx;
+        if (y >= 0 && y < a.Hb && x >= 0 && x < a.Wb)
+          load4(A + (size_t)(lo[i] + dy * a.Wb + dx) * a.cin + c, va[i]);
+        else
+          va[i][0] = va[i][1] = va[i][2] = va[i][3] = 0.f;
+      }
+#pragma unroll
+      for (int i = 0; i < LB; i++)
+        load4(wrow + (size_t)(i * (NT / Q) * a.taps + tap) * a.cin + c, vb[i]);
+      c += BK;
+      if (c >= a.cin) {
+        c = lc;
+        tap++;
+        if (++dx == 2) { dx = -1; dy++; }
+      }
+    } else {
+      const int c2 = (ls - n_main) * BK + lc;
+#pragma unroll
+      for (int i = 0; i < LA; i++) {
+        if (ly[i] >= 0)
+          load4(A2 + (size_t)lo[i] * a.k2 + c2, va[i]);
+        else
+          va[i][0] = va[i][1] = va[i][2] = va[i][3] = 0.f;
+      }
+#pragma unroll
+      for (int i = 0; i < LB; i++)
+        load4(W2 + (size_t)(n0 + tid / Q + i * (NT / Q)) * a.k2 + c2, vb[i]);
+    }
+    ls++;
+  };
+  const int sw = (tid % Q) * SW;   // the swizzle of this thread's quads
+  auto store = [&](int buf) {
+#pragma unroll
+    for (int i = 0; i < LA; i++)
+#pragma unroll
+      for (int j = 0; j < 4; j++) As[buf][lc + j][(tid / Q + i * (NT / Q)) ^ sw] = va[i][j];
+#pragma unroll
+    for (int i = 0; i < LB; i++)
+#pragma unroll
+      for (int j = 0; j < 4; j++) Bs[buf][lc + j][(tid / Q + i * (NT / Q)) ^ sw] = vb[i][j];
   };
 
-  const T *A = reinterpret_cast<const T *>(a.A);
-  const T *Wt = reinterpret_cast<const T *>(a.Wt);
-  for (int tap = 0; tap < a.taps; tap++) {
-    const int y = py + tap / 3 - 1, x = px + tap % 3 - 1;
-    const bool in = y >= 0 && y < a.Hb && x >= 0 && x < a.Wb;
-    const T *arow = A + (((size_t)b * a.Hb + y) * a.Wb + x) * a.cin;
-    const T *brow = Wt + ((size_t)(n0 + bn) * a.taps + tap) * a.cin;
-    for (int c0 = 0; c0 < a.cin; c0 += 16) {
-      float v[4] = {0.f, 0.f, 0.f, 0.f};
-      if (in) load4(arow + c0 + lc, v);
+  const int p0 = (warp / WN) * 8 * TM + (lane >> 2) * PG;   // this thread's first pixel / channel
+  const int c0 = (warp % WN) * 4 * TN + (lane & 3) * 4;
+  unsigned long long acc[TM][TN / 2];   // [pixel][channel pair]
 #pragma unroll
-      for (int j = 0; j < 4; j++) As[lc + j][lp] = v[j];
-      float w[4];
-      load4(brow + c0 + bk, w);
+  for (int i = 0; i < TM; i++)
 #pragma unroll
-      for (int j = 0; j < 4; j++) Bs[bk + j][bn] = w[j];
-      __syncthreads();
-      mac();
-      __syncthreads();
+    for (int j = 0; j < TN / 2; j++) acc[i][j] = 0ull;
+
+  load();
+  store(0);
+  if (n_slices > 1) load();
+  __syncthreads();
+  for (int s = 0; s < n_slices; s++) {
+    const int buf = s & 1;
+#pragma unroll
+    for (int k = 0; k < BK; k++) {
+      const int x = ((k >> 2) % Q) * SW;
+      float ar[TM];
+      ulonglong2 bv[GN];
+#pragma unroll
+      for (int g = 0; g < GM; g++) {
+        const float *p = &As[buf][k][(p0 + 8 * PG * g) ^ x];
+        if constexpr (PG == 4) {
+          const float4 t = *reinterpret_cast<const float4 *>(p);
+          ar[4 * g] = t.x; ar[4 * g + 1] = t.y; ar[4 * g + 2] = t.z; ar[4 * g + 3] = t.w;
+        } else {
+          const float2 t = *reinterpret_cast<const float2 *>(p);
+          ar[2 * g] = t.x; ar[2 * g + 1] = t.y;
+        }
+      }
+#pragma unroll
+      for (int g = 0; g < GN; g++)
+        bv[g] = *reinterpret_cast<const ulonglong2 *>(&Bs[buf][k][(c0 + 16 * g) ^ x]);
+#pragma unroll
+      for (int i = 0; i < TM; i++) {
+        const unsigned long long ad = dup2(ar[i]);
+#pragma unroll
+        for (int j = 0; j < GN; j++) {
+          fma2(acc[i][2 * j], ad, bv[j].x);
+          fma2(acc[i][2 * j + 1], ad, bv[j].y);
+        }
+      }
+    }
+    if (s + 1 < n_slices) {
+      store(buf ^ 1);
+      if (s + 2 < n_slices) load();
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int i = 0; i < TM; i++) {
+    int b, y, x;
+    if (!pixel(p0 + (i / PG) * 8 * PG + i % PG, b, y, x)) continue;
+#pragma unroll
+    for (int g = 0; g < GN; g++) {
+      float v[4];
+#pragma unroll
+      for (int j = 0; j < 4; j++) {
+        const unsigned long long t = acc[i][2 * g + (j >> 1)];
+        v[j] = __uint_as_float((unsigned)((j & 1) ? t >> 32 : t));
+      }
+      conv_epilogue4<T>(a, b, y, x, n0 + c0 + 16 * g, v);
     }
   }
-  if (a.k2 > 0) {
-    const T *A2 = reinterpret_cast<const T *>(a.A2);
-    const T *W2 = reinterpret_cast<const T *>(a.W2);
-    const bool in = py < a.Hb && px < a.Wb;
-    const T *arow = A2 + (((size_t)b * a.Hb + py) * a.Wb + px) * a.k2;
-    const T *brow = W2 + (size_t)(n0 + bn) * a.k2;
-    for (int c0 = 0; c0 < a.k2; c0 += 16) {
-      float v[4] = {0.f, 0.f, 0.f, 0.f};
-      if (in) load4(arow + c0 + lc, v);
-#pragma unroll
-      for (int j = 0; j < 4; j++) As[lc + j][lp] = v[j];
-      float w[4];
-      load4(brow + c0 + bk, w);
-#pragma unroll
-      for (int j = 0; j < 4; j++) Bs[bk + j][bn] = w[j];
-      __syncthreads();
-      mac();
-      __syncthreads();
-    }
+}
+
+template <typename T, int BM, int BN, int TM, int TN, int BK, int MINB>
+static void launch_simt_tile(const ConvArgs &a, cudaStream_t s) {
+  const long long px = (long long)a.B * a.Hb * a.Wb;
+  const int nt = a.tiles ? a.n_mtiles : (int)((px + BM - 1) / BM);
+  if (nt <= 0) return;
+  conv_simt_kernel<T, BM, BN, TM, TN, BK, MINB>
+      <<<dim3(nt, a.cout / BN), (BM / TM) * (BN / TN), 0, s>>>(a);
+}
+
+// Tile of a launch over px pixels. Large launches take the tile with the fewest shared-memory
+// reads per FMA; the smaller ones trade that for CTAs (152 SMs). Times in us, start of the line =
+// the launch (pixels, channels in -> out):
+//                          128x128  64x64   64x64   32x32   32x32
+//                          8x16     8x8     4x8     4x4     2x4
+//   33,856  512 -> 512     2,771    2,900   3,326   4,184   6,303
+//    9,248  256 -> 256     266      246     273     343     512
+//   18,786  128 -> 64      -        72      68      86      121
+//    4,096  128 -> 128     124      68      41      45      64
+//    3,960  64 -> 64       -        43      26      19      21
+//      884  512 -> 256     464      242     148     101     125
+//       16  512 -> 512     457      238     142     84      78
+// Between the first two the number of waves decides (304 and 608 CTAs run at once; the second has
+// a quarter of the first's work each, at 0.955 of its rate).
+SimtTile conv_simt_tile(long long px, int cin, int cout, int k2) {
+  if (cin % 32 || k2 % 32) return kSimt64x64k16;
+  const long long n64 = (px + 63) / 64 * (cout / 64), n32 = (px + 31) / 32 * (cout / 32);
+  if (n32 <= 152) return kSimt32x32t2;
+  if (n64 < 100) return kSimt32x32;
+  if (n64 <= 304) return kSimt64x64t4;
+  if (cout % 128 == 0) {
+    const double w128 = (double)((px + 127) / 128 * (cout / 128)) / 304, w64 = (double)n64 / 608;
+    const double c128 = w128 <= 1 ? 1.0 : w128 + 0.3, c64 = w64 <= 1 ? 1.0 : w64 + 0.3;
+    if (c128 <= 0.524 * c64) return kSimt128x128;
   }
-#pragma unroll
-  for (int i = 0; i < 4; i++) {
-    const int p = tp * 4 + i;
-    const int y = ty * 8 + (p >> 3), x = tx * 8 + (p & 7);
-    if (y < a.Hb && x < a.Wb) conv_epilogue4<T>(a, b, y, x, n0 + tc * 4, acc[i]);
-  }
+  return kSimt64x64;
+}
+int conv_simt_tile_px(SimtTile t) {
+  return t == kSimt128x128 ? 128 : t == kSimt32x32 || t == kSimt32x32t2 ? 32 : 64;
 }
 
 template <typename T>
 void launch_conv_simt(const ConvArgs &a, cudaStream_t s) {
-  dim3 grid(((a.Wb + 7) / 8) * ((a.Hb + 7) / 8) * a.B, a.cout / 64);
-  conv_simt_kernel<T><<<grid, 256, 0, s>>>(a);
+  const long long px = (long long)a.B * a.Hb * a.Wb;
+  // (with a tile list: the tile it was cut for)
+  switch (a.tiles ? (SimtTile)a.TW : conv_simt_tile(px, a.taps ? a.cin : 0, a.cout, a.k2)) {
+    case kSimt128x128: launch_simt_tile<T, 128, 128, 8, 16, 16, 2>(a, s); break;
+    case kSimt64x64: launch_simt_tile<T, 64, 64, 8, 8, 32, 4>(a, s); break;
+    case kSimt64x64t4: launch_simt_tile<T, 64, 64, 4, 8, 32, 2>(a, s); break;
+    case kSimt32x32: launch_simt_tile<T, 32, 32, 4, 4, 32, 4>(a, s); break;
+    case kSimt32x32t2: launch_simt_tile<T, 32, 32, 2, 4, 32, 2>(a, s); break;
+    case kSimt64x64k16: launch_simt_tile<T, 64, 64, 8, 8, 16, 6>(a, s); break;
+  }
 }
 template void launch_conv_simt<float>(const ConvArgs &, cudaStream_t);
 template void launch_conv_simt<__nv_bfloat16>(const ConvArgs &, cudaStream_t);

@@ -513,8 +513,6 @@ nst_status build_plan(nst_ctx *ctx, int H, int W, int margin, PassPlan **out) {
   auto add_list = [&](const Batch &bt, int level, int cin, int cout, int taps, int k2, bool pool,
                       auto pick) -> PatchList {
     PatchList pl{(int)patches.size(), 0, 0, 0};
-    int rows, fth, ftw;
-    conv_tc_patch_rule(cin, cout, taps, k2, pool, &rows, &fth, &ftw);
     std::vector<Iv> ry(bt.B), rx(bt.B);
     std::vector<int> hs(bt.B), wsz(bt.B);
     for (int j = 0; j < bt.B; j++) {
@@ -526,6 +524,23 @@ nst_status build_plan(nst_ctx *ctx, int H, int W, int margin, PassPlan **out) {
       hs[j] = std::max(0, ry[j].b - ry[j].a);
       wsz[j] = std::max(0, rx[j].b - rx[j].a);
     }
+    if (!ctx->use_tc) {
+      // CUDA cores: each rectangle's pixels in row-major order, cut into runs of one CTA tile
+      // (16-bit fields; a longer block side leaves TH = 0: the launch covers whole blocks)
+      if (p.Hb >= 65536 || p.Wb >= 65536) return pl;
+      long long px = 0;
+      for (int j = 0; j < bt.B; j++) px += (long long)hs[j] * wsz[j];
+      const SimtTile tile = conv_simt_tile(px, taps ? cin : 0, cout, k2);
+      pl.TH = conv_simt_tile_px(tile);
+      pl.TW = tile;
+      for (int j = 0; j < bt.B; j++)
+        for (int q = 0; q < hs[j] * wsz[j]; q += pl.TH)
+          patches.push_back(make_int4(j, q, ry[j].a << 16 | rx[j].a, hs[j] << 16 | wsz[j]));
+      pl.n = (int)patches.size() - pl.off;
+      return pl;
+    }
+    int rows, fth, ftw;
+    conv_tc_patch_rule(cin, cout, taps, k2, pool, &rows, &fth, &ftw);
     conv_tc_pick_patch(hs.data(), wsz.data(), bt.B, rows, fth, ftw, pool, &pl.TH, &pl.TW);
     for (int j = 0; j < bt.B; j++)
       for (int y = ry[j].a; y < ry[j].b; y += pl.TH)
@@ -676,9 +691,9 @@ nst_status ensure_buffers(nst_ctx *ctx, const PassPlan &p, Workspace &ws) {
 }
 
 // ---- convolution dispatch -----------------------------------------------------------------------
-// the tensor-core engine computes only the launch's patch list (the CUDA-core engine ignores it
-// and computes whole blocks, with the same values where the list's patches lie)
+// both engines compute only the launch's list: each block's needed rectangle
 void use_patches(ConvArgs &a, const PassPlan &p, const PatchList &pl) {
+  if (!pl.TH) return;   // no list: whole blocks
   a.tiles = p.d_patches + pl.off;
   a.n_mtiles = pl.n;
   a.TH = pl.TH;
@@ -689,8 +704,8 @@ nst_status run_conv(nst_ctx *ctx, ConvArgs a, cudaStream_t s) {
   a.err = ctx->d_err;
   ctx->launches++;
   ctx->conv_launches++;
-  const double px = ctx->use_tc && a.tiles ? (double)a.n_mtiles * a.TH * a.TW
-                                           : (double)a.B * a.Hb * a.Wb;
+  const double px = a.tiles ? (double)a.n_mtiles * a.TH * (ctx->use_tc ? a.TW : 1)
+                            : (double)a.B * a.Hb * a.Wb;
   ctx->conv_flops += 2.0 * px * a.cout * ((double)a.taps * a.cin + a.k2);
   Timer tm(ctx, kTConv, s);
   if (ctx->use_tc) {

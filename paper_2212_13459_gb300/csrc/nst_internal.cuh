@@ -81,7 +81,8 @@ struct ConvArgs {
   unsigned char *pool_idx;  // forward with pool_out: also the window positions of the maximum,
                             // 4 bits per pooled value ([B][Hb/2][Wb/2][cout] / 2 bytes), or null
   // tensor-core engine: the output patches to compute, one {block, y0, x0, 0} per patch (its
-  // origin in the block's [Hb][Wb] buffer), each TH x TW; null = every patch of the buffer
+  // origin in the block's [Hb][Wb] buffer), each TH x TW; null = every patch of the buffer.
+  // CUDA-core engine: runs of TH pixels of rectangles (see launch_conv_simt), TW = the CTA tile
   const int4 *tiles;
   int n_mtiles, TH, TW;
 };

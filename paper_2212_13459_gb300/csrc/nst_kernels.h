@@ -44,6 +44,16 @@ struct Conv11W {
 };
 
 // k_simt.cu
+// CTA tiles of the CUDA-core convolution (pixels x channels; t2 / t4: pixels per thread where the
+// plain name has more; k16: input channels that are a multiple of 16 but not of 32)
+enum SimtTile : int {
+  kSimt128x128, kSimt64x64, kSimt64x64t4, kSimt32x32, kSimt32x32t2, kSimt64x64k16
+};
+// the tile of a launch over px output pixels (cin = 0: no main phase), and its pixels
+SimtTile conv_simt_tile(long long px, int cin, int cout, int k2);
+int conv_simt_tile_px(SimtTile t);
+// a.tiles: entries {block, first pixel, y0 << 16 | x0, height << 16 | width}, one per CTA: that
+// many pixels (a.TH, those of tile a.TW) of the rectangle, in row-major order; null = whole buffers
 template <typename T> void launch_conv_simt(const ConvArgs &a, cudaStream_t s);
 template <typename T>
 void launch_conv11_fwd(const float *img, int H, int W, const Conv11W &cw, const BlockGeom *geom,
