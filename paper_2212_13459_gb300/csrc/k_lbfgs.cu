@@ -7,9 +7,12 @@
 //     the same matrix the two-loop recursion applies. A step reads every stored vector twice
 //     (one fused pass for all dot products, one pass forming the step) instead of four times;
 //     S^T Y and Y^T Y are kept up to date from the new pair's dot products. Dots are FP32 chunks
-//     summed in FP64 with fixed-order reductions; the small solve runs in FP64 on one thread.
+//     summed in compensated FP32 and FP64 with fixed-order reductions; the small solve runs in
+//     FP64 in one CTA.
 //     History slots are resolved on the device, so a step needs no host round trip.
 //   * bicubic x2 upscaling used to initialise each scale after the first (Algorithm 2).
+#include <type_traits>
+
 #include "nst_internal.cuh"
 #include "nst_kernels.h"
 #include "nst_lbfgs_dev.h"
@@ -27,43 +30,64 @@ static int dot_blocks(int m) {   // CTAs per group; fixed for a given m (reprodu
 int lbfgs_partials_count(int m) { return 4 * (m + 1) * dot_blocks(m); }
 
 // Position p of the fused pass: p = 0 is the candidate pair (spare slot: last step s and the new
-// y), p = 1 .. count the stored pairs order[p - 1]. partials[(4 p + q) * nb + cta] for the dots
-// q = 0: s.g, 1: y.g, 2: s.y_new, 3: y.y_new. Elements go four at a time (float4) when every
-// vector is 16-byte aligned, with all of an element group's loads issued before its FMAs.
+// y), p = 1 .. count the stored pairs order[p - 1]; c->dots[4 p + q], q = 0: s.g, 1: y.g,
+// 2: s.y_new, 3: y.y_new. Elements go four at a time (float4) when every vector is 16-byte
+// aligned, with all of an element group's loads issued before its FMAs.
+//
+// Bound: HBM (2 (count + 1) + 2 vectors read once). What kept it from there was the FP64 unit,
+// which retires two operations per SM and clock on this GPU: a double add (and a conversion) per
+// 16 elements and dot, and 80 double shuffle-adds per warp at the end. So a thread's FP32 chunks
+// are added in compensated FP32 (Sum): the error of the chunks themselves, about 2^-24 / sqrt(their
+// number), stays seven orders above that of adding them. The warp reduction is a reduce-scatter
+// (16 exchanges for 16 dots, not 80), and the last CTA of a group to finish adds the CTAs'
+// partials in FP64 in index order, in parallel over the groups, where the single CTA of the solve
+// spent 15 us on it. CTAs of all groups that read the same elements are neighbours in launch
+// order, so g and g_prev come from L2 for all but one of them. Measured with 100 stored pairs of
+// 2.29 M elements: 594 -> 345 us (5.4 TB/s); 10 pairs of 36.6 M: 634 us (5.8 TB/s).
+struct Sum {   // s + c: the sum with the rounding errors of its additions (Knuth's TwoSum)
+  float s, c;
+  __device__ __forceinline__ void add(float x) {
+    const float t = s + x, z = t - s;
+    c += (s - (t - z)) + (x - z);
+    s = t;
+  }
+  __device__ __forceinline__ void merge(float xs, float xc) {
+    add(xs);
+    c += xc;
+  }
+};
+
 template <int G>
 struct DotAcc {
-  double acc[G][4];
-  float part[G][4];
+  Sum acc[4 * G];
+  float part[4 * G];
   __device__ __forceinline__ void clear() {
 #pragma unroll
-    for (int j = 0; j < G; j++)
-#pragma unroll
-      for (int q = 0; q < 4; q++) acc[j][q] = 0.0, part[j][q] = 0.f;
+    for (int d = 0; d < 4 * G; d++) acc[d].s = acc[d].c = part[d] = 0.f;
   }
   __device__ __forceinline__ void flush() {
 #pragma unroll
-    for (int j = 0; j < G; j++)
-#pragma unroll
-      for (int q = 0; q < 4; q++) acc[j][q] += (double)part[j][q], part[j][q] = 0.f;
+    for (int d = 0; d < 4 * G; d++) acc[d].add(part[d]), part[d] = 0.f;
   }
   __device__ __forceinline__ void add(int j, float sv, float wv, float gv, float yv) {
-    part[j][0] = fmaf(sv, gv, part[j][0]);
-    part[j][1] = fmaf(wv, gv, part[j][1]);
-    part[j][2] = fmaf(sv, yv, part[j][2]);
-    part[j][3] = fmaf(wv, yv, part[j][3]);
+    part[4 * j] = fmaf(sv, gv, part[4 * j]);
+    part[4 * j + 1] = fmaf(wv, gv, part[4 * j + 1]);
+    part[4 * j + 2] = fmaf(sv, yv, part[4 * j + 2]);
+    part[4 * j + 3] = fmaf(wv, yv, part[4 * j + 3]);
   }
 };
 
 __global__ void __launch_bounds__(kDotThreads) lbfgs_dots_kernel(
     const float *__restrict__ g, const float *__restrict__ g_prev, const float *__restrict__ S,
-    float *__restrict__ Y, long long stride, long long n, const LbfgsCtl *__restrict__ c,
-    int first, int vec, double *__restrict__ partials) {
+    float *__restrict__ Y, long long stride, long long n, LbfgsCtl *c, int first, int vec,
+    double *partials) {
   constexpr int G = kLbGroup;
+  static_assert(4 * G == 16, "the warp reduce-scatter below takes 16 dots");
   __shared__ long long off[G];
-  __shared__ int nj_sh;
+  __shared__ int nj_sh, last_sh;
   __shared__ long long sp_off;
-  __shared__ double red[kDotThreads / 32][4 * G];
-  const int grp = blockIdx.y, nb = gridDim.x;
+  __shared__ Sum red[kDotThreads / 32][4 * G];
+  const int grp = blockIdx.x, nb = gridDim.y, cta = blockIdx.y;
   if (threadIdx.x == 0) {
     const int count = c->count;
     int nj = 0;
@@ -84,7 +108,7 @@ __global__ void __launch_bounds__(kDotThreads) lbfgs_dots_kernel(
   float *ynew = Y + sp_off;
   const bool own_y = grp == 0;   // group 0 holds the candidate (position 0) and writes its y
   const long long tstride = (long long)nb * kDotThreads;
-  const long long t0 = (long long)blockIdx.x * kDotThreads + threadIdx.x;
+  const long long t0 = (long long)cta * kDotThreads + threadIdx.x;
   DotAcc<G> A;
   A.clear();
   int chunk = 0;
@@ -92,7 +116,7 @@ __global__ void __launch_bounds__(kDotThreads) lbfgs_dots_kernel(
   for (long long v = t0; v < n4; v += tstride) {
     const float4 gv = reinterpret_cast<const float4 *>(g)[v];
     if (first) {
-      A.part[0][0] += fabsf(gv.x) + fabsf(gv.y) + fabsf(gv.z) + fabsf(gv.w);
+      A.part[0] += fabsf(gv.x) + fabsf(gv.y) + fabsf(gv.z) + fabsf(gv.w);
     } else {
       const float4 gp = reinterpret_cast<const float4 *>(g_prev)[v];
       const float4 yv = make_float4(gv.x - gp.x, gv.y - gp.y, gv.z - gp.z, gv.w - gp.w);
@@ -115,12 +139,12 @@ __global__ void __launch_bounds__(kDotThreads) lbfgs_dots_kernel(
         }
       }
     }
-    if (++chunk == 4) { chunk = 0; A.flush(); }   // FP32 over 16 elements, FP64 across chunks
+    if (++chunk == 4) { chunk = 0; A.flush(); }   // plain FP32 over 16 elements at most
   }
   for (long long i = n4 * 4 + t0; i < n; i += tstride) {   // scalar path / tail
     const float gv = g[i];
     if (first) {
-      A.part[0][0] += fabsf(gv);
+      A.part[0] += fabsf(gv);
     } else {
       const float yv = gv - g_prev[i];
       if (own_y) ynew[i] = yv;
@@ -131,127 +155,251 @@ __global__ void __launch_bounds__(kDotThreads) lbfgs_dots_kernel(
     if (++chunk == 16) { chunk = 0; A.flush(); }
   }
   A.flush();
-  // fixed-order block reduction: warp shuffles, then the warps in index order
+  // fixed-order block reduction. Reduce-scatter over the warp: at distance 2^b (b = 4 .. 1) a lane
+  // keeps the half of its dots whose index bit b - 1 equals its lane bit b and passes on the rest,
+  // so lane l ends with dot l >> 1, which lanes 2d and 2d + 1 then add
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  auto level = [&](auto bit) {
+    constexpr int b = decltype(bit)::value, h = 1 << (b - 1);
+    const bool up = (lane >> b) & 1;
 #pragma unroll
-  for (int j = 0; j < G; j++)
-#pragma unroll
-    for (int q = 0; q < 4; q++) {
-      double v = A.acc[j][q];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == 0) red[warp][j * 4 + q] = v;
+    for (int d = 0; d < h; d++) {
+      const Sum lo = A.acc[d], hi = A.acc[d + h];
+      A.acc[d].s = up ? hi.s : lo.s;
+      A.acc[d].c = up ? hi.c : lo.c;
+      A.acc[d].merge(__shfl_xor_sync(0xffffffffu, up ? lo.s : hi.s, 1 << b),
+                     __shfl_xor_sync(0xffffffffu, up ? lo.c : hi.c, 1 << b));
     }
+  };
+  level(std::integral_constant<int, 4>{});
+  level(std::integral_constant<int, 3>{});
+  level(std::integral_constant<int, 2>{});
+  level(std::integral_constant<int, 1>{});
+  A.acc[0].merge(__shfl_xor_sync(0xffffffffu, A.acc[0].s, 1),
+                 __shfl_xor_sync(0xffffffffu, A.acc[0].c, 1));
+  if (!(lane & 1)) red[warp][lane >> 1] = A.acc[0];
   __syncthreads();
-  if (threadIdx.x < 4 * nj) {
-    double v = 0.0;
-    for (int w = 0; w < kDotThreads / 32; w++) v += red[w][threadIdx.x];
-    const int d = grp * G * 4 + threadIdx.x;   // = 4 p + q
-    partials[(size_t)d * nb + blockIdx.x] = v;
+  if (threadIdx.x < 4 * nj) {   // the warps in index order
+    Sum v = red[0][threadIdx.x];
+    for (int w = 1; w < kDotThreads / 32; w++) v.merge(red[w][threadIdx.x].s, red[w][threadIdx.x].c);
+    partials[(size_t)(grp * G * 4 + threadIdx.x) * nb + cta] = (double)v.s + (double)v.c;
+    __threadfence();
   }
+  __syncthreads();
+  // the group's last CTA adds its partials: 16 lanes per dot, lane l the CTAs l, l + 16, ... in
+  // order, then a fixed tree
+  if (threadIdx.x == 0) last_sh = atomicAdd(&c->arrived[grp], 1u) == (unsigned)nb - 1;
+  __syncthreads();
+  if (!last_sh) return;
+  __threadfence();
+  const int d = threadIdx.x >> 4, l = threadIdx.x & 15;
+  double v = 0.0;
+  if (d < 4 * nj)
+    for (int q = l; q < nb; q += 16) v += __ldcg(partials + (size_t)(grp * G * 4 + d) * nb + q);
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if (l == 0 && d < 4 * nj) c->dots[grp * G * 4 + d] = v;
+  if (threadIdx.x == 0) c->arrived[grp] = 0u;
 }
 
 static bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
 void launch_lbfgs_dots(const float *g, const float *g_prev, const float *S, float *Y,
-                       long long stride, long long n, const LbfgsCtl *c, int m, int first,
+                       long long stride, long long n, LbfgsCtl *c, int m, int first,
                        double *partials, cudaStream_t s) {
-  dim3 grid(dot_blocks(m), first ? 1 : dot_groups(m));
   const int vec = aligned16(g) && aligned16(g_prev) && aligned16(S) && aligned16(Y) &&
                   stride % 4 == 0;
+  // no CTA without elements (a thread that has work has the same elements as with all CTAs)
+  const long long need = ((vec ? n / 4 : n) + kDotThreads - 1) / kDotThreads;
+  const int nb = (int)(need < 1 ? 1 : need < dot_blocks(m) ? need : dot_blocks(m));
+  dim3 grid(first ? 1 : dot_groups(m), nb);
   lbfgs_dots_kernel<<<grid, kDotThreads, 0, s>>>(g, g_prev, S, Y, stride, n, c, first, vec,
                                                  partials);
 }
 
-__global__ void __launch_bounds__(256) lbfgs_solve_kernel(LbfgsCtl *__restrict__ c,
-                                                          const double *__restrict__ partials,
-                                                          int nb, int m, int first, double eps,
-                                                          double *__restrict__ SY,
-                                                          double *__restrict__ YY) {
-  __shared__ double dots[4 * (kMaxHistory + 1)];
-  __shared__ double sg[kMaxHistory + 1], yg[kMaxHistory + 1];   // by slot
-  __shared__ double u[kMaxHistory], w[kMaxHistory], pv[kMaxHistory];
-  __shared__ int sl[kMaxHistory];
-  const int count0 = c->count;
-  const int nd = first ? 1 : 4 * (count0 + 1);
-  for (int d = threadIdx.x; d < nd; d += blockDim.x) {
-    double v = 0.0;
-    for (int b = 0; b < nb; b++) v += partials[(size_t)d * nb + b];   // fixed order
-    dots[d] = v;
-  }
-  __syncthreads();
-  if (threadIdx.x != 0) return;
+// The small solve: curvature test, bookkeeping, the two triangular systems and the coefficients
+// of the step, one CTA. k = stored pairs, oldest first; R = D Rs with D = diag R, Rs unit upper:
+//   u = Rs^-1 D^-1 (S^T g),  w = (D + gamma Y^T Y) u - gamma Y^T g,  p = D^-1 Rs^-T w.
+// Bound: latency, and the FP64 unit (two operations per SM and clock). Rs is scaled and kept in
+// shared memory; one warp runs both triangular systems column by column with the vector in
+// registers (lane l: rows l, l + 32, ...), so a column costs one shuffle and one FMA of latency;
+// Y^T Y is read into registers before the first system and used after it. One thread working from
+// global memory took 1,496 us at k = 100 and 58 us at k = 10; this takes 47 and 17 us (all
+// cold, under the profiler).
+constexpr int kSolveThreads = 512;
+constexpr int kSolveParts = kSolveThreads / kMaxHistory;          // threads per row of Y^T Y
+constexpr int kSolveRow = kMaxHistory / kSolveParts;              // its elements each holds
+static size_t solve_smem(int m) { return (size_t)m * (m | 1) * sizeof(double); }
+
+__global__ void __launch_bounds__(kSolveThreads) lbfgs_solve_kernel(LbfgsCtl *c, int m, int first,
+                                                                    double eps, double *SY,
+                                                                    double *YY) {
+  extern __shared__ double Rs[];   // [k][m | 1]: odd row stride, columns without bank conflicts
+  __shared__ double sg[kMaxHistory], yg[kMaxHistory], snew[kMaxHistory], ynew[kMaxHistory];
+  __shared__ double diag[kMaxHistory], u[kMaxHistory], w[kMaxHistory];
+  __shared__ double wpart[kSolveParts][kMaxHistory];
+  __shared__ int sl[kMaxHistory], old[kMaxHistory];
+  const int tid = threadIdx.x, lane = tid & 31;
   if (first) {
-    const double l1 = dots[0];
-    c->k = 0;
-    c->cg = (float)-(l1 > 1.0 ? 1.0 / l1 : 1.0);   // t = min(1, 1 / ||g||_1), d = -g
+    if (tid == 0) {
+      const double l1 = c->dots[0];
+      c->k = 0;
+      c->cg = (float)-(l1 > 1.0 ? 1.0 / l1 : 1.0);   // t = min(1, 1 / ||g||_1), d = -g
+    }
     return;
   }
-  const int ld = m + 1;
-  const int sp = c->spare;
-  sg[sp] = dots[0];
-  yg[sp] = dots[1];
-  for (int p = 1; p <= count0; p++) {
-    sg[c->order[p - 1]] = dots[4 * p];
-    yg[c->order[p - 1]] = dots[4 * p + 1];
+  const int count0 = c->count, sp = c->spare, ld = m + 1;
+  const double ys = c->dots[2], yy = c->dots[3];
+  // the candidate becomes the newest pair (dropping the oldest of m) or is left out
+  const bool take = ys > eps;
+  const int keep = take ? (count0 < m ? count0 : m - 1) : count0;   // older pairs kept
+  const int k = keep + (take ? 1 : 0);
+  const double gamma = take ? ys / yy : (k > 0 ? c->gamma : 1.0);
+  if (tid < kMaxHistory) old[tid] = c->order[tid];   // newest first
+  __syncthreads();
+  if (tid < k) {
+    // pair tid (oldest first): its position in the fused pass, its slot, its four dots
+    const int p = k - 1 - tid + (take ? 0 : 1);
+    sl[tid] = p == 0 ? sp : old[p - 1];
+    sg[tid] = c->dots[4 * p];
+    yg[tid] = c->dots[4 * p + 1];
+    snew[tid] = c->dots[4 * p + 2];
+    ynew[tid] = c->dots[4 * p + 3];
   }
-  const double ys = dots[2], yy = dots[3];
-  if (ys > eps) {
-    // the candidate becomes the newest pair: its column of S^T Y and row / column of Y^T Y
-    for (int p = 1; p <= count0; p++) {
-      const int a = c->order[p - 1];
-      SY[(size_t)a * ld + sp] = dots[4 * p + 2];
-      YY[(size_t)a * ld + sp] = dots[4 * p + 3];
-      YY[(size_t)sp * ld + a] = dots[4 * p + 3];
+  __syncthreads();
+  const int newest = take ? k - 1 : -1;   // its column and row come from the dots
+  // this thread's part of row i of Y^T Y (symmetric: read down the column, coalesced over i)
+  const int i = tid % kMaxHistory, part = tid / kMaxHistory;
+  double yv[kSolveRow];
+#pragma unroll
+  for (int q = 0; q < kSolveRow; q++) {
+    const int j = part * kSolveRow + q;
+    yv[q] = 0.0;
+    if (i < k && j < k)
+      yv[q] = i == newest ? ynew[j] : j == newest ? ynew[i] : YY[(size_t)sl[j] * ld + sl[i]];
+  }
+  if (tid < k) {
+    diag[tid] = tid == newest ? ys : SY[(size_t)sl[tid] * ld + sl[tid]];
+    w[tid] = 1.0 / diag[tid];
+  }
+  __syncthreads();
+  const int rs = m | 1;
+  for (int r = tid >> 5; r < k; r += kSolveThreads / 32)   // a warp per row
+    for (int j = r + 1 + lane; j < k; j += 32)
+      Rs[r * rs + j] = w[r] * (j == newest ? snew[r] : SY[(size_t)sl[r] * ld + sl[j]]);
+  if (tid < k) u[tid] = sg[tid] * w[tid];
+  __syncthreads();
+  constexpr int NR = kMaxHistory / 32;
+  if (tid < 32) {   // Rs u = D^-1 (S^T g), from the last row up
+    double v[NR];
+#pragma unroll
+    for (int r = 0; r < NR; r++) v[r] = lane + 32 * r < k ? u[lane + 32 * r] : 0.0;
+#pragma unroll
+    for (int b = NR - 1; b >= 0; b--) {
+      for (int q = 31; q >= 0; q--) {
+        const int col = 32 * b + q;
+        if (col >= k) continue;
+        double a[NR];
+#pragma unroll
+        for (int r = 0; r <= b; r++) a[r] = lane + 32 * r < col ? Rs[(lane + 32 * r) * rs + col] : 0.0;
+        const double x = __shfl_sync(0xffffffffu, v[b], q);
+#pragma unroll
+        for (int r = 0; r <= b; r++) v[r] -= a[r] * x;
+      }
     }
-    SY[(size_t)sp * ld + sp] = ys;
-    YY[(size_t)sp * ld + sp] = yy;
-    c->gamma = ys / yy;
-    const int keep = count0 < m ? count0 : m - 1;
-    for (int i = keep; i >= 1; i--) c->order[i] = c->order[i - 1];
-    c->order[0] = sp;
-    c->count = keep + 1;
-    for (int i = c->count; i < m; i++) c->order[i] = -1;
-    for (int s = 0; s <= m; s++) {   // first slot not in use receives the next step
-      bool used = false;
-      for (int i = 0; i < c->count; i++) used |= c->order[i] == s;
-      if (!used) { c->spare = s; break; }
-    }
+#pragma unroll
+    for (int r = 0; r < NR; r++)
+      if (lane + 32 * r < k) u[lane + 32 * r] = v[r];
   }
-  const int k = c->count;
-  const double gamma = k > 0 ? c->gamma : 1.0;
-  for (int i = 0; i < k; i++) sl[i] = c->order[k - 1 - i];   // oldest first
-  // u = R^-1 (S^T g), R_ij = s_i . y_j (i <= j)
-  for (int i = k - 1; i >= 0; i--) {
-    double v = sg[sl[i]];
-    for (int j = i + 1; j < k; j++) v -= SY[(size_t)sl[i] * ld + sl[j]] * u[j];
-    u[i] = v / SY[(size_t)sl[i] * ld + sl[i]];
-  }
-  // w = (D + gamma Y^T Y) u - gamma Y^T g
-  for (int i = 0; i < k; i++) {
+  __syncthreads();
+  {   // Y^T Y u, kSolveParts threads per row
     double v = 0.0;
-    for (int j = 0; j < k; j++) v += YY[(size_t)sl[i] * ld + sl[j]] * u[j];
-    w[i] = SY[(size_t)sl[i] * ld + sl[i]] * u[i] + gamma * (v - yg[sl[i]]);
+#pragma unroll
+    for (int q = 0; q < kSolveRow; q++) {
+      const int j = part * kSolveRow + q;
+      if (j < k) v += yv[q] * u[j];
+    }
+    wpart[part][i] = v;
   }
-  // p = R^-T w
-  for (int i = 0; i < k; i++) {
-    double v = w[i];
-    for (int j = 0; j < i; j++) v -= SY[(size_t)sl[j] * ld + sl[i]] * pv[j];
-    pv[i] = v / SY[(size_t)sl[i] * ld + sl[i]];
+  __syncthreads();
+  if (tid < 32) {   // Rs^T z = w, from the first row down; p = D^-1 z
+    double v[NR];
+#pragma unroll
+    for (int r = 0; r < NR; r++) {
+      const int j = lane + 32 * r;
+      v[r] = 0.0;
+      if (j < k) {
+        double t = 0.0;
+#pragma unroll
+        for (int q = 0; q < kSolveParts; q++) t += wpart[q][j];
+        v[r] = diag[j] * u[j] + gamma * (t - yg[j]);
+      }
+    }
+#pragma unroll
+    for (int b = 0; b < NR; b++) {
+      for (int q = 0; q < 32; q++) {
+        const int row = 32 * b + q;
+        if (row >= k) break;
+        double a[NR];
+#pragma unroll
+        for (int r = b; r < NR; r++) {
+          const int j = lane + 32 * r;
+          a[r] = j > row && j < k ? Rs[row * rs + j] : 0.0;
+        }
+        const double x = __shfl_sync(0xffffffffu, v[b], q);
+#pragma unroll
+        for (int r = b; r < NR; r++) v[r] -= a[r] * x;
+      }
+    }
+    // d = -H g = -gamma g - S p + gamma Y u; step length 1
+#pragma unroll
+    for (int r = 0; r < NR; r++) {
+      const int j = lane + 32 * r;
+      if (j < k) {
+        c->slot[j] = sl[j];
+        c->cS[j] = (float)(-v[r] * w[j]);
+        c->cY[j] = (float)(gamma * u[j]);
+      }
+    }
+    if (lane == 0) {
+      c->k = k;
+      c->cg = (float)(-gamma);
+    }
+  } else if (take && tid < 64) {
+    // the first slot not in use receives the next step
+    int free_slot = -1;
+    for (int s0 = 0; s0 <= m && free_slot < 0; s0 += 32) {
+      bool used = s0 + lane > m;
+      for (int q = 0; q < k; q++) used |= sl[q] == s0 + lane;
+      const unsigned f = ~__ballot_sync(0xffffffffu, used);
+      if (f) free_slot = s0 + __ffs(f) - 1;
+    }
+    if (lane == 0) {
+      c->spare = free_slot;
+      c->count = k;
+      c->gamma = gamma;
+    }
+  } else if (take) {
+    for (int q = tid - 64; q < k; q += kSolveThreads - 64) {
+      c->order[q] = sl[k - 1 - q];
+      // the candidate's column of S^T Y and row / column of Y^T Y
+      SY[(size_t)sl[q] * ld + sp] = snew[q];
+      YY[(size_t)sl[q] * ld + sp] = ynew[q];
+      YY[(size_t)sp * ld + sl[q]] = ynew[q];
+    }
   }
-  // d = -H g = -gamma g - S p + gamma Y u; step length 1
-  c->k = k;
-  for (int i = 0; i < k; i++) {
-    c->slot[i] = sl[i];
-    c->cS[i] = (float)(-pv[i]);
-    c->cY[i] = (float)(gamma * u[i]);
-  }
-  c->cg = (float)(-gamma);
 }
 
-void launch_lbfgs_solve(LbfgsCtl *c, const double *partials, int m, int first, double eps,
-                        double *SY, double *YY, cudaStream_t s) {
-  lbfgs_solve_kernel<<<1, 256, 0, s>>>(c, partials, dot_blocks(m), m, first, eps, SY, YY);
+cudaError_t launch_lbfgs_solve(LbfgsCtl *c, int m, int first, double eps, double *SY, double *YY,
+                               cudaStream_t s) {
+  const size_t smem = solve_smem(m);
+  if (smem > 32 * 1024) {   // beyond what a launch may ask for without saying so
+    const cudaError_t e = cudaFuncSetAttribute(
+        lbfgs_solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)solve_smem(kMaxHistory));
+    if (e != cudaSuccess) return e;
+  }
+  lbfgs_solve_kernel<<<1, kSolveThreads, smem, s>>>(c, m, first, eps, SY, YY);
+  return cudaSuccess;
 }
 
 __global__ void __launch_bounds__(256) lbfgs_combine_kernel(

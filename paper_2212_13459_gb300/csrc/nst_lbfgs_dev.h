@@ -18,17 +18,20 @@ struct LbfgsCtl {
   int slot[kMaxHistory];
   float cg;
   float cS[kMaxHistory], cY[kMaxHistory];
+  // written by the fused pass for the solve: the four dot products of each position, and how many
+  // CTAs of each group have written their partials (zero between launches)
+  double dots[4 * (kMaxHistory + kLbGroup)];
+  unsigned arrived[kMaxHistory / kLbGroup + 1];
 };
 
 // the fused pass over the vectors: y = g - g_prev into the spare slot and, per stored pair and
 // the candidate, the four dot products s.g, y.g, s.y_new, y.y_new (first: only ||g||_1)
 void launch_lbfgs_dots(const float *g, const float *g_prev, const float *S, float *Y,
-                       long long stride, long long n, const LbfgsCtl *c, int m, int first,
+                       long long stride, long long n, LbfgsCtl *c, int m, int first,
                        double *partials, cudaStream_t s);
-// one CTA: fixed-order reductions, curvature test and history bookkeeping, the compact-form
-// solve, coefficients of the step
-void launch_lbfgs_solve(LbfgsCtl *c, const double *partials, int m, int first, double eps,
-                        double *SY, double *YY, cudaStream_t s);
+// one CTA: curvature test and history bookkeeping, the compact-form solve, coefficients of the step
+cudaError_t launch_lbfgs_solve(LbfgsCtl *c, int m, int first, double eps, double *SY, double *YY,
+                               cudaStream_t s);
 // the step: s = t d into the spare slot, x += s, g_prev = g
 void launch_lbfgs_combine(float *x, float *S, const float *Y, long long stride, float *g_prev,
                           const float *g, long long n, const LbfgsCtl *c, cudaStream_t s);
