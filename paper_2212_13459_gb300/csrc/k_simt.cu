@@ -914,64 +914,128 @@ void launch_style_finalize(const StyleFinalizeArgs &a, cudaStream_t s) {
   style_sum_kernel<<<1, 32, 0, s>>>(a, kFinalizeChunks - 1);
 }
 
-// channel sums over owned pixels: partial[c][j] = sum over chunk c of V[p][j] (FP32 runs of 64
-// pixels added in FP64)
+// ---- channel sums over owned pixels, all style layers in one launch -------------------------------
+// FP32 sums of runs of 64 pixels (of each chunk, in pixel order), added in FP64. Bound: the read of
+// the activations; a thread per channel took a pixel at a time (2 bytes a load, a division per
+// pixel, 40 CTAs at the deep layers: 1,980 us for the five layers of 1512 x 2016). Here C / 8 lanes
+// take a run, 16 bytes of a pixel each with eight pixels' loads in flight; a CTA holds 2048 / C
+// runs at a time, and the runs of a chunk are dealt to as many CTAs as fill the chip:
+// 174 us, 744 MB.
+constexpr int kChansumThreads = 256, kChansumRun = 64;
 template <typename T>
-__global__ void __launch_bounds__(256) chansum_partial_kernel(
-    const T *__restrict__ V, int Hb, int Wb, int C, const OwnRect *__restrict__ own,
-    const GramChunk *__restrict__ chunks, double *__restrict__ partial) {
-  const GramChunk ch = chunks[blockIdx.x];
-  const OwnRect r = own[ch.b];
-  const int rw = r.x1 - r.x0;
-  for (int j = threadIdx.x; j < C; j += blockDim.x) {
-    double acc = 0.0;
-    for (int q0 = ch.p0; q0 < ch.p1; q0 += 64) {
-      float f = 0.f;
-      const int q1 = q0 + 64 < ch.p1 ? q0 + 64 : ch.p1;
-      for (int q = q0; q < q1; q++) {
-        const int y = r.y0 + q / rw, x = r.x0 + q % rw;
-        f += to_f(V[(((size_t)ch.b * Hb + y) * Wb + x) * C + j]);
+__global__ void __launch_bounds__(kChansumThreads) chansum_partial_kernel(ChansumArgs a) {
+  __shared__ double red[kChansumThreads * 8];   // [lane group][C]
+  int l = 0;
+  while (l + 1 < kNStyle && (int)blockIdx.x >= a.L[l + 1].cta0) l++;
+  const ChansumLayer L = a.L[l];
+  const int idx = blockIdx.x - L.cta0, chunk = idx / L.split, s = idx - chunk * L.split;
+  const GramChunk ch = L.chunks[chunk];
+  const OwnRect r = L.own[ch.b];
+  const int rw = r.x1 - r.x0, C = L.C, G = C / 8, NG = kChansumThreads / G;
+  const int grp = threadIdx.x / G, c0 = (threadIdx.x % G) * 8;
+  const T *V = reinterpret_cast<const T *>(L.V);
+  double acc[8];
+#pragma unroll
+  for (int j = 0; j < 8; j++) acc[j] = 0.0;
+  // this CTA's runs: s, s + split, ...; this lane group's: every NG-th of those
+  for (long long run = s + (long long)L.split * grp;; run += (long long)L.split * NG) {
+    const long long qs = ch.p0 + run * kChansumRun;
+    if (grp >= NG || qs >= ch.p1) break;
+    int q = (int)qs;
+    const int q1 = min(q + kChansumRun, ch.p1);
+    int x = q % rw;
+    const T *p = V + (((size_t)ch.b * L.Hb + r.y0 + q / rw) * L.Wb + r.x0 + x) * C + c0;
+    auto next = [&]() {
+      p += C;
+      if (++x == rw) { x = 0; p += (size_t)(L.Wb - rw) * C; }
+    };
+    float f[8];
+#pragma unroll
+    for (int j = 0; j < 8; j++) f[j] = 0.f;
+    for (; q + 8 <= q1; q += 8) {
+      float v[8][8];
+#pragma unroll
+      for (int k = 0; k < 8; k++) {
+        load8(p, v[k]);
+        next();
       }
-      acc += (double)f;
+#pragma unroll
+      for (int k = 0; k < 8; k++)
+#pragma unroll
+        for (int j = 0; j < 8; j++) f[j] += v[k][j];
     }
-    partial[(size_t)blockIdx.x * C + j] = acc;
+    for (; q < q1; q++) {
+      float v[8];
+      load8(p, v);
+      next();
+#pragma unroll
+      for (int j = 0; j < 8; j++) f[j] += v[j];
+    }
+#pragma unroll
+    for (int j = 0; j < 8; j++) acc[j] += (double)f[j];
+  }
+  if (grp < NG)
+#pragma unroll
+    for (int j = 0; j < 8; j++) red[grp * C + c0 + j] = acc[j];
+  __syncthreads();
+  for (int j = threadIdx.x; j < C; j += kChansumThreads) {   // the groups in index order
+    double t = 0.0;
+    for (int g = 0; g < NG; g++) t += red[g * C + j];
+    L.partial[(size_t)idx * C + j] = t;
   }
 }
 
-// S[j] += sum over chunks of partial[c][j]: a CTA takes 32 channels (lane = channel), its 8 warps
-// split the chunks (warp w: chunks w, w + 8, ... in order), then the warps are added in order
-__global__ void __launch_bounds__(256) chansum_reduce_kernel(const double *__restrict__ partial,
-                                                             int nchunks, int C,
-                                                             double *__restrict__ S) {
-  __shared__ double red[8][32];
+// S[j] += sum of the layer's partials: a CTA takes 32 channels (lane = channel), its 16 warps
+// split the partials (warp w: w, w + 16, ... in order), then the warps are added in order
+constexpr int kChansumWarps = 16;
+__global__ void __launch_bounds__(32 * kChansumWarps) chansum_reduce_kernel(ChansumArgs a) {
+  __shared__ double red[kChansumWarps][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int j = blockIdx.x * 32 + lane;
+  int l = 0, b = blockIdx.x;
+  while (b >= a.L[l].C / 32) b -= a.L[l++].C / 32;
+  const ChansumLayer L = a.L[l];
+  const int j = b * 32 + lane, n = L.nchunks * L.split;
   double s = 0.0;
-  if (j < C)
-    for (int c = warp; c < nchunks; c += 8) s += partial[(size_t)c * C + j];
+  for (int c0 = warp; c0 < n; c0 += 8 * kChansumWarps) {   // eight loads in flight
+    double v[8];
+#pragma unroll
+    for (int k = 0; k < 8; k++) {
+      const int c = c0 + k * kChansumWarps;
+      v[k] = c < n ? L.partial[(size_t)c * L.C + j] : 0.0;
+    }
+#pragma unroll
+    for (int k = 0; k < 8; k++) s += v[k];
+  }
   red[warp][lane] = s;
   __syncthreads();
-  if (warp == 0 && j < C) {
+  if (warp == 0) {
     double t = 0.0;
 #pragma unroll
-    for (int w = 0; w < 8; w++) t += red[w][lane];
-    S[j] += t;
+    for (int w = 0; w < kChansumWarps; w++) t += red[w][lane];
+    L.S[j] += t;
   }
 }
 
-template <typename T>
-void launch_chansum(const T *V, int Hb, int Wb, int C, const OwnRect *own,
-                    const GramChunk *chunks, int nchunks, double *partial, double *S,
-                    cudaStream_t s) {
-  if (nchunks <= 0) return;
-  chansum_partial_kernel<T><<<nchunks, 256, 0, s>>>(V, Hb, Wb, C, own, chunks, partial);
-  chansum_reduce_kernel<<<(C + 31) / 32, 256, 0, s>>>(partial, nchunks, C, S);
+int chansum_split(int nchunks, int max_chunk_px) {
+  const int runs = (max_chunk_px + kChansumRun - 1) / kChansumRun;
+  const int want = nchunks > 0 ? 1216 / nchunks : 1;   // eight CTAs per SM
+  return want < 1 ? 1 : want > runs ? (runs > 0 ? runs : 1) : want;
 }
-template void launch_chansum<float>(const float *, int, int, int, const OwnRect *,
-                                    const GramChunk *, int, double *, double *, cudaStream_t);
-template void launch_chansum<__nv_bfloat16>(const __nv_bfloat16 *, int, int, int,
-                                            const OwnRect *, const GramChunk *, int, double *,
-                                            double *, cudaStream_t);
+
+template <typename T>
+void launch_chansum(ChansumArgs a, cudaStream_t s) {
+  int ctas = 0, rctas = 0;
+  for (int l = 0; l < kNStyle; l++) {
+    a.L[l].cta0 = ctas;
+    ctas += a.L[l].nchunks * a.L[l].split;
+    rctas += a.L[l].C / 32;
+  }
+  if (ctas <= 0) return;
+  chansum_partial_kernel<T><<<ctas, kChansumThreads, 0, s>>>(a);
+  chansum_reduce_kernel<<<rctas, 32 * kChansumWarps, 0, s>>>(a);
+}
+template void launch_chansum<float>(ChansumArgs, cudaStream_t);
+template void launch_chansum<__nv_bfloat16>(ChansumArgs, cudaStream_t);
 
 
 // ---- content loss over owned pixels: partial[c] = sum (V - Vu)^2 (FP64) ----------------------------

@@ -124,6 +124,7 @@ struct Batch {
   PatchList unpool[kNConv];                   // pooled layer l: one pooled rectangle per block
                                               // ({y0, y1, x0, x1}; TH = largest area)
   int chunk_off[kNStyle + 1], nchunks[kNStyle + 1];  // Gram chunks per style layer; [5] content
+  int cs_split[kNStyle];                      // channel sums: CTAs per chunk
   int tc_off[kNStyle], tc_runs[kNStyle];      // tensor-core Gram runs per style layer
   int max_inner_px, max_content_px;
   int max_inner_h, max_inner_w;
@@ -139,7 +140,7 @@ struct PassPlan {
   GramChunk *d_chunks = nullptr;  // all chunks
   size_t gram_part_floats = 0;    // largest nchunks * npairs * 4096 (or tensor-core tiles)
   int max_content_chunks = 0;
-  size_t chansum_doubles = 0;     // largest nchunks * C (channel-sum partials)
+  size_t chansum_doubles = 0;     // channel-sum partials of a batch, all style layers
   // tensor-core Gram: box shape per style layer, runs, and per-block owned-rectangle maps
   int tc_TH[kNStyle], tc_TW[kNStyle];
   GramTcChunk *d_tcchunks = nullptr;
@@ -452,11 +453,15 @@ nst_status build_plan(nst_ctx *ctx, int H, int W, int margin, PassPlan **out) {
       bt.nchunks[s] = (int)chunks.size() - bt.chunk_off[s];
       if (s < kNStyle) {
         p.gram_part_floats = std::max(p.gram_part_floats, (size_t)bt.nchunks[s] * npairs * 4096);
-        p.chansum_doubles = std::max(p.chansum_doubles, (size_t)bt.nchunks[s] * C);
+        bt.cs_split[s] = chansum_split(bt.nchunks[s], (int)std::min(tot, ch));
       }
       else
         p.max_content_chunks = std::max(p.max_content_chunks, bt.nchunks[s]);
     }
+    size_t cs = 0;
+    for (int si = 0; si < kNStyle; si++)
+      cs += (size_t)bt.nchunks[si] * bt.cs_split[si] * kStyleC[si];
+    p.chansum_doubles = std::max(p.chansum_doubles, cs);
     for (int si = 0; si < kNStyle; si++) {
       int N, nI, nJ;
       gram_tc_shape(kStyleC[si], &N, &nI, &nJ);
@@ -811,15 +816,20 @@ template <typename T>
 nst_status gram_batch(nst_ctx *ctx, PassPlan &p, const Batch &bt, const Workspace &ws,
                       cudaStream_t s, bool moments) {
   const int nt = (int)p.tiles.size();
-  if (moments)
+  if (moments) {
+    Timer tm(ctx, kTGram, s);
+    ctx->launches += 2;
+    ChansumArgs a{};
+    double *part = ctx->d_cspart;
     for (int si = 0; si < kNStyle; si++) {
       const int l = kStyleConv[si], lv = kLevel[l];
-      Timer tm(ctx, kTGram, s);
-      ctx->launches += 2;
-      launch_chansum<T>((const T *)ws.act[l], p.Hb >> lv, p.Wb >> lv, kCout[l],
-                        p.d_own + (size_t)si * nt + bt.t0, p.d_chunks + bt.chunk_off[si],
-                        bt.nchunks[si], ctx->d_cspart, ctx->d_sacc + moment_offset(si), s);
+      a.L[si] = {ws.act[l], p.Hb >> lv, p.Wb >> lv, kCout[l],
+                 p.d_own + (size_t)si * nt + bt.t0, p.d_chunks + bt.chunk_off[si],
+                 bt.nchunks[si], bt.cs_split[si], part, ctx->d_sacc + moment_offset(si), 0};
+      part += (size_t)bt.nchunks[si] * bt.cs_split[si] * kCout[l];
     }
+    launch_chansum<T>(a, s);
+  }
   if (ctx->use_tc) {
     nst_status st = ensure_gram_maps(ctx, p, ws);
     if (st) return st;

@@ -82,10 +82,23 @@ void launch_gram_partial_flat(const T *V, long long npix, int C, long long chunk
                               float *part, cudaStream_t s);
 void launch_gram_reduce(const float *part, int nchunks, int C, double *Gacc, cudaStream_t s);
 void launch_style_finalize(const StyleFinalizeArgs &a, cudaStream_t s);
+// channel sums of the style layers' owned pixels: S[j] += sum over the chunks of V[p][j]
+struct ChansumLayer {
+  const void *V;            // [B][Hb][Wb][C], C a multiple of 64, at most 512
+  int Hb, Wb, C;
+  const OwnRect *own;       // per block
+  const GramChunk *chunks;
+  int nchunks, split;       // split: CTAs per chunk (chansum_split)
+  double *partial;          // [nchunks * split][C]
+  double *S;
+  int cta0;                 // set by the launcher
+};
+struct ChansumArgs {
+  ChansumLayer L[kNStyle];
+};
+int chansum_split(int nchunks, int max_chunk_px);
 template <typename T>
-void launch_chansum(const T *V, int Hb, int Wb, int C, const OwnRect *own,
-                    const GramChunk *chunks, int nchunks, double *partial, double *S,
-                    cudaStream_t s);
+void launch_chansum(ChansumArgs a, cudaStream_t s);
 template <typename T>
 void launch_content_loss(const T *V, int Hb, int Wb, const T *Vu, int Hc, int Wc,
                          const BlockGeom *geom, const OwnRect *own, const GramChunk *chunks,
