@@ -16,6 +16,12 @@
 // drain the accumulator (tcgen05.ld), apply the epilogue and store BF16. Two TMEM accumulators
 // let the epilogue of one tile overlap the main loop of the next. Every mbarrier wait is bounded:
 // on timeout the kernel latches kErrTimeout in the status word and returns.
+//
+// The issue loops (producer and MMA) run on the whole warp, one elected lane at the TMA and MMA
+// instructions, without divisions: run by a single lane they took about 570 clocks per K-block,
+// more than the 512 its 256-wide MMAs need and the bound of every launch. 512 -> 512 channels at
+// 64 x 94 x 100 pixels: 1,627 -> 1,458 us (1.95 PFLOP/s; 1,317 us without any loads); at
+// 4 x 8 x 8: 31 -> 19 us.
 #include <cuda.h>
 
 #include <mutex>
@@ -41,10 +47,25 @@ struct TcGeom {
   int tx_bytes;         // bytes one stage's TMA loads deliver
   int tiles_x, tiles_y; // patches per block image
   int n_tiles;          // N tiles (cout / BN)
-  int total;            // M tiles * N tiles
+  int total;            // M tiles * N tiles (counting the parts of split ones)
+  int full, split;      // main kernel: tiles 0 .. full - 1 are whole; every later one is `split`
+                        // parts of BN / split channels
   int kb_main;          // taps * cin / 64
   int kb2;              // k2 / 64
-  int cin_blocks;       // cin / 64
+};
+
+// The K-blocks of a tile in order: taps (dy, dx) outermost, 64-channel blocks of the input inside;
+// then phase 2. c = input channel, k = column of the weight matrix [cout][tap][cin].
+struct KWalk {
+  int c = 0, k = 0, dx = -1, dy = -1;
+  __device__ __forceinline__ void next(int cin) {
+    c += kBK;
+    k += kBK;
+    if (c == cin) {
+      c = 0;
+      if (++dx == 2) { dx = -1; dy++; }
+    }
+  }
 };
 
 // Origin of output patch (M tile) mt: from the launch's patch list when it has one (each
@@ -391,16 +412,33 @@ __device__ __forceinline__ void swap_pool8(const ConvArgs &a, const BlockGeom &g
 }
 
 // ---- the kernel -------------------------------------------------------------------------------------
+// Tile t of the main kernel: M tile, first output channel and channel count (see TcGeom::split).
+// tmBp / tmB2p: the weight maps with boxes of BN / split rows.
+template <int BN>
+__device__ __forceinline__ void tile_of(const TcGeom &tg, int t, int &mt, int &n0, int &nn) {
+  int part = 0;
+  nn = BN;
+  if (t >= tg.full) {
+    const int u = t - tg.full;
+    part = u % tg.split;
+    t = tg.full + u / tg.split;
+    nn = BN / tg.split;
+  }
+  mt = t / tg.n_tiles;
+  n0 = (t % tg.n_tiles) * BN + part * nn;
+}
+
 template <int BN, int STAGES>
 __global__ void __launch_bounds__(kThreads, 1)
     conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                    const __grid_constant__ CUtensorMap tmA2,
-                   const __grid_constant__ CUtensorMap tmB2, const ConvArgs a, const TcGeom tg) {
+                   const __grid_constant__ CUtensorMap tmB2,
+                   const __grid_constant__ CUtensorMap tmBp,
+                   const __grid_constant__ CUtensorMap tmB2p, const ConvArgs a, const TcGeom tg) {
   constexpr uint32_t A_BYTES = 128 * kBK * 2;
   constexpr uint32_t B_BYTES = BN * kBK * 2;
   constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES;
   constexpr uint32_t TMEM_COLS = 2 * BN;
-  constexpr uint32_t IDESC = make_idesc(BN);
 
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full_bar[STAGES], empty_bar[STAGES];
@@ -409,7 +447,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ volatile int abort_flag;
 
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; s++) {
@@ -432,69 +470,75 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   if (warp == 0) {
     // ---------------- TMA producer ----------------
-    if (lane == 0) {
-      asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
-      asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmB)) : "memory");
-      int stage = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      for (int t = blockIdx.x; t < tg.total && ok; t += gridDim.x) {
-        const int nt = t % tg.n_tiles, mt = t / tg.n_tiles;
-        int b, y0, x0;
-        patch_origin(a, tg, mt, b, y0, x0);
-        const int n0 = nt * BN;
-        for (int kb = 0; kb < kb_total; kb++) {
-          if (!mbar_wait(smem_u32(&empty_bar[stage]), phase ^ 1, &abort_flag, a.err)) {
-            ok = false;
-            break;
-          }
+    int stage = 0;
+    uint32_t phase = 1;   // parity of the empty barriers to wait for
+    bool ok = true;
+    for (int t = blockIdx.x; t < tg.total && ok; t += gridDim.x) {
+      int mt, n0, nn, b, y0, x0;
+      tile_of<BN>(tg, t, mt, n0, nn);
+      patch_origin(a, tg, mt, b, y0, x0);
+      const uint32_t tx = (uint32_t)(tg.TH * tg.TW + nn) * (kBK * 2);
+      const CUtensorMap *wB = nn == BN ? &tmB : &tmBp, *wB2 = nn == BN ? &tmB2 : &tmB2p;
+      KWalk w;
+      for (int kb = 0; kb < kb_total; kb++) {
+        if (!mbar_wait_warp(smem_u32(&empty_bar[stage]), phase, &abort_flag, a.err)) {
+          ok = false;
+          break;
+        }
+        if (elect_one()) {
           const uint32_t fb = smem_u32(&full_bar[stage]);
           const uint32_t sa = smem_base + stage * STAGE_BYTES, sb = sa + A_BYTES;
-          mbar_expect_tx(fb, (uint32_t)tg.tx_bytes);
+          mbar_expect_tx(fb, tx);
           if (kb < tg.kb_main) {
-            const int tap = kb / tg.cin_blocks, cb = kb % tg.cin_blocks;
-            const int dy = tap / 3 - 1, dx = tap % 3 - 1;
-            tma_load_4d(sa, &tmA, fb, cb * kBK, x0 + dx, y0 + dy, b);
-            tma_load_2d(sb, &tmB, fb, tap * a.cin + cb * kBK, n0);
+            tma_load_4d(sa, &tmA, fb, w.c, x0 + w.dx, y0 + w.dy, b);
+            tma_load_2d(sb, wB, fb, w.k, n0);
           } else {
-            const int cb = kb - tg.kb_main;
-            tma_load_4d(sa, &tmA2, fb, cb * kBK, x0, y0, b);
-            tma_load_2d(sb, &tmB2, fb, cb * kBK, n0);
+            const int c = (kb - tg.kb_main) * kBK;
+            tma_load_4d(sa, &tmA2, fb, c, x0, y0, b);
+            tma_load_2d(sb, wB2, fb, c, n0);
           }
-          if (++stage == STAGES) { stage = 0; phase ^= 1; }
         }
+        __syncwarp();
+        w.next(a.cin);
+        if (++stage == STAGES) { stage = 0; phase ^= 1; }
       }
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
-    if (lane == 0) {
-      int stage = 0;
-      uint32_t phase = 0;
-      int it = 0;
-      bool ok = true;
-      for (int t = blockIdx.x; t < tg.total && ok; t += gridDim.x, it++) {
-        const int acc = it & 1;
-        const uint32_t use = (uint32_t)(it >> 1);
-        if (!mbar_wait(smem_u32(&tempty_bar[acc]), (use & 1) ^ 1, &abort_flag, a.err)) break;
+    int stage = 0, it = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    const uint64_t da0 = sw128_desc(smem_base);
+    for (int t = blockIdx.x; t < tg.total && ok; t += gridDim.x, it++) {
+      const int acc = it & 1;
+      const uint32_t use = (uint32_t)(it >> 1);
+      if (!mbar_wait_warp(smem_u32(&tempty_bar[acc]), (use & 1) ^ 1, &abort_flag, a.err)) break;
+      tc_fence_after();
+      const uint32_t d = tmem_base + (uint32_t)(acc * BN);
+      int mt, n0, nn;
+      tile_of<BN>(tg, t, mt, n0, nn);
+      const uint32_t idesc = make_idesc(nn);
+      for (int kb = 0; kb < kb_total; kb++) {
+        if (!mbar_wait_warp(smem_u32(&full_bar[stage]), phase, &abort_flag, a.err)) {
+          ok = false;
+          break;
+        }
         tc_fence_after();
-        const uint32_t d = tmem_base + (uint32_t)(acc * BN);
-        for (int kb = 0; kb < kb_total; kb++) {
-          if (!mbar_wait(smem_u32(&full_bar[stage]), phase, &abort_flag, a.err)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t sa = smem_base + stage * STAGE_BYTES, sb = sa + A_BYTES;
-          const uint64_t da = sw128_desc(sa), db = sw128_desc(sb);
+        if (elect_one()) {
+          // descriptors: the first stage's plus a multiple of the stage size (16-byte units)
+          const uint64_t da = da0 + (uint64_t)(stage * (int)(STAGE_BYTES >> 4));
+          const uint64_t db = da + (A_BYTES >> 4);
 #pragma unroll
           for (int k = 0; k < kBK / 16; k++)
-            mma_bf16(d, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), IDESC,
+            mma_bf16(d, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), idesc,
                      (kb > 0 || k > 0) ? 1u : 0u);
           mma_commit(smem_u32(&empty_bar[stage]));
-          if (++stage == STAGES) { stage = 0; phase ^= 1; }
         }
-        if (ok) mma_commit(smem_u32(&tfull_bar[acc]));
+        __syncwarp();
+        if (++stage == STAGES) { stage = 0; phase ^= 1; }
       }
+      if (ok && elect_one()) mma_commit(smem_u32(&tfull_bar[acc]));
+      __syncwarp();
     }
   } else {
     // ---------------- epilogue (warps 2..5) ----------------
@@ -512,14 +556,14 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (lane == 0) ready = mbar_wait_sleep(smem_u32(&tfull_bar[acc]), use & 1, &abort_flag, a.err);
       if (!__shfl_sync(0xffffffffu, ready, 0)) break;
       tc_fence_after();
-      const int nt = t % tg.n_tiles, mt = t / tg.n_tiles;
-      int b, oy, ox;
+      int mt, n0, nn, b, oy, ox;
+      tile_of<BN>(tg, t, mt, n0, nn);
       patch_origin(a, tg, mt, b, oy, ox);
       const BlockGeom g = a.geom[b];
       const uint32_t tbase = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN);
       const int cg = lane & 3;
 #pragma unroll 1
-      for (int c = half * (BN / 2); c < (half + 1) * (BN / 2); c += 32) {
+      for (int c = half * (nn / 2); c < (half + 1) * (nn / 2); c += 32) {
         float v[32];
         tmem_ld32(tbase + (uint32_t)c, v);   // row = this lane's pixel, 32 channels
 #pragma unroll
@@ -528,7 +572,7 @@ __global__ void __launch_bounds__(kThreads, 1)
               make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
         __syncwarp();
         float cbias[8];   // (forward) the bias of this thread's 8 channels of the chunk
-        if (a.mode == kEpiForward) load8_bias(a.bias + nt * BN + c + cg * 8, cbias);
+        if (a.mode == kEpiForward) load8_bias(a.bias + n0 + c + cg * 8, cbias);
 #pragma unroll
         for (int k = 0; k < 4; k++) {
           const int j = k * 8 + (lane >> 2);
@@ -537,11 +581,11 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (pp < tg.TH * tg.TW && y < a.Hb && x < a.Wb) {
             float r[8];
             swap_tile_read8(tsm, j, cg, r);
-            epilogue8(a, g, b, y, x, nt * BN + c + cg * 8, r,
+            epilogue8(a, g, b, y, x, n0 + c + cg * 8, r,
                       a.mode == kEpiForward ? cbias : nullptr);
           }
         }
-        if (a.pool_out) swap_pool8(a, g, b, oy, ox, tg, q * 32, nt * BN + c, tsm);
+        if (a.pool_out) swap_pool8(a, g, b, oy, ox, tg, q * 32, n0 + c, tsm);
         __syncwarp();
       }
       tc_fence_before();
@@ -622,7 +666,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t w_base = smem_base, a_base = smem_base + Cfg::W_BYTES;
   const uint32_t v_base = a_base + SA * kHaloStage;   // (MASK_SMEM) the phase-2 ring
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   // this CTA's N slice, and its share of the M tiles
   const int nt = blockIdx.x % NT, m_first = blockIdx.x / NT, m_step = gridDim.x / NT;
   const int m_total = tg.total;
@@ -651,7 +695,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t tmem_base = tmem_base_sh;
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       // resident weights of slice nt: tile (tap, cb) at w_base + (tap * KB + cb) * TILE_B, then
       // the phase-2 tiles (R rows of the slice)
       const uint32_t wb = smem_u32(&w_bar);
@@ -662,28 +706,34 @@ __global__ void __launch_bounds__(kThreads, 1)
                       nt * BN);
       for (int cb = 0; cb < P2KB; cb++)
         tma_load_2d(w_base + (9 * KB + cb) * Cfg::TILE_B, &tmB2, wb, cb * kBK, nt * BN);
-      int stage = 0, vst = 0;
-      uint32_t phase = 0, vph = 0;
-      bool ok = true;
-      for (int t = m_first; t < m_total && ok; t += m_step) {
-        int b, oy, ox;
-        patch_origin(a, tg, t, b, oy, ox);
-        for (int kb = 0; kb < KBT; kb++) {
-          if (MASK_SMEM && kb == KB) {   // the tile's own pixels of V (no halo)
-            if (!mbar_wait(smem_u32(&vempty_bar[vst]), vph ^ 1, &abort_flag, a.err)) {
-              ok = false;
-              break;
-            }
-            const uint32_t fb = smem_u32(&vfull_bar[vst]);
-            mbar_expect_tx(fb, kMaskVStage);
-            tma_load_4d(v_base + vst * kMaskVStage, &tmA2, fb, 0, ox, oy, b);
-            if (++vst == SV) { vst = 0; vph ^= 1; }
-            continue;
-          }
-          if (!mbar_wait(smem_u32(&empty_bar[stage]), phase ^ 1, &abort_flag, a.err)) {
+    }
+    __syncwarp();
+    int stage = 0, vst = 0;
+    uint32_t phase = 0, vph = 0;
+    bool ok = true;
+    for (int t = m_first; t < m_total && ok; t += m_step) {
+      int b, oy, ox;
+      patch_origin(a, tg, t, b, oy, ox);
+      for (int kb = 0; kb < KBT; kb++) {
+        if (MASK_SMEM && kb == KB) {   // the tile's own pixels of V (no halo)
+          if (!mbar_wait_warp(smem_u32(&vempty_bar[vst]), vph ^ 1, &abort_flag, a.err)) {
             ok = false;
             break;
           }
+          if (elect_one()) {
+            const uint32_t fb = smem_u32(&vfull_bar[vst]);
+            mbar_expect_tx(fb, kMaskVStage);
+            tma_load_4d(v_base + vst * kMaskVStage, &tmA2, fb, 0, ox, oy, b);
+          }
+          __syncwarp();
+          if (++vst == SV) { vst = 0; vph ^= 1; }
+          continue;
+        }
+        if (!mbar_wait_warp(smem_u32(&empty_bar[stage]), phase ^ 1, &abort_flag, a.err)) {
+          ok = false;
+          break;
+        }
+        if (elect_one()) {
           const uint32_t fb = smem_u32(&full_bar[stage]);
           mbar_expect_tx(fb, kHaloBoxBytes);
           const uint32_t sa = a_base + stage * kHaloStage;
@@ -691,16 +741,13 @@ __global__ void __launch_bounds__(kThreads, 1)
             tma_load_4d(sa, &tmA, fb, kb * kBK, ox - 1, oy - 1, b);
           else
             tma_load_4d(sa, &tmA2, fb, (kb - KB) * kBK, ox - 1, oy - 1, b);
-          if (++stage == SA) { stage = 0; phase ^= 1; }
         }
+        __syncwarp();
+        if (++stage == SA) { stage = 0; phase ^= 1; }
       }
     }
   } else if (warp == 1) {
-    // The whole warp runs the issue loop (its waits and loop control are warp-uniform), and one
-    // elected lane issues each K-block's MMAs and commit: a loop run by a single lane issues
-    // several times slower once epilogue warps keep this warp's scheduler busy, and a 64-wide
-    // MMA takes only 48 cycles. (The 256-wide MMAs of the other kernels take 128 cycles; there
-    // the single-lane loop keeps up and measured slightly faster.)
+    // (as in every kernel here, the whole warp runs the issue loop and one elected lane issues)
     bool ok = mbar_wait_warp(smem_u32(&w_bar), 0, &abort_flag, a.err);
     int stage = 0, vst = 0;
     uint32_t phase = 0, vph = 0;
@@ -888,7 +935,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t *smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; s++) {
@@ -911,69 +958,69 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   if (warp == 0) {
     // ---------------- TMA producer: weight box (A) + activation box (B) per K-block ----------------
-    if (lane == 0) {
-      asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
-      asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmB)) : "memory");
-      int stage = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      for (int t = blockIdx.x; t < tg.total && ok; t += gridDim.x) {
-        const int nt = t % tg.n_tiles, mt = t / tg.n_tiles;
-        int b, y0, x0;
-        patch_origin(a, tg, mt, b, y0, x0);
-        const int n0 = nt * kSwapBN;
-        for (int kb = 0; kb < kb_total; kb++) {
-          if (!mbar_wait(smem_u32(&empty_bar[stage]), phase ^ 1, &abort_flag, a.err)) {
-            ok = false;
-            break;
-          }
+    int stage = 0;
+    uint32_t phase = 1;
+    bool ok = true;
+    for (int t = blockIdx.x; t < tg.total && ok; t += gridDim.x) {
+      const int mt = t / tg.n_tiles, n0 = (t % tg.n_tiles) * kSwapBN;
+      int b, y0, x0;
+      patch_origin(a, tg, mt, b, y0, x0);
+      KWalk w;
+      for (int kb = 0; kb < kb_total; kb++) {
+        if (!mbar_wait_warp(smem_u32(&empty_bar[stage]), phase, &abort_flag, a.err)) {
+          ok = false;
+          break;
+        }
+        if (elect_one()) {
           const uint32_t fb = smem_u32(&full_bar[stage]);
           const uint32_t sw = smem_base + stage * STAGE_BYTES, sx = sw + kSwapA;
           mbar_expect_tx(fb, (uint32_t)tg.tx_bytes);
           if (kb < tg.kb_main) {
-            const int tap = kb / tg.cin_blocks, cb = kb % tg.cin_blocks;
-            const int dy = tap / 3 - 1, dx = tap % 3 - 1;
-            tma_load_2d(sw, &tmB, fb, tap * a.cin + cb * kBK, n0);
-            tma_load_4d(sx, &tmA, fb, cb * kBK, x0 + dx, y0 + dy, b);
+            tma_load_2d(sw, &tmB, fb, w.k, n0);
+            tma_load_4d(sx, &tmA, fb, w.c, x0 + w.dx, y0 + w.dy, b);
           } else {
-            const int cb = kb - tg.kb_main;
-            tma_load_2d(sw, &tmB2, fb, cb * kBK, n0);
-            tma_load_4d(sx, &tmA2, fb, cb * kBK, x0, y0, b);
+            const int c = (kb - tg.kb_main) * kBK;
+            tma_load_2d(sw, &tmB2, fb, c, n0);
+            tma_load_4d(sx, &tmA2, fb, c, x0, y0, b);
           }
-          if (++stage == STAGES) { stage = 0; phase ^= 1; }
         }
+        __syncwarp();
+        w.next(a.cin);
+        if (++stage == STAGES) { stage = 0; phase ^= 1; }
       }
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer: D[128 ch][256 px] += W[128 x 64] X[256 x 64]^T ----------------
-    if (lane == 0) {
-      int stage = 0;
-      uint32_t phase = 0;
-      int it = 0;
-      bool ok = true;
-      for (int t = blockIdx.x; t < tg.total && ok; t += gridDim.x, it++) {
-        const int acc = it & 1;
-        const uint32_t use = (uint32_t)(it >> 1);
-        if (!mbar_wait(smem_u32(&tempty_bar[acc]), (use & 1) ^ 1, &abort_flag, a.err)) break;
+    int stage = 0, it = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    const uint64_t dw0 = sw128_desc(smem_base);
+    for (int t = blockIdx.x; t < tg.total && ok; t += gridDim.x, it++) {
+      const int acc = it & 1;
+      const uint32_t use = (uint32_t)(it >> 1);
+      if (!mbar_wait_warp(smem_u32(&tempty_bar[acc]), (use & 1) ^ 1, &abort_flag, a.err)) break;
+      tc_fence_after();
+      const uint32_t d = tmem_base + (uint32_t)(acc * kSwapBP);
+      for (int kb = 0; kb < kb_total; kb++) {
+        if (!mbar_wait_warp(smem_u32(&full_bar[stage]), phase, &abort_flag, a.err)) {
+          ok = false;
+          break;
+        }
         tc_fence_after();
-        const uint32_t d = tmem_base + (uint32_t)(acc * kSwapBP);
-        for (int kb = 0; kb < kb_total; kb++) {
-          if (!mbar_wait(smem_u32(&full_bar[stage]), phase, &abort_flag, a.err)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t sw = smem_base + stage * STAGE_BYTES, sx = sw + kSwapA;
-          const uint64_t dw = sw128_desc(sw), dx = sw128_desc(sx);
+        if (elect_one()) {
+          const uint64_t dw = dw0 + (uint64_t)(stage * (int)(STAGE_BYTES >> 4));
+          const uint64_t dx = dw + (kSwapA >> 4);
 #pragma unroll
           for (int k = 0; k < kBK / 16; k++)
             mma_bf16(d, dw + (uint64_t)(k * 2), dx + (uint64_t)(k * 2), IDESC,
                      (kb > 0 || k > 0) ? 1u : 0u);
           mma_commit(smem_u32(&empty_bar[stage]));
-          if (++stage == STAGES) { stage = 0; phase ^= 1; }
         }
-        if (ok) mma_commit(smem_u32(&tfull_bar[acc]));
+        __syncwarp();
+        if (++stage == STAGES) { stage = 0; phase ^= 1; }
       }
+      if (ok && elect_one()) mma_commit(smem_u32(&tfull_bar[acc]));
+      __syncwarp();
     }
   } else {
     // ---------------- epilogue (warps 2..9) ----------------
@@ -1074,7 +1121,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t *smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
   const uint32_t box_base = smem_base, w_base = smem_base + kSHBoxStages * kSHBoxStage;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kSHBoxStages; s++) {
@@ -1100,53 +1147,55 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   if (warp == 0) {
     // ---------------- TMA producer: one box per tile, one weight tile per tap ----------------
-    if (lane == 0) {
-      asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
-      asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmW)) : "memory");
-      int bs = 0, ws = 0;
-      uint32_t bph = 0, wph = 0;
-      bool ok = true;
-      for (int t = blockIdx.x; t < tg.total && ok; t += gridDim.x) {
-        int b, oy, ox;
-        patch_origin(a, tg, t, b, oy, ox);
-        if (!mbar_wait(smem_u32(&bempty[bs]), bph ^ 1, &abort_flag, a.err)) break;
+    int bs = 0, ws = 0;
+    uint32_t bph = 0, wph = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < tg.total && ok; t += gridDim.x) {
+      int b, oy, ox;
+      patch_origin(a, tg, t, b, oy, ox);
+      if (!mbar_wait_warp(smem_u32(&bempty[bs]), bph ^ 1, &abort_flag, a.err)) break;
+      if (elect_one()) {
         mbar_expect_tx(smem_u32(&bfull[bs]), kSHBoxBytes);
         tma_load_4d(box_base + bs * kSHBoxStage, &tmA, smem_u32(&bfull[bs]), 0, ox - 1, oy - 1, b);
-        if (++bs == kSHBoxStages) { bs = 0; bph ^= 1; }
-        for (int tap = 0; tap < 9; tap++) {
-          if (!mbar_wait(smem_u32(&wempty[ws]), wph ^ 1, &abort_flag, a.err)) {
-            ok = false;
-            break;
-          }
+      }
+      __syncwarp();
+      if (++bs == kSHBoxStages) { bs = 0; bph ^= 1; }
+      for (int tap = 0; tap < 9; tap++) {
+        if (!mbar_wait_warp(smem_u32(&wempty[ws]), wph ^ 1, &abort_flag, a.err)) {
+          ok = false;
+          break;
+        }
+        if (elect_one()) {
           mbar_expect_tx(smem_u32(&wfull[ws]), kSHWTile);
           tma_load_2d(w_base + ws * kSHWTile, &tmW, smem_u32(&wfull[ws]), tap * kBK, 0);
-          if (++ws == kSHWStages) { ws = 0; wph ^= 1; }
         }
+        __syncwarp();
+        if (++ws == kSHWStages) { ws = 0; wph ^= 1; }
       }
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer: D[128 ch][256 px] += W_tap[128 x 64] X_tap[256 x 64]^T ----------
-    if (lane == 0) {
-      int bs = 0, ws = 0, it = 0;
-      uint32_t bph = 0, wph = 0;
-      bool ok = true;
-      for (int t = blockIdx.x; t < tg.total && ok; t += gridDim.x, it++) {
-        const int acc = it & 1;
-        const uint32_t use = (uint32_t)(it >> 1);
-        if (!mbar_wait(smem_u32(&tempty_bar[acc]), (use & 1) ^ 1, &abort_flag, a.err)) break;
+    int bs = 0, ws = 0, it = 0;
+    uint32_t bph = 0, wph = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < tg.total && ok; t += gridDim.x, it++) {
+      const int acc = it & 1;
+      const uint32_t use = (uint32_t)(it >> 1);
+      if (!mbar_wait_warp(smem_u32(&tempty_bar[acc]), (use & 1) ^ 1, &abort_flag, a.err)) break;
+      if (!mbar_wait_warp(smem_u32(&bfull[bs]), bph, &abort_flag, a.err)) break;
+      tc_fence_after();
+      const uint32_t d = tmem_base + (uint32_t)(acc * kSwapBP);
+      // the box's 8-row groups (patch rows) are one box row apart; the swizzle follows
+      // absolute address bits, so shifted starts keep the phase field at 0
+      const uint64_t db0 = sw128_desc_k(box_base + bs * kSHBoxStage, kSHBoxW * 128, 0);
+#pragma unroll 1
+      for (int tap = 0; tap < 9; tap++) {
+        if (!mbar_wait_warp(smem_u32(&wfull[ws]), wph, &abort_flag, a.err)) {
+          ok = false;
+          break;
+        }
         tc_fence_after();
-        if (!mbar_wait(smem_u32(&bfull[bs]), bph, &abort_flag, a.err)) break;
-        tc_fence_after();
-        const uint32_t d = tmem_base + (uint32_t)(acc * kSwapBP);
-        // the box's 8-row groups (patch rows) are one box row apart; the swizzle follows
-        // absolute address bits, so shifted starts keep the phase field at 0
-        const uint64_t db0 = sw128_desc_k(box_base + bs * kSHBoxStage, kSHBoxW * 128, 0);
-        for (int tap = 0; tap < 9; tap++) {
-          if (!mbar_wait(smem_u32(&wfull[ws]), wph, &abort_flag, a.err)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
+        if (elect_one()) {
           const uint64_t da = sw128_desc(w_base + ws * kSHWTile);
           const uint64_t db = db0 + (uint64_t)(((tap / 3) * kSHBoxW + tap % 3) * 8);
 #pragma unroll
@@ -1154,13 +1203,17 @@ __global__ void __launch_bounds__(kThreads, 1)
             mma_bf16(d, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), IDESC,
                      (tap > 0 || k > 0) ? 1u : 0u);
           mma_commit(smem_u32(&wempty[ws]));
-          if (++ws == kSHWStages) { ws = 0; wph ^= 1; }
         }
-        if (!ok) break;
+        __syncwarp();
+        if (++ws == kSHWStages) { ws = 0; wph ^= 1; }
+      }
+      if (!ok) break;
+      if (elect_one()) {
         mma_commit(smem_u32(&bempty[bs]));
-        if (++bs == kSHBoxStages) { bs = 0; bph ^= 1; }
         mma_commit(smem_u32(&tfull_bar[acc]));
       }
+      __syncwarp();
+      if (++bs == kSHBoxStages) { bs = 0; bph ^= 1; }
     }
   } else {
     // ---------------- epilogue (warps 2..9), as in the pixels-as-N kernel ----------------
@@ -1292,8 +1345,8 @@ cudaError_t encode_wt(CUtensorMap *m, const void *ptr, int N, int K, int BN) {
 
 template <int BN, int STAGES>
 cudaError_t launch_bn(const CUtensorMap &A, const CUtensorMap &B, const CUtensorMap &A2,
-                      const CUtensorMap &B2, const ConvArgs &a, const TcGeom &tg,
-                      cudaStream_t s) {
+                      const CUtensorMap &B2, const CUtensorMap &Bp, const CUtensorMap &B2p,
+                      const ConvArgs &a, const TcGeom &tg, cudaStream_t s) {
   constexpr size_t smem = (size_t)STAGES * (128 * kBK * 2 + BN * kBK * 2) + 8 * kTileT + 1024;
   static_assert(smem <= 227 * 1024, "tcgen05 convolution shared memory");
   static bool attr_set = false;
@@ -1304,7 +1357,7 @@ cudaError_t launch_bn(const CUtensorMap &A, const CUtensorMap &B, const CUtensor
     attr_set = true;
   }
   const int grid = std::min(tg.total, g_num_sms);
-  conv_tc_kernel<BN, STAGES><<<grid, kThreads, smem, s>>>(A, B, A2, B2, a, tg);
+  conv_tc_kernel<BN, STAGES><<<grid, kThreads, smem, s>>>(A, B, A2, B2, Bp, B2p, a, tg);
   return cudaGetLastError();
 }
 
@@ -1553,7 +1606,7 @@ cudaError_t launch_conv_tc(const ConvArgs &a, cudaStream_t s) {
   }
   // 128 output channels: pixels as the MMA's N (256 wide) instead of channels (128 wide)
   const bool swap = a.cout == kSwapBN;
-  const int BN = swap ? kSwapBN : (a.cout >= 256 ? 256 : a.cout);
+  int BN = swap ? kSwapBN : (a.cout >= 256 ? 256 : a.cout);
   const int rows = swap ? kSwapBP : 128;
   TcGeom tg;
   if (a.tiles) {
@@ -1566,14 +1619,44 @@ cudaError_t launch_conv_tc(const ConvArgs &a, cudaStream_t s) {
   } else {
     pick_patch_rows(a.Hb, a.Wb, rows, tg.TH, tg.TW, a.pool_out != nullptr);
   }
-  tg.tx_bytes = tg.TH * tg.TW * kBK * 2 + BN * kBK * 2;
+  tg.tx_bytes = (tg.TH * tg.TW + kSwapBN) * kBK * 2;   // (pixels-as-N kernel)
   tg.tiles_x = (a.Wb + tg.TW - 1) / tg.TW;
   tg.tiles_y = (a.Hb + tg.TH - 1) / tg.TH;
+  const int m_tiles = a.tiles ? a.n_mtiles : a.B * tg.tiles_x * tg.tiles_y;
   tg.n_tiles = a.cout / BN;
-  tg.total = (a.tiles ? a.n_mtiles : a.B * tg.tiles_x * tg.tiles_y) * tg.n_tiles;
+  tg.total = m_tiles * tg.n_tiles;
   if (tg.total <= 0) return cudaSuccess;
-  tg.cin_blocks = a.taps ? a.cin / kBK : 0;
-  tg.kb_main = a.taps * tg.cin_blocks;
+  tg.full = tg.total;
+  tg.split = 1;
+  if (BN == 256) {
+    // The last, partly filled wave of 256-channel tiles runs as 128- or 64-channel parts (the
+    // same sums in the same order) where that ends earlier. Time of a tile: 256 : 128 : 64
+    // channels = 1 : 0.57 : 0.47 (64 blocks of 94 x 100 pixels, 512 -> 512 channels, all tiles of
+    // that width: 1,458, 1,674, 2,763 us). 512 -> 512 at 94 x 126 (192 tiles on 152 SMs):
+    // 58 -> 40 us together with the warp-wide issue loops.
+    const int rest = tg.total % g_num_sms;
+    const int cost[3] = {100, 57, 47};
+    int best = 0;
+    for (int i = 0; i < 3; i++) {
+      const int c = ((rest << i) + g_num_sms - 1) / g_num_sms * cost[i];
+      if (i == 0 || c < best) {
+        best = c;
+        tg.split = 1 << i;
+      }
+    }
+    if (tg.total < g_num_sms && tg.split > 1) {
+      // a launch below one wave: the narrow tile's own kernel (more, smaller stages in flight)
+      BN = 256 / tg.split;
+      tg.n_tiles = a.cout / BN;
+      tg.total = m_tiles * tg.n_tiles;
+      tg.full = tg.total;
+      tg.split = 1;
+    } else {
+      tg.full = tg.total - rest;
+      tg.total = tg.full + rest * tg.split;
+    }
+  }
+  tg.kb_main = a.taps ? a.taps * (a.cin / kBK) : 0;
   tg.kb2 = a.k2 / kBK;
   CUtensorMap mA, mB, mA2, mB2;
   cudaError_t e;
@@ -1587,11 +1670,18 @@ cudaError_t launch_conv_tc(const ConvArgs &a, cudaStream_t s) {
   }
   if (!a.taps) { mA = mA2; mB = mB2; }
   if (!a.k2) { mA2 = mA; mB2 = mB; }
+  CUtensorMap mBp = mB, mB2p = mB2;
+  if (tg.split > 1) {
+    if (a.taps &&
+        (e = encode_wt(&mBp, a.Wt, a.cout, a.taps * a.cin, BN / tg.split)) != cudaSuccess)
+      return e;
+    if (a.k2 && (e = encode_wt(&mB2p, a.W2, a.cout, a.k2, BN / tg.split)) != cudaSuccess) return e;
+  }
   if (swap) return launch_swap<4>(mA, mB, mA2, mB2, a, tg, s);
   switch (BN) {
-    case 64: return launch_bn<64, 8>(mA, mB, mA2, mB2, a, tg, s);
-    case 128: return launch_bn<128, 6>(mA, mB, mA2, mB2, a, tg, s);
-    case 256: return launch_bn<256, 4>(mA, mB, mA2, mB2, a, tg, s);
+    case 64: return launch_bn<64, 8>(mA, mB, mA2, mB2, mBp, mB2p, a, tg, s);
+    case 128: return launch_bn<128, 6>(mA, mB, mA2, mB2, mBp, mB2p, a, tg, s);
+    case 256: return launch_bn<256, 4>(mA, mB, mA2, mB2, mBp, mB2p, a, tg, s);
     default: return cudaErrorInvalidValue;
   }
 }

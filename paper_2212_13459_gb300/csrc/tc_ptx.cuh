@@ -86,12 +86,24 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
                                           unsigned *err) {
   return mbar_wait_limit(bar, parity, abort_flag, err, kWaitCycles);
 }
-// Bounded wait taken by lane 0 and broadcast, so that the whole warp continues or leaves as one.
+// Bounded wait of a whole warp: every lane tests the barrier, and the warp continues or leaves as
+// one. A loop that a single lane runs (waits, descriptors, the operands of TMA and MMA
+// instructions, which live in uniform registers) issues several times slower than the same loop
+// run by the whole warp with one elected lane at the TMA / MMA instructions; so does a wait that
+// lane 0 takes and broadcasts.
+static __device__ __noinline__ bool mbar_wait_warp_slow(uint32_t bar, uint32_t parity,
+                                                 volatile int *abort_flag, unsigned *err) {
+  const bool ok = mbar_wait(bar, parity, abort_flag, err);
+  return __all_sync(0xffffffffu, ok);
+}
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity,
                                                volatile int *abort_flag, unsigned *err) {
-  int ok = 0;
-  if ((threadIdx.x & 31) == 0) ok = mbar_wait(bar, parity, abort_flag, err) ? 1 : 0;
-  return __shfl_sync(0xffffffffu, ok, 0) != 0;
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  return mbar_wait_warp_slow(bar, parity, abort_flag, err);
+}
+// This thread's warp index as a value the compiler knows to be the same in all lanes
+__device__ __forceinline__ int warp_index() {
+  return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
 }
 // One lane of a fully active warp (the same lane every time): the issuing lane of tcgen05.mma
 // and tcgen05.commit in loops that the whole warp runs.
