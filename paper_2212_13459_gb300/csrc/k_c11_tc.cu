@@ -43,11 +43,14 @@ __device__ __forceinline__ uint32_t sw128_chunk(int r, int c) {
 // ------------------------------------------------------------------------------------------------
 // Step 1: the block image in the BF16 form, one 16-byte pixel per buffer pixel:
 // xs[b][y][x] = (hi_0, hi_1, hi_2, lo_0, lo_1, lo_2, 0, 0) inside the block's valid extent, zero
-// elsewhere (the block is a standalone image with zero padding).
+// elsewhere (the block is a standalone image with zero padding). err (optional): a non-finite
+// image value is latched there (every image pixel is some block's).
 __global__ void __launch_bounds__(256) conv11_stage_kernel(const float *__restrict__ img, int H,
                                                            int W, const BlockGeom *__restrict__ geom,
                                                            int B, int Hb, int Wb,
-                                                           uint4 *__restrict__ xs) {
+                                                           uint4 *__restrict__ xs,
+                                                           unsigned *__restrict__ err) {
+  bool bad = false;
   const int npix = B * Hb * Wb;
   const size_t plane = (size_t)H * W;
   for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < npix; p += gridDim.x * blockDim.x) {
@@ -61,6 +64,7 @@ __global__ void __launch_bounds__(256) conv11_stage_kernel(const float *__restri
 #pragma unroll
       for (int ci = 0; ci < 3; ci++) {
         const float v = __ldg(img + ci * plane + off);
+        bad |= !isfinite(v);
         hi[ci] = __bfloat162float(__float2bfloat16_rn(v));
         lo[ci] = v - hi[ci];   // exact in FP32; rounded to BF16 by the packing below
       }
@@ -69,6 +73,7 @@ __global__ void __launch_bounds__(256) conv11_stage_kernel(const float *__restri
     }
     xs[p] = o;
   }
+  if (err && __syncthreads_or(bad) && threadIdx.x == 0) atomicOr(err, kErrNonfinite);
 }
 
 // Step 2: the convolution, D[p][n] = sum_k A[p][k] B[n][k] with M = a 16 x 8 output patch and
@@ -564,8 +569,8 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t
 cudaError_t launch_conv11_fwd_tc(const float *img, int H, int W, const float *w11,
                                  const float *bias, const BlockGeom *geom, int B, int Hb, int Wb,
                                  void *stage_buf, __nv_bfloat16 *out, const int4 *patches,
-                                 int npatches, float *gram_part, int *gram_runs, unsigned *err,
-                                 cudaStream_t s) {
+                                 int npatches, float *gram_part, int *gram_runs,
+                                 bool check_finite, unsigned *err, cudaStream_t s) {
   if (gram_runs) *gram_runs = 0;
   if (gram_part && (!patches || !gram_runs)) return cudaErrorInvalidValue;
   static bool attr = false;
@@ -582,7 +587,8 @@ cudaError_t launch_conv11_fwd_tc(const float *img, int H, int W, const float *w1
   if (reinterpret_cast<uintptr_t>(stage_buf) % 16) return cudaErrorInvalidValue;
   const int sgrid = (int)std::min<long long>((npix + 255) / 256, 32LL * tc_num_sms());
   conv11_stage_kernel<<<sgrid, 256, 0, s>>>(img, H, W, geom, B, Hb, Wb,
-                                            reinterpret_cast<uint4 *>(stage_buf));
+                                            reinterpret_cast<uint4 *>(stage_buf),
+                                            check_finite ? err : nullptr);
   EncodeTiledFn enc = reinterpret_cast<EncodeTiledFn>(tc_encode_tiled_fn());
   if (!enc) return cudaErrorNotSupported;
   CUtensorMap m;

@@ -189,70 +189,65 @@ __device__ __forceinline__ void two_sum_add(float &s, float &c, float x) {
   s = t;
 }
 
-// Gacc[i][j] += sum over runs (fixed order, compensated FP32, then FP64) of the FP32 tile
-// partials. A CTA takes 32 V consecutive elements (V per lane: one float4 load per run when
-// V = 4, coalesced); its NW warps split the runs (warp w sums runs w, w + NW, ... in order) and
-// the NW partial pairs are added in warp order (deterministic); each element's pair is converted
-// to FP64 once and added to Gacc. A warp issues the loads of up to 8 of its runs before adding
-// them (in run order), so the loads are in flight together instead of one after another.
-// C^2 is a multiple of 4096 and V consecutive elements stay inside one N-wide tile row, so the
-// V elements of a lane are contiguous in every run's partial.
-template <int V, int NW>
-__global__ void __launch_bounds__(NW * 32) gram_tc_reduce_kernel(const float *__restrict__ part,
-                                                                 int nruns, int C, int N, int nI,
-                                                                 int nJ,
-                                                                 double *__restrict__ Gacc) {
-  __shared__ float2 red[NW][32 * V];
-  const long long n = (long long)C * C;
+// Gacc[i][j] (+)= sum over runs (fixed order, compensated FP32, then FP64) of the FP32 tile
+// partials, all style layers in one launch. A warp takes 128 consecutive elements (a float4 per
+// lane and run, coalesced; C^2 is a multiple of 4096 and four consecutive elements stay inside one
+// N-wide tile row) and issues the loads of up to 8 of its runs before adding them in run order; a
+// layer with many runs splits them over `split` warps of a CTA (warp s: runs s, s + split, ...),
+// whose pairs are added in warp order (deterministic). Each element's pair becomes FP64 once.
+// Bound: the read of the partials from L2. One launch per layer, with 64-bit index divisions and
+// two barriers per 128 elements, took 58 us (64 x 64 pixels) to 83 us (756 x 1008) per evaluation;
+// this takes 13 and 60 us (cold, under the profiler; 125 MB of partials at 756 x 1008).
+constexpr int kRedWarps = 16;
+__global__ void __launch_bounds__(kRedWarps * 32) gram_tc_reduce_kernel(GramReduceArgs a) {
+  __shared__ float2 red[kRedWarps][128];
+  int l = 0;
+  while (l + 1 < a.n && (int)blockIdx.x >= a.L[l + 1].cta0) l++;
+  const GramReduceLayer L = a.L[l];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const size_t stride = (size_t)nI * nJ * 128 * N;
-  for (long long e0 = (long long)blockIdx.x * 32 * V; e0 < n;
-       e0 += (long long)gridDim.x * 32 * V) {
-    const long long e = e0 + (long long)lane * V;
-    float s[V], c[V];
+  const int sub = warp % L.split, grp = warp / L.split;
+  const int e = (((int)blockIdx.x - L.cta0) * (kRedWarps / L.split) + grp) * 128 + lane * 4;
+  const bool live = e < L.C * L.C;
+  float s[4] = {0.f, 0.f, 0.f, 0.f}, c[4] = {0.f, 0.f, 0.f, 0.f};
+  if (live) {
+    const int i = e / L.C, j = e % L.C;
+    const size_t off = ((size_t)((i / 128) * L.nJ + j / L.N) * 128 + (i % 128)) * L.N + (j % L.N);
+    const size_t stride = (size_t)L.nI * L.nJ * 128 * L.N;
+    for (int r0 = sub; r0 < L.nruns; r0 += 8 * L.split) {
+      float4 v[8];
 #pragma unroll
-    for (int k = 0; k < V; k++) s[k] = c[k] = 0.f;
-    if (e < n) {
-      const int i = (int)(e / C), j = (int)(e % C);
-      const int tile = (i / 128) * nJ + j / N;
-      const size_t off = ((size_t)tile * 128 + (i % 128)) * N + (j % N);
-      for (int r0 = warp; r0 < nruns; r0 += 8 * NW) {
-        float v[8][V];
+      for (int u = 0; u < 8; u++)
+        if (r0 + L.split * u < L.nruns)
+          v[u] = __ldg(reinterpret_cast<const float4 *>(L.part + (size_t)(r0 + L.split * u) * stride + off));
 #pragma unroll
-        for (int u = 0; u < 8; u++) {
-          const int r = r0 + NW * u;
-          if constexpr (V == 4) {
-            const float4 q = r < nruns
-                                 ? __ldg(reinterpret_cast<const float4 *>(part + (size_t)r * stride + off))
-                                 : make_float4(0.f, 0.f, 0.f, 0.f);
-            v[u][0] = q.x; v[u][1] = q.y; v[u][2] = q.z; v[u][3] = q.w;
-          } else {
-            v[u][0] = r < nruns ? __ldg(part + (size_t)r * stride + off) : 0.f;
-          }
+      for (int u = 0; u < 8; u++)
+        if (r0 + L.split * u < L.nruns) {
+          two_sum_add(s[0], c[0], v[u].x);
+          two_sum_add(s[1], c[1], v[u].y);
+          two_sum_add(s[2], c[2], v[u].z);
+          two_sum_add(s[3], c[3], v[u].w);
         }
-#pragma unroll
-        for (int u = 0; u < 8; u++)
-          if (r0 + NW * u < nruns)
-#pragma unroll
-            for (int k = 0; k < V; k++) two_sum_add(s[k], c[k], v[u][k]);
-      }
     }
+  }
+  if (L.split > 1) {
 #pragma unroll
-    for (int k = 0; k < V; k++) red[warp][lane * V + k] = make_float2(s[k], c[k]);
+    for (int k = 0; k < 4; k++) red[warp][lane * 4 + k] = make_float2(s[k], c[k]);
     __syncthreads();
-    for (int q = threadIdx.x; q < 32 * V; q += NW * 32) {
-      if (e0 + q < n) {
-        float ts = 0.f, tc = 0.f;
+    if (sub) return;
+    for (int w = 1; w < L.split; w++)
 #pragma unroll
-        for (int w = 0; w < NW; w++) {
-          const float2 p = red[w][q];
-          two_sum_add(ts, tc, p.x);
-          tc += p.y;
-        }
-        Gacc[e0 + q] += (double)ts + (double)tc;
+      for (int k = 0; k < 4; k++) {
+        const float2 p = red[warp + w][lane * 4 + k];
+        two_sum_add(s[k], c[k], p.x);
+        c[k] += p.y;
       }
-    }
-    __syncthreads();
+  }
+  if (!live) return;
+  double *g = L.Gacc + e;
+#pragma unroll
+  for (int k = 0; k < 4; k++) {
+    const double v = (double)s[k] + (double)c[k];
+    g[k] = a.overwrite ? v : g[k] + v;
   }
 }
 
@@ -322,34 +317,29 @@ cudaError_t encode_gram_map(CUtensorMap *m, const void *base, int C, int own_w, 
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-cudaError_t launch_gram_tc(const GramTcArgs &a, int nruns, double *Gacc, cudaStream_t s) {
+cudaError_t launch_gram_tc(const GramTcArgs &a, int nruns, cudaStream_t s) {
   if (nruns <= 0) return cudaSuccess;
-  cudaError_t e;
   const bool aload = gram_needs_aload(a);
   switch (a.N) {
-    case 64: e = aload ? launch_n<64, true>(a, nruns, s) : launch_n<64, false>(a, nruns, s); break;
-    case 128: e = aload ? launch_n<128, true>(a, nruns, s) : launch_n<128, false>(a, nruns, s); break;
-    case 256: e = aload ? launch_n<256, true>(a, nruns, s) : launch_n<256, false>(a, nruns, s); break;
+    case 64: return aload ? launch_n<64, true>(a, nruns, s) : launch_n<64, false>(a, nruns, s);
+    case 128: return aload ? launch_n<128, true>(a, nruns, s) : launch_n<128, false>(a, nruns, s);
+    case 256: return aload ? launch_n<256, true>(a, nruns, s) : launch_n<256, false>(a, nruns, s);
     default: return cudaErrorInvalidValue;
   }
-  if (e != cudaSuccess) return e;
-  return launch_gram_tc_reduce(a.part, nruns, a.C, a.N, a.nI, a.nJ, Gacc, s);
 }
 
-cudaError_t launch_gram_tc_reduce(const float *part, int nruns, int C, int N, int nI, int nJ,
-                                  double *Gacc, cudaStream_t s) {
-  if (nruns <= 0) return cudaSuccess;
-  // float4 lanes where that still gives two CTAs per SM; otherwise one element per lane and 16
-  // warps per CTA splitting the runs (C = 64, 128: few elements, several hundred runs)
-  const long long n = (long long)C * C;
-  const int sms = tc_num_sms();
-  if (n / 128 >= 2LL * sms) {
-    const int grid = (int)std::min<long long>(n / 128, 8LL * sms);
-    gram_tc_reduce_kernel<4, 8><<<grid, 256, 0, s>>>(part, nruns, C, N, nI, nJ, Gacc);
-  } else {
-    const int grid = (int)std::min<long long>(n / 32, 4LL * sms);
-    gram_tc_reduce_kernel<1, 16><<<grid, 512, 0, s>>>(part, nruns, C, N, nI, nJ, Gacc);
+cudaError_t launch_gram_tc_reduce(GramReduceArgs a, cudaStream_t s) {
+  int ctas = 0;
+  for (int l = 0; l < a.n; l++) {
+    GramReduceLayer &L = a.L[l];
+    // about eight runs per warp: one batch of loads
+    L.split = L.nruns <= 8 ? 1 : L.nruns <= 16 ? 2 : L.nruns <= 32 ? 4 : L.nruns <= 64 ? 8 : 16;
+    L.cta0 = ctas;
+    const int per = 128 * (kRedWarps / L.split);
+    ctas += (L.C * L.C + per - 1) / per;
   }
+  if (ctas <= 0) return cudaSuccess;
+  gram_tc_reduce_kernel<<<ctas, kRedWarps * 32, 0, s>>>(a);
   return cudaGetLastError();
 }
 

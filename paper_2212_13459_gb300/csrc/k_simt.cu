@@ -831,87 +831,96 @@ void launch_gram_reduce(const float *part, int nchunks, int C, double *Gacc, cud
 }
 
 // ---- style finalisation: G = Gacc / np, E_L = w ||G - Ghat||^2, R = (4 w / np)(G - Ghat) -------------
-// One CTA of 1024 threads per style layer; deterministic reduction.
-// Stage 1 (one CTA per layer): mean / std terms of Eq. 5 per channel, from the channel sums and
-// diag(G): beta_j (added to R's diagonal), alpha_j (epilogue offset), the moment loss, and the
-// moments themselves when requested.
-__global__ void __launch_bounds__(512) style_moments_kernel(StyleFinalizeArgs a) {
-  __shared__ double red[512];
-  const StyleLayerArgs L = a.L[blockIdx.x];
-  const double inv = 1.0 / L.np;
-  double s = 0.0;
-  for (int j = threadIdx.x; j < L.C; j += blockDim.x) {
-    double b = 0.0;
-    if (L.S) {
+// One launch over the elements of all layers. The thread of a diagonal element also forms the
+// channel's mean / std terms of Eq. 5 from the channel sum and G_jj: beta_j (added to R_jj),
+// alpha_j (epilogue offset), its share of the moment loss, and the moments themselves when
+// requested. The CTAs' loss partials are added per layer, in CTA order, by the last CTA to finish.
+// Bound: FP64 (about seven operations per element at two per SM and clock) and latency; four
+// elements per thread are loaded together. Three launches with 16 elements in turn per thread and
+// 64-bit divisions took 36 us; this takes 16.
+constexpr int kFinThreads = 256, kFinPer = 4 * kFinThreads;   // elements per CTA
+static_assert(kFinalizeCtas * kFinPer >= 64 * 64 + 128 * 128 + 256 * 256 + 2 * 512 * 512 &&
+              4096 % kFinPer == 0, "every CTA lies in one layer");
+__global__ void __launch_bounds__(kFinThreads) style_finalize_kernel(StyleFinalizeArgs a) {
+  __shared__ double red[kFinThreads];
+  __shared__ int last_sh;
+  const int tid = threadIdx.x;
+  int l = 0, b = blockIdx.x;
+  while (b >= a.L[l].C * a.L[l].C / kFinPer) b -= a.L[l].C * a.L[l].C / kFinPer, l++;
+  const StyleLayerArgs L = a.L[l];
+  const double inv = L.inv_np, rs = L.rs;
+  double s = 0.0, g[4], h[4];
+  const int e0 = b * kFinPer + tid;
+#pragma unroll
+  for (int k = 0; k < 4; k++) {
+    g[k] = L.Gacc[e0 + k * kFinThreads];
+    h[k] = L.Ghat ? L.Ghat[e0 + k * kFinThreads] : 0.0;
+  }
+#pragma unroll
+  for (int k = 0; k < 4; k++) {
+    const int e = e0 + k * kFinThreads;
+    const double G = g[k] * inv, d = G - h[k];
+    L.Gout[e] = G;
+    s += L.w * d * d;
+    double r = rs * d;
+    const int i = e / L.C, j = e % L.C;
+    if (i == j && L.S) {
       // rounded products (no contraction into an FMA), so the loss pass reproduces the target
       // pass's mean bit for bit when x = v
       const double m = __dmul_rn(L.S[j], inv);
-      const double var = __dmul_rn(L.Gacc[(long long)j * L.C + j], inv) - __dmul_rn(m, m);
+      const double var = __dmul_rn(g[k], inv) - __dmul_rn(m, m);
       const double sd = var > 0.0 ? sqrt(var) : 0.0;
       if (L.mean_out) L.mean_out[j] = m;
       if (L.std_out) L.std_out[j] = sd;
       if (L.mu) {
         s += L.wm * (m - L.mu[j]) * (m - L.mu[j]) + L.ws * (sd - L.sigma[j]) * (sd - L.sigma[j]);
-        b = sd > 0.0 ? L.ws * 2.0 * inv * (sd - L.sigma[j]) / sd : 0.0;
-        if (L.alpha) L.alpha[j] = (float)(L.wm * 2.0 * inv * (m - L.mu[j]) - b * m);
+        const double beta = sd > 0.0 ? L.ws * 2.0 * inv * (sd - L.sigma[j]) / sd : 0.0;
+        if (L.alpha) L.alpha[j] = (float)(L.wm * 2.0 * inv * (m - L.mu[j]) - beta * m);
+        r += beta;
       }
     }
-    a.beta[blockIdx.x * 512 + j] = b;
-  }
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int k = 256; k > 0; k >>= 1) {
-    if (threadIdx.x < k) red[threadIdx.x] += red[threadIdx.x + k];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) a.partial[blockIdx.x * kFinalizeChunks] = red[0];
-}
-
-// Stage 2 (grid: layer x chunk): G = Gacc / np, R = (4 w / np)(G - Ghat) + diag(beta), and the
-// chunk's share of w ||G - Ghat||^2 into partial[layer][1 + chunk]
-__global__ void __launch_bounds__(256) style_residual_kernel(StyleFinalizeArgs a) {
-  __shared__ double red[256];
-  const StyleLayerArgs L = a.L[blockIdx.x];
-  const long long n = (long long)L.C * L.C;
-  const long long per = (n + gridDim.y - 1) / gridDim.y;
-  const long long e0 = blockIdx.y * per, e1 = e0 + per < n ? e0 + per : n;
-  const double inv = 1.0 / L.np, rs = 4.0 * L.w / L.np;
-  double s = 0.0;
-  for (long long e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
-    const double G = L.Gacc[e] * inv;
-    const double d = G - L.Ghat[e];
-    L.Gout[e] = G;
-    s += L.w * d * d;
-    const int i = (int)(e / L.C), j = (int)(e % L.C);
-    const double r = rs * d + (i == j ? a.beta[blockIdx.x * 512 + j] : 0.0);
     if (a.r_is_bf16)
       reinterpret_cast<__nv_bfloat16 *>(L.R)[e] = __float2bfloat16_rn((float)r);
     else
       reinterpret_cast<float *>(L.R)[e] = (float)r;
   }
-  red[threadIdx.x] = s;
+  red[tid] = s;
   __syncthreads();
-  for (int k = 128; k > 0; k >>= 1) {
-    if (threadIdx.x < k) red[threadIdx.x] += red[threadIdx.x + k];
+  for (int k = kFinThreads / 2; k > 0; k >>= 1) {
+    if (tid < k) red[tid] += red[tid + k];
     __syncthreads();
   }
-  if (threadIdx.x == 0) a.partial[blockIdx.x * kFinalizeChunks + 1 + blockIdx.y] = red[0];
-}
-
-// Stage 3: E_L = sum of the layer's partials in a fixed order
-__global__ void style_sum_kernel(StyleFinalizeArgs a, int chunks) {
-  const int l = threadIdx.x;
-  if (l < kNStyle) {
-    double s = 0.0;
-    for (int c = 0; c <= chunks; c++) s += a.partial[l * kFinalizeChunks + c];
-    a.Eparts[l] = s;
+  if (tid == 0) {
+    a.partial[blockIdx.x] = red[0];
+    __threadfence();
+    last_sh = atomicAdd(a.arrived, 1u) == gridDim.x - 1;
   }
+  __syncthreads();
+  if (!last_sh) return;
+  __threadfence();
+  if (tid < 32 * kNStyle) {   // a warp per layer: lane q the CTAs q, q + 32, ... in order, a tree
+    const int wl = tid >> 5;
+    int c0 = 0;
+    for (int q = 0; q < wl; q++) c0 += a.L[q].C * a.L[q].C / kFinPer;
+    const int n = a.L[wl].C * a.L[wl].C / kFinPer;
+    double t = 0.0;
+    for (int q = tid & 31; q < n; q += 32) t += __ldcg(a.partial + c0 + q);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if ((tid & 31) == 0) a.Eparts[wl] = t;
+  }
+  if (tid == 0) *a.arrived = 0u;
 }
 
 void launch_style_finalize(const StyleFinalizeArgs &a, cudaStream_t s) {
-  style_moments_kernel<<<kNStyle, 512, 0, s>>>(a);
-  style_residual_kernel<<<dim3(kNStyle, kFinalizeChunks - 1), 256, 0, s>>>(a);
-  style_sum_kernel<<<1, 32, 0, s>>>(a, kFinalizeChunks - 1);
+  int n = 0;
+  StyleFinalizeArgs b = a;
+  for (int l = 0; l < kNStyle; l++) {
+    n += a.L[l].C * a.L[l].C;
+    b.L[l].inv_np = 1.0 / a.L[l].np;   // (two FP64 divisions per thread are half the kernel)
+    b.L[l].rs = 4.0 * a.L[l].w / a.L[l].np;
+  }
+  style_finalize_kernel<<<n / kFinPer, kFinThreads, 0, s>>>(b);
 }
 
 // ---- channel sums over owned pixels, all style layers in one launch -------------------------------
@@ -1038,82 +1047,78 @@ template void launch_chansum<float>(ChansumArgs, cudaStream_t);
 template void launch_chansum<__nv_bfloat16>(ChansumArgs, cudaStream_t);
 
 
-// ---- content loss over owned pixels: partial[c] = sum (V - Vu)^2 (FP64) ----------------------------
+// ---- content loss over owned pixels: parts[5] (+)= lambda sum (V - Vu)^2 ----------------------------
+// partial[c] = chunk c's sum; the last CTA to finish adds the partials (thread t: t, t + 256, ... in
+// order, then a fixed tree) and, for the evaluation's last batch, the six parts into the loss.
 template <typename T>
-__global__ void __launch_bounds__(256) content_partial_kernel(
-    const T *__restrict__ V, int Hb, int Wb, const T *__restrict__ Vu, int Hc, int Wc,
-    const BlockGeom *__restrict__ geom, const OwnRect *__restrict__ own,
-    const GramChunk *__restrict__ chunks, double *__restrict__ partial) {
+__global__ void __launch_bounds__(256) content_loss_kernel(ContentLossArgs a) {
   __shared__ double red[256];
-  const GramChunk ch = chunks[blockIdx.x];
-  const OwnRect r = own[ch.b];
-  const BlockGeom g = geom[ch.b];
-  const int rw = r.x1 - r.x0;
-  const int oy = g.ey0 >> kContentLevel, ox = g.ex0 >> kContentLevel;
-  double s = 0.0;
-  // 64 threads per pixel row of 512 channels (8 each)
-  for (int q = ch.p0 + (threadIdx.x >> 6); q < ch.p1; q += 4) {
-    const int y = r.y0 + q / rw, x = r.x0 + q % rw;
-    const int c = (threadIdx.x & 63) * 8;
-    float a[8], t[8];
-    load8(V + (((size_t)ch.b * Hb + y) * Wb + x) * 512 + c, a);
-    load8(Vu + ((size_t)(oy + y) * Wc + ox + x) * 512 + c, t);
-    // differences of two stored values are exact in FP32 (BF16 inputs) or nearly so (FP32
-    // inputs); 8 squares summed in FP32, then accumulated in FP64
-    float f = 0.f;
-#pragma unroll
-    for (int j = 0; j < 8; j++) {
-      const float d = a[j] - t[j];
-      f = fmaf(d, d, f);
+  __shared__ int last_sh;
+  auto tree = [&]() {
+    __syncthreads();
+    for (int k = 128; k > 0; k >>= 1) {
+      if (threadIdx.x < k) red[threadIdx.x] += red[threadIdx.x + k];
+      __syncthreads();
     }
-    s += (double)f;
-  }
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int k = 128; k > 0; k >>= 1) {
-    if (threadIdx.x < k) red[threadIdx.x] += red[threadIdx.x + k];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) partial[blockIdx.x] = red[0];
-}
-
-// acc += lambda * sum_c partial[c] in a fixed order
-// (256 threads: thread t adds partials t, t + 256, ... in order, then a fixed tree; the same
-// order every time, several times faster than one thread adding a thousand partials in turn)
-__global__ void __launch_bounds__(256) content_reduce_kernel(const double *__restrict__ partial,
-                                                             int n, double lambda,
-                                                             double *__restrict__ acc) {
-  __shared__ double red[256];
+  };
   double s = 0.0;
-  for (int i = threadIdx.x; i < n; i += 256) s += partial[i];
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int k = 128; k > 0; k >>= 1) {
-    if (threadIdx.x < k) red[threadIdx.x] += red[threadIdx.x + k];
-    __syncthreads();
+  if ((int)blockIdx.x < a.nchunks) {
+    const GramChunk ch = a.chunks[blockIdx.x];
+    const OwnRect r = a.own[ch.b];
+    const BlockGeom g = a.geom[ch.b];
+    const int rw = r.x1 - r.x0;
+    const int oy = g.ey0 >> kContentLevel, ox = g.ex0 >> kContentLevel;
+    const T *V = reinterpret_cast<const T *>(a.V), *Vu = reinterpret_cast<const T *>(a.Vu);
+    // 64 threads per pixel row of 512 channels (8 each)
+    for (int q = ch.p0 + (threadIdx.x >> 6); q < ch.p1; q += 4) {
+      const int y = r.y0 + q / rw, x = r.x0 + q % rw;
+      const int c = (threadIdx.x & 63) * 8;
+      float v[8], t[8];
+      load8(V + (((size_t)ch.b * a.Hb + y) * a.Wb + x) * 512 + c, v);
+      load8(Vu + ((size_t)(oy + y) * a.Wc + ox + x) * 512 + c, t);
+      // differences of two stored values are exact in FP32 (BF16 inputs) or nearly so (FP32
+      // inputs); 8 squares summed in FP32, then accumulated in FP64
+      float f = 0.f;
+#pragma unroll
+      for (int j = 0; j < 8; j++) {
+        const float d = v[j] - t[j];
+        f = fmaf(d, d, f);
+      }
+      s += (double)f;
+    }
   }
-  if (threadIdx.x == 0) *acc += lambda * red[0];
+  red[threadIdx.x] = s;
+  tree();
+  if (threadIdx.x == 0) {
+    a.partial[blockIdx.x] = red[0];
+    __threadfence();
+    last_sh = atomicAdd(a.arrived, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last_sh) return;
+  __threadfence();
+  s = 0.0;
+  for (int i = threadIdx.x; i < (int)gridDim.x; i += 256) s += __ldcg(a.partial + i);
+  red[threadIdx.x] = s;
+  tree();
+  if (threadIdx.x == 0) {
+    const double c = a.lambda * red[0] + (a.first ? 0.0 : a.parts[kNStyle]);
+    a.parts[kNStyle] = c;
+    if (a.loss) {
+      double t = 0.0;
+      for (int i = 0; i < kNStyle; i++) t += a.parts[i];
+      *a.loss = t + c;
+    }
+    *a.arrived = 0u;
+  }
 }
 
 template <typename T>
-void launch_content_loss(const T *V, int Hb, int Wb, const T *Vu, int Hc, int Wc,
-                         const BlockGeom *geom, const OwnRect *own, const GramChunk *chunks,
-                         int nchunks, double *partial, double lambda, double *acc,
-                         cudaStream_t s) {
-  if (nchunks > 0) {
-    content_partial_kernel<T><<<nchunks, 256, 0, s>>>(V, Hb, Wb, Vu, Hc, Wc, geom, own, chunks,
-                                                      partial);
-    content_reduce_kernel<<<1, 256, 0, s>>>(partial, nchunks, lambda, acc);
-  }
+void launch_content_loss(const ContentLossArgs &a, cudaStream_t s) {
+  content_loss_kernel<T><<<a.nchunks > 0 ? a.nchunks : 1, 256, 0, s>>>(a);
 }
-template void launch_content_loss<float>(const float *, int, int, const float *, int, int,
-                                         const BlockGeom *, const OwnRect *, const GramChunk *,
-                                         int, double *, double, double *, cudaStream_t);
-template void launch_content_loss<__nv_bfloat16>(const __nv_bfloat16 *, int, int,
-                                                 const __nv_bfloat16 *, int, int,
-                                                 const BlockGeom *, const OwnRect *,
-                                                 const GramChunk *, int, double *, double,
-                                                 double *, cudaStream_t);
+template void launch_content_loss<float>(const ContentLossArgs &, cudaStream_t);
+template void launch_content_loss<__nv_bfloat16>(const ContentLossArgs &, cudaStream_t);
 
 // ---- content target crop: owned ReLU4_2 features of each block into the global map ------------------
 template <typename T>
@@ -1166,18 +1171,6 @@ __global__ void check_finite_kernel(const float *__restrict__ x, long long n,
 }
 void launch_check_finite(const float *x, long long n, unsigned *err, cudaStream_t s) {
   check_finite_kernel<<<ew_grid(n), 256, 0, s>>>(x, n, err);
-}
-
-// loss = sum of the five style parts + content part, in fixed order
-__global__ void finish_loss_kernel(const double *__restrict__ parts, double *__restrict__ loss) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double s = 0.0;
-    for (int i = 0; i < kNStyle + 1; i++) s += parts[i];
-    if (loss) *loss = s;
-  }
-}
-void launch_finish_loss(const double *parts, double *loss, cudaStream_t s) {
-  finish_loss_kernel<<<1, 32, 0, s>>>(parts, loss);
 }
 
 }  // namespace nst

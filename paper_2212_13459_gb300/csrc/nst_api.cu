@@ -199,7 +199,8 @@ struct nst_ctx {
   double *d_sacc = nullptr, *d_mu = nullptr, *d_sigma = nullptr, *d_cspart = nullptr;
   float *d_alpha = nullptr;
   size_t cspart_cap = 0;
-  double *d_fin = nullptr;   // style finaliser scratch: beta [5][512] then partials
+  double *d_fin = nullptr;        // style finaliser: loss partials
+  unsigned *d_arrived = nullptr;  // [2] arrival counters: style finaliser, content loss
   // workspace (grow-only)
   void *d_ws = nullptr;
   size_t ws_cap = 0;
@@ -441,8 +442,10 @@ nst_status build_plan(nst_ctx *ctx, int H, int W, int margin, PassPlan **out) {
         tot += (long long)(r.y1 - r.y0) * (r.x1 - r.x0);
       }
       const long long target = s < kNStyle ? std::max(1, 1216 / npairs) : 608;
-      long long ch = std::max(256LL, (tot + target - 1) / target);
-      ch = (ch + 31) / 32 * 32;
+      // (the content loss has no partial tile to write per chunk: short chunks, more CTAs)
+      const long long unit = s < kNStyle ? 32 : 8;
+      long long ch = std::max(s < kNStyle ? 256LL : 8LL, (tot + target - 1) / target);
+      ch = (ch + unit - 1) / unit * unit;
       bt.chunk_off[s] = (int)chunks.size();
       for (int i = t0; i < t0 + bt.B; i++) {
         const OwnRect &r = own[(size_t)slot * nt + i];
@@ -462,6 +465,7 @@ nst_status build_plan(nst_ctx *ctx, int H, int W, int margin, PassPlan **out) {
     for (int si = 0; si < kNStyle; si++)
       cs += (size_t)bt.nchunks[si] * bt.cs_split[si] * kStyleC[si];
     p.chansum_doubles = std::max(p.chansum_doubles, cs);
+    size_t tc_part = 0;   // all layers' partial tiles
     for (int si = 0; si < kNStyle; si++) {
       int N, nI, nJ;
       gram_tc_shape(kStyleC[si], &N, &nI, &nJ);
@@ -490,9 +494,9 @@ nst_status build_plan(nst_ctx *ctx, int H, int W, int margin, PassPlan **out) {
           tcchunks.push_back({i - t0, (int)k, (int)std::min(nb, k + per), nbx});
       }
       bt.tc_runs[si] = (int)tcchunks.size() - bt.tc_off[si];
-      p.gram_part_floats = std::max(p.gram_part_floats,
-                                    (size_t)bt.tc_runs[si] * nI * nJ * 128 * N);
+      tc_part += (size_t)bt.tc_runs[si] * nI * nJ * 128 * N;
     }
+    p.gram_part_floats = std::max(p.gram_part_floats, tc_part);
     bt.max_inner_px = 0;
     bt.max_content_px = 0;
     bt.max_inner_h = bt.max_inner_w = 0;
@@ -686,11 +690,11 @@ nst_status ensure_buffers(nst_ctx *ctx, const PassPlan &p, Workspace &ws) {
     CK(cudaMalloc(&ctx->d_cspart, sizeof(double) * p.chansum_doubles));
     ctx->cspart_cap = p.chansum_doubles;
   }
-  if ((size_t)p.max_content_chunks > ctx->cpart_cap) {
+  if ((size_t)std::max(1, p.max_content_chunks) > ctx->cpart_cap) {
     if (ctx->d_cpart) CK(cudaFree(ctx->d_cpart));
     ctx->d_cpart = nullptr;
-    CK(cudaMalloc(&ctx->d_cpart, sizeof(double) * p.max_content_chunks));
-    ctx->cpart_cap = p.max_content_chunks;
+    CK(cudaMalloc(&ctx->d_cpart, sizeof(double) * std::max(1, p.max_content_chunks)));
+    ctx->cpart_cap = std::max(1, p.max_content_chunks);
   }
   return NST_OK;
 }
@@ -727,7 +731,7 @@ nst_status run_conv(nst_ctx *ctx, ConvArgs a, cudaStream_t s) {
 template <typename T>
 nst_status forward_batch(nst_ctx *ctx, const PassPlan &p, const Batch &bt, const Workspace &ws,
                          const float *img, int last_conv, bool for_backward, cudaStream_t s,
-                         bool grams = false) {
+                         bool grams = false, bool check_finite = false) {
   const BlockGeom *geom = p.d_geom + bt.t0;
   ctx->g11_runs = 0;
   // grams: gram_batch follows; on the tensor cores the conv1_1 forward also takes the ReLU1_1
@@ -746,7 +750,7 @@ nst_status forward_batch(nst_ctx *ctx, const PassPlan &p, const Batch &bt, const
                                            p.Hb, p.Wb, ws.g[1], (__nv_bfloat16 *)ws.act[0],
                                            p.d_patches + pl.off, pl.n,
                                            fuse_g11 ? ctx->d_g11part : nullptr, &ctx->g11_runs,
-                                           ctx->d_err, s);
+                                           check_finite, ctx->d_err, s);
       if (e != cudaSuccess) return cuda_fail(ctx, e, "conv1_1 tensor-core forward launch");
     } else {
       launch_conv11_fwd<T>(img, p.H, p.W, ctx->h_c11, geom, bt.B, p.Hb, p.Wb, (T *)ws.act[0], s);
@@ -814,7 +818,7 @@ nst_status ensure_gram_maps(nst_ctx *ctx, PassPlan &p, const Workspace &ws) {
 
 template <typename T>
 nst_status gram_batch(nst_ctx *ctx, PassPlan &p, const Batch &bt, const Workspace &ws,
-                      cudaStream_t s, bool moments) {
+                      cudaStream_t s, bool moments, bool first) {
   const int nt = (int)p.tiles.size();
   if (moments) {
     Timer tm(ctx, kTGram, s);
@@ -833,33 +837,53 @@ nst_status gram_batch(nst_ctx *ctx, PassPlan &p, const Batch &bt, const Workspac
   if (ctx->use_tc) {
     nst_status st = ensure_gram_maps(ctx, p, ws);
     if (st) return st;
-  }
-  for (int si = 0; si < kNStyle; si++) {
-    const int l = kStyleConv[si], lv = kLevel[l];
     Timer tm(ctx, kTGram, s);
-    ctx->launches += 2;
-    if (ctx->use_tc && si == 0 && ctx->g11_runs > 0) {
-      // ReLU1_1: the conv1_1 forward took the Gram of its owned patches; reduce its partials
-      cudaError_t e = launch_gram_tc_reduce(ctx->d_g11part, ctx->g11_runs, 64, 64, 1, 1,
-                                            ctx->d_gacc + gram_offset(0), s);
-      if (e != cudaSuccess) return cuda_fail(ctx, e, "ReLU1_1 Gram reduction launch");
-      continue;
-    }
-    if (ctx->use_tc) {
+    GramReduceArgs red{};
+    red.n = kNStyle;
+    red.overwrite = first ? 1 : 0;
+    float *part = ctx->d_gpart;
+    for (int si = 0; si < kNStyle; si++) {
+      GramReduceLayer &L = red.L[si];
+      L.C = kStyleC[si];
+      L.Gacc = ctx->d_gacc + gram_offset(si);
+      if (si == 0 && ctx->g11_runs > 0) {
+        // ReLU1_1: the conv1_1 forward took the Gram of its owned patches
+        L.part = ctx->d_g11part;
+        L.nruns = ctx->g11_runs;
+        L.N = 64;
+        L.nI = L.nJ = 1;
+        continue;
+      }
       GramTcArgs a{};
       a.maps = p.d_maps + (size_t)si * nt + bt.t0;
       a.chunks = p.d_tcchunks + bt.tc_off[si];
-      a.C = kCout[l];
+      a.C = L.C;
       gram_tc_shape(a.C, &a.N, &a.nI, &a.nJ);
       a.TH = p.tc_TH[si];
       a.TW = p.tc_TW[si];
-      a.part = ctx->d_gpart;
+      a.part = part;
       a.err = ctx->d_err;
-      cudaError_t e = launch_gram_tc(a, bt.tc_runs[si], ctx->d_gacc + gram_offset(si), s);
+      L.part = part;
+      L.nruns = bt.tc_runs[si];
+      L.N = a.N;
+      L.nI = a.nI;
+      L.nJ = a.nJ;
+      part += (size_t)L.nruns * a.nI * a.nJ * 128 * a.N;
+      ctx->launches++;
+      cudaError_t e = launch_gram_tc(a, bt.tc_runs[si], s);
       if (e != cudaSuccess) return cuda_fail(ctx, e, "tensor-core Gram launch");
-      continue;
     }
+    ctx->launches++;
+    cudaError_t e = launch_gram_tc_reduce(red, s);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "Gram reduction launch");
+    return NST_OK;
+  }
+  if (first) CK(cudaMemsetAsync(ctx->d_gacc, 0, sizeof(double) * kGramTotal, s));
+  for (int si = 0; si < kNStyle; si++) {
+    const int l = kStyleConv[si], lv = kLevel[l];
     if (bt.nchunks[si] == 0) continue;
+    Timer tm(ctx, kTGram, s);
+    ctx->launches += 2;
     launch_gram_partial<T>((const T *)ws.act[l], p.Hb >> lv, p.Wb >> lv, kCout[l],
                            p.d_own + (size_t)si * nt + bt.t0, p.d_chunks + bt.chunk_off[si],
                            bt.nchunks[si], ctx->d_gpart, s);
@@ -961,7 +985,7 @@ enum PassKind { kPassStyleStats, kPassContentTarget };
 
 template <typename T>
 nst_status stats_pass(nst_ctx *ctx, const float *img, int H, int W, PassKind kind,
-                      cudaStream_t s, bool moments = false) {
+                      cudaStream_t s, bool moments = false, bool check_finite = false) {
   PassPlan *p = nullptr;
   nst_status st = build_plan(ctx, H, W, ctx->cfg.margin1, &p);
   if (st) return st;
@@ -971,10 +995,11 @@ nst_status stats_pass(nst_ctx *ctx, const float *img, int H, int W, PassKind kin
   const int nt = (int)p->tiles.size();
   for (const Batch &bt : p->batches) {
     const int last = kind == kPassContentTarget ? kContentConv : kNConv - 1;
-    st = forward_batch<T>(ctx, *p, bt, ws, img, last, false, s, kind == kPassStyleStats);
+    st = forward_batch<T>(ctx, *p, bt, ws, img, last, false, s, kind == kPassStyleStats,
+                          check_finite);
     if (st) return st;
     if (kind == kPassStyleStats) {
-      st = gram_batch<T>(ctx, *p, bt, ws, s, moments);
+      st = gram_batch<T>(ctx, *p, bt, ws, s, moments, bt.t0 == 0);
       if (st) return st;
     } else {
       ctx->launches++;
@@ -991,10 +1016,11 @@ template <typename T>
 nst_status loss_grad_impl(nst_ctx *ctx, const float *x, float *grad, double *loss,
                           cudaStream_t s) {
   const int H = ctx->H, W = ctx->W;
-  ctx->launches++;
-  launch_check_finite(x, 3LL * H * W, ctx->d_err, s);
+  if (!ctx->use_tc) {   // (the tensor-core form checks x where it stages it)
+    ctx->launches++;
+    launch_check_finite(x, 3LL * H * W, ctx->d_err, s);
+  }
   // Step 1: global statistics of x
-  CK(cudaMemsetAsync(ctx->d_gacc, 0, sizeof(double) * kGramTotal, s));
   if (ctx->aug) CK(cudaMemsetAsync(ctx->d_sacc, 0, sizeof(double) * kMomentTotal, s));
   PassPlan *p = nullptr;
   nst_status st = build_plan(ctx, H, W, ctx->cfg.margin2, &p);
@@ -1011,12 +1037,12 @@ nst_status loss_grad_impl(nst_ctx *ctx, const float *x, float *grad, double *los
   ctx->pass_batches = (int)p->batches.size();
   if (resident) {
     const Batch &bt = p->batches[0];
-    st = forward_batch<T>(ctx, *p, bt, ws, x, kNConv - 1, true, s, true);
+    st = forward_batch<T>(ctx, *p, bt, ws, x, kNConv - 1, true, s, true, true);
     if (st) return st;
-    st = gram_batch<T>(ctx, *p, bt, ws, s, ctx->aug);
+    st = gram_batch<T>(ctx, *p, bt, ws, s, ctx->aug, true);
     if (st) return st;
   } else {
-    st = stats_pass<T>(ctx, x, H, W, kPassStyleStats, s, ctx->aug);
+    st = stats_pass<T>(ctx, x, H, W, kPassStyleStats, s, ctx->aug, true);
     if (st) return st;
     st = ensure_buffers(ctx, *p, ws);   // the Step-1 plan may have moved the workspace
     if (st) return st;
@@ -1043,12 +1069,11 @@ nst_status loss_grad_impl(nst_ctx *ctx, const float *x, float *grad, double *los
   }
   fa.Eparts = ctx->d_parts;
   fa.r_is_bf16 = ctx->bf16 ? 1 : 0;
-  fa.beta = ctx->d_fin;
-  fa.partial = ctx->d_fin + kNStyle * 512;
-  ctx->launches += 3;   // moments, residuals, sums
+  fa.partial = ctx->d_fin;
+  fa.arrived = ctx->d_arrived;
+  ctx->launches++;
   launch_style_finalize(fa, s);
   // Step 2: loss and gradient block by block
-  CK(cudaMemsetAsync(ctx->d_parts + kNStyle, 0, sizeof(double), s));
   const int nt = (int)p->tiles.size();
   for (const Batch &bt : p->batches) {
     if (!resident) {
@@ -1057,18 +1082,28 @@ nst_status loss_grad_impl(nst_ctx *ctx, const float *x, float *grad, double *los
     }
     {
       Timer tm(ctx, kTOther, s);
-      ctx->launches += 2;
-      launch_content_loss<T>((const T *)ws.act[kContentConv], p->Hb >> kContentLevel,
-                             p->Wb >> kContentLevel, (const T *)ctx->d_ctgt, ctx->Hc, ctx->Wc,
-                             p->d_geom + bt.t0, p->d_own + (size_t)kOwnContent * nt + bt.t0,
-                             p->d_chunks + bt.chunk_off[kNStyle], bt.nchunks[kNStyle],
-                             ctx->d_cpart, (double)ctx->cfg.lambda_c, ctx->d_parts + kNStyle, s);
+      ctx->launches++;
+      ContentLossArgs ca{};
+      ca.V = ws.act[kContentConv];
+      ca.Vu = ctx->d_ctgt;
+      ca.Hb = p->Hb >> kContentLevel;
+      ca.Wb = p->Wb >> kContentLevel;
+      ca.Wc = ctx->Wc;
+      ca.geom = p->d_geom + bt.t0;
+      ca.own = p->d_own + (size_t)kOwnContent * nt + bt.t0;
+      ca.chunks = p->d_chunks + bt.chunk_off[kNStyle];
+      ca.nchunks = bt.nchunks[kNStyle];
+      ca.partial = ctx->d_cpart;
+      ca.arrived = ctx->d_arrived + 1;
+      ca.lambda = (double)ctx->cfg.lambda_c;
+      ca.parts = ctx->d_parts;
+      ca.first = bt.t0 == 0;
+      if (&bt == &p->batches.back()) ca.loss = loss ? loss : ctx->d_loss;
+      launch_content_loss<T>(ca, s);
     }
     st = backward_batch<T>(ctx, *p, bt, ws, grad, s);
     if (st) return st;
   }
-  ctx->launches++;
-  launch_finish_loss(ctx->d_parts, loss ? loss : ctx->d_loss, s);
   CK(cudaGetLastError());
   return NST_OK;
 }
@@ -1221,11 +1256,12 @@ nst_status nst_create(nst_ctx **out, const float *params, long long n_params,
       cudaMalloc(&ctx->d_mu, sizeof(double) * kMomentTotal) != cudaSuccess ||
       cudaMalloc(&ctx->d_sigma, sizeof(double) * kMomentTotal) != cudaSuccess ||
       cudaMalloc(&ctx->d_alpha, sizeof(float) * kMomentTotal) != cudaSuccess ||
-      cudaMalloc(&ctx->d_fin, sizeof(double) * (kNStyle * 512 + kNStyle * kFinalizeChunks)) !=
-          cudaSuccess)
+      cudaMalloc(&ctx->d_fin, sizeof(double) * kFinalizeCtas) != cudaSuccess ||
+      cudaMalloc(&ctx->d_arrived, sizeof(unsigned) * 2) != cudaSuccess)
     return bad(NST_ERR_OOM);
   for (int i = 0; i < 5; i++) ctx->aug |= cfg->w_mean[i] != 0.f || cfg->w_std[i] != 0.f;
   cudaMemset(ctx->d_err, 0, sizeof(unsigned));
+  cudaMemset(ctx->d_arrived, 0, sizeof(unsigned) * 2);
   cudaMemset(ctx->d_parts, 0, sizeof(double) * 8);
   cudaMemset(ctx->d_gx, 0, sizeof(double) * kGramTotal);
   e = cudaDeviceSynchronize();
@@ -1250,6 +1286,7 @@ nst_status nst_destroy(nst_ctx *ctx) {
   cudaFree(ctx->d_sacc); cudaFree(ctx->d_mu); cudaFree(ctx->d_sigma); cudaFree(ctx->d_alpha);
   cudaFree(ctx->d_cspart);
   cudaFree(ctx->d_fin);
+  cudaFree(ctx->d_arrived);
   for (auto &kv : ctx->plans) {
     cudaFree(kv.second.d_geom);
     cudaFree(kv.second.d_own);
@@ -1267,18 +1304,15 @@ nst_status nst_style_targets(nst_ctx *ctx, const float *v, int Hv, int Wv, void 
   nst_status st = check_img(ctx, v, Hv, Wv);
   if (st) return st;
   cudaStream_t s = (cudaStream_t)stream;
-  CK(cudaMemsetAsync(ctx->d_gacc, 0, sizeof(double) * kGramTotal, s));
   CK(cudaMemsetAsync(ctx->d_sacc, 0, sizeof(double) * kMomentTotal, s));
   st = ctx->bf16 ? stats_pass<__nv_bfloat16>(ctx, v, Hv, Wv, kPassStyleStats, s, true)
                  : stats_pass<float>(ctx, v, Hv, Wv, kPassStyleStats, s, true);
   if (st) return st;
-  // G^L(v) = sum / n_p: the finaliser with w = 0 against a zero reference
+  // G^L(v) = sum / n_p: the finaliser with w = 0 and no reference
   StyleFinalizeArgs fa{};
-  CK(cudaMemsetAsync(ctx->d_gx, 0, sizeof(double) * kGramTotal, s));
   for (int si = 0; si < kNStyle; si++) {
     const int stv = 1 << si;
     fa.L[si].Gacc = ctx->d_gacc + gram_offset(si);
-    fa.L[si].Ghat = ctx->d_gx + gram_offset(si);  // zero reference
     fa.L[si].Gout = ctx->d_ghat + gram_offset(si);
     fa.L[si].R = (char *)ctx->d_R + gram_offset(si) * ctx->esz;
     fa.L[si].C = kStyleC[si];
@@ -1291,8 +1325,8 @@ nst_status nst_style_targets(nst_ctx *ctx, const float *v, int Hv, int Wv, void 
   }
   fa.Eparts = ctx->d_parts;
   fa.r_is_bf16 = ctx->bf16 ? 1 : 0;
-  fa.beta = ctx->d_fin;
-  fa.partial = ctx->d_fin + kNStyle * 512;
+  fa.partial = ctx->d_fin;
+  fa.arrived = ctx->d_arrived;
   launch_style_finalize(fa, s);
   CK(cudaGetLastError());
   ctx->have_style = true;

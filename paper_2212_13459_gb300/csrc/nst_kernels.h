@@ -13,12 +13,13 @@ struct GramChunk {
 
 struct StyleLayerArgs {
   const double *Gacc;  // sum over owned pixels of V V^T (FP64)
-  const double *Ghat;  // G^L(v)
+  const double *Ghat;  // G^L(v), or null: zero
   double *Gout;        // G^L(x) = Gacc / np
   void *R;             // (4 w / np)(G - Ghat) + diag(beta), FP32 or BF16
   int C;
   double np;
   double w;
+  double inv_np, rs;   // 1 / np and 4 w / np (set by the launcher)
   // mean / std terms (Eq. 5), all optional: channel sums S, targets mu / sigma with weights
   // wm / ws; alpha receives the per-channel gradient offset; mean_out / std_out the moments
   const double *S;
@@ -27,13 +28,13 @@ struct StyleLayerArgs {
   float *alpha;
   double *mean_out, *std_out;
 };
-constexpr int kFinalizeChunks = 65;   // per layer: moment term + 64 residual chunks
+constexpr int kFinalizeCtas = 596;    // 1,024 elements of the five Gram matrices each
 struct StyleFinalizeArgs {
   StyleLayerArgs L[kNStyle];
   double *Eparts;   // [5]
   int r_is_bf16;
-  double *beta;     // scratch [5][512]
-  double *partial;  // scratch [5][kFinalizeChunks]
+  double *partial;    // scratch [kFinalizeCtas]
+  unsigned *arrived;  // zero between launches
 };
 
 // conv1_1 weights and biases as one kernel parameter (7,168 bytes): w[k][c] = W1[c][k] with
@@ -99,16 +100,27 @@ struct ChansumArgs {
 int chansum_split(int nchunks, int max_chunk_px);
 template <typename T>
 void launch_chansum(ChansumArgs a, cudaStream_t s);
+struct ContentLossArgs {
+  const void *V, *Vu;       // ReLU4_2 of the batch's blocks [B][Hb][Wb][512]; the target [Hc][Wc][512]
+  int Hb, Wb, Wc;
+  const BlockGeom *geom;
+  const OwnRect *own;
+  const GramChunk *chunks;
+  int nchunks;
+  double *partial;          // [max(1, nchunks)]
+  unsigned *arrived;        // zero between launches
+  double lambda;
+  double *parts;            // [6]; parts[5] is set (first) or added to
+  int first;
+  double *loss;             // the evaluation's last batch: receives the sum of the parts; else null
+};
 template <typename T>
-void launch_content_loss(const T *V, int Hb, int Wb, const T *Vu, int Hc, int Wc,
-                         const BlockGeom *geom, const OwnRect *own, const GramChunk *chunks,
-                         int nchunks, double *partial, double lambda, double *acc, cudaStream_t s);
+void launch_content_loss(const ContentLossArgs &a, cudaStream_t s);
 template <typename T>
 void launch_crop_content(const T *V, int B, int Hb, int Wb, const BlockGeom *geom,
                          const OwnRect *own, T *Vu, int Hc, int Wc, int max_own_px,
                          cudaStream_t s);
 void launch_check_finite(const float *x, long long n, unsigned *err, cudaStream_t s);
-void launch_finish_loss(const double *parts, double *loss, cudaStream_t s);
 
 // k_tc.cu: tcgen05 / TMEM / TMA implicit-GEMM convolution (BF16 in, FP32 accumulate)
 // Returns cudaSuccess or the error of tensor-map encoding / launch.
@@ -137,14 +149,15 @@ cudaError_t launch_timeout_check(long long limit_cycles, unsigned *err, cudaStre
 // the Gram sum_p V_p V_p^T over the patches with owned != 0 (each wholly inside its block's owned
 // rectangle, or past the valid extent, where V = 0) is accumulated per CTA on the tensor cores
 // and written as *gram_runs partials of 128 x 64 floats (rows 0..63 used), the layout
-// launch_gram_tc_reduce reads (C = N = 64, one tile). Input gradient:
+// launch_gram_tc_reduce reads (C = N = 64, one tile). check_finite: a NaN or infinity in the
+// blocks' pixels sets kErrNonfinite in *err. Input gradient:
 // grad[ci][ey0 + y][ex0 + x] for the owned (inner) pixels of every block, from the gated
 // ReLU1_1 gradient g [B][Hb][Wb][64].
 cudaError_t launch_conv11_fwd_tc(const float *img, int H, int W, const float *w11,
                                  const float *bias, const BlockGeom *geom, int B, int Hb, int Wb,
                                  void *stage_buf, __nv_bfloat16 *out, const int4 *patches,
-                                 int npatches, float *gram_part, int *gram_runs, unsigned *err,
-                                 cudaStream_t s);
+                                 int npatches, float *gram_part, int *gram_runs,
+                                 bool check_finite, unsigned *err, cudaStream_t s);
 cudaError_t launch_conv11_dgrad_tc(const __nv_bfloat16 *g, const float *w11,
                                    const BlockGeom *geom, const OwnRect *inner, int B, int Hb,
                                    int Wb, int max_inner_h, int max_inner_w, float *grad, int H,
@@ -165,11 +178,21 @@ void gram_tc_shape(int C, int *N, int *nI, int *nJ);
 void gram_tc_patch(int own_h, int own_w, int *TH, int *TW);
 cudaError_t encode_gram_map(CUtensorMap *m, const void *base, int C, int own_w, int own_h,
                             long long row_stride_px, int TH, int TW);
-cudaError_t launch_gram_tc(const GramTcArgs &a, int nruns, double *Gacc, cudaStream_t s);
-// Gacc[i][j] += the sum over nruns FP32 partial tiles (run r at part + r * nI * nJ * 128 * N,
-// tile (I, J) of 128 x N floats), fixed order; the reduction launch_gram_tc ends with.
-cudaError_t launch_gram_tc_reduce(const float *part, int nruns, int C, int N, int nI, int nJ,
-                                  double *Gacc, cudaStream_t s);
+cudaError_t launch_gram_tc(const GramTcArgs &a, int nruns, cudaStream_t s);
+// Gacc[i][j] (+)= the sum over nruns FP32 partial tiles (run r at part + r * nI * nJ * 128 * N,
+// tile (I, J) of 128 x N floats) of n layers, fixed order
+struct GramReduceLayer {
+  const float *part;
+  int nruns, C, N, nI, nJ;
+  double *Gacc;
+  int split, cta0;   // set by the launcher
+};
+struct GramReduceArgs {
+  GramReduceLayer L[kNStyle];
+  int n;
+  int overwrite;     // the first batch: Gacc is set, not added to
+};
+cudaError_t launch_gram_tc_reduce(GramReduceArgs a, cudaStream_t s);
 
 // Chunking of a flat [npix][C] feature matrix for the CUDA-core Gram kernels: about 1,216 CTAs
 // over the 64 x 64 block pairs (npairs = nb (nb + 1) / 2, nb = C / 64), chunks of a multiple of
