@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2)
   uint8_t *smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
   const uint32_t b_base = smem_base, a_base = smem_base + kFwdB;
   const uint32_t o_off = kFwdB + kFwdStages * kFwdStage;   // output staging tiles
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int ntiles = patches ? npatches : B * tiles_x * tiles_y;
   auto origin = [&](int t, int &b, int &y0, int &x0) {
     if (patches) {
@@ -204,33 +204,32 @@ __global__ void __launch_bounds__(kFwdThreads, 2)
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_sh;
 
+  // (the whole warp runs the issue loops, one elected lane issues: see mbar_wait_warp)
   if (warp == 0) {
-    if (lane == 0) {
-      asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmX)) : "memory");
-      int it = 0;
-      for (int t = blockIdx.x; t < ntiles; t += gridDim.x, it++) {
-        const int stage = it % kFwdStages;
-        const uint32_t phase = (uint32_t)(it / kFwdStages) & 1u;
-        int b, oy, ox;
-        origin(t, b, oy, ox);
-        if (!mbar_wait(smem_u32(&empty_bar[stage]), phase ^ 1u, &abort_flag, err)) break;
+    int stage = 0;
+    uint32_t phase = 1;
+    for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+      int b, oy, ox;
+      origin(t, b, oy, ox);
+      if (!mbar_wait_warp(smem_u32(&empty_bar[stage]), phase, &abort_flag, err)) break;
+      if (elect_one()) {
         const uint32_t fb = smem_u32(&full_bar[stage]);
         mbar_expect_tx(fb, kFwdBoxBytes);
         tma_load_4d(a_base + stage * kFwdStage, &tmX, fb, 0, ox - 1, oy - 1, b);
       }
+      __syncwarp();
+      if (++stage == kFwdStages) { stage = 0; phase ^= 1; }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      int it = 0;
-      for (int t = blockIdx.x; t < ntiles; t += gridDim.x, it++) {
-        const int stage = it % kFwdStages;
-        const uint32_t phase = (uint32_t)(it / kFwdStages) & 1u;
-        const int acc = it & 1;
-        const uint32_t use = (uint32_t)(it >> 1);
-        if (!mbar_wait(smem_u32(&tempty_bar[acc]), (use & 1u) ^ 1u, &abort_flag, err)) break;
-        tc_fence_after();
-        if (!mbar_wait(smem_u32(&full_bar[stage]), phase, &abort_flag, err)) break;
-        tc_fence_after();
+    int stage = 0, it = 0;
+    uint32_t phase = 0;
+    for (int t = blockIdx.x; t < ntiles; t += gridDim.x, it++) {
+      const int acc = it & 1;
+      const uint32_t use = (uint32_t)(it >> 1);
+      if (!mbar_wait_warp(smem_u32(&tempty_bar[acc]), (use & 1u) ^ 1u, &abort_flag, err)) break;
+      if (!mbar_wait_warp(smem_u32(&full_bar[stage]), phase, &abort_flag, err)) break;
+      tc_fence_after();
+      if (elect_one()) {
         const uint32_t sa = a_base + stage * kFwdStage;
         const uint32_t d = tmem_base + (uint32_t)(acc * 64);
 #pragma unroll
@@ -243,6 +242,8 @@ __global__ void __launch_bounds__(kFwdThreads, 2)
         mma_commit(smem_u32(&empty_bar[stage]));
         mma_commit(smem_u32(&tfull_bar[acc]));
       }
+      __syncwarp();
+      if (++stage == kFwdStages) { stage = 0; phase ^= 1; }
     }
   } else {
     // ---------------- epilogue: bias, ReLU, valid-extent mask, BF16 tile -> TMA store ----------------
@@ -401,7 +402,7 @@ __global__ void __launch_bounds__(kDgThreads, 2)
   uint8_t *smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
   const uint32_t b_base = smem_base, a_base = smem_base + kDgB;
   float *Ps = reinterpret_cast<float *>(smem_gen + kDgB + kDgStages * kDgStage);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int per_block = tiles_x * tiles_y;
   const int ntiles = B * per_block;
 
@@ -449,37 +450,34 @@ __global__ void __launch_bounds__(kDgThreads, 2)
   };
 
   if (warp == 0) {
-    if (lane == 0) {
-      asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmG)) : "memory");
-      int it = 0;
-      for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        int b, y0, x0;
-        OwnRect r;
-        if (!tile_at(t, b, y0, x0, r)) continue;
-        const int stage = it % kDgStages;
-        const uint32_t phase = (uint32_t)(it / kDgStages) & 1u;
-        if (!mbar_wait(smem_u32(&empty_bar[stage]), phase ^ 1u, &abort_flag, err)) break;
+    int stage = 0;
+    uint32_t phase = 1;
+    for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+      int b, y0, x0;
+      OwnRect r;
+      if (!tile_at(t, b, y0, x0, r)) continue;
+      if (!mbar_wait_warp(smem_u32(&empty_bar[stage]), phase, &abort_flag, err)) break;
+      if (elect_one()) {
         const uint32_t fb = smem_u32(&full_bar[stage]);
         mbar_expect_tx(fb, kDgBoxBytes);
         tma_load_4d(a_base + stage * kDgStage, &tmG, fb, 0, x0 - 1, y0 - 1, b);
-        it++;
       }
+      __syncwarp();
+      if (++stage == kDgStages) { stage = 0; phase ^= 1; }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      int it = 0;
-      for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        int b, y0, x0;
-        OwnRect r;
-        if (!tile_at(t, b, y0, x0, r)) continue;
-        const int stage = it % kDgStages;
-        const uint32_t phase = (uint32_t)(it / kDgStages) & 1u;
-        const int acc = it & 1;
-        const uint32_t use = (uint32_t)(it >> 1);
-        if (!mbar_wait(smem_u32(&tempty_bar[acc]), (use & 1u) ^ 1u, &abort_flag, err)) break;
-        tc_fence_after();
-        if (!mbar_wait(smem_u32(&full_bar[stage]), phase, &abort_flag, err)) break;
-        tc_fence_after();
+    int stage = 0, it = 0;
+    uint32_t phase = 0;
+    for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+      int b, y0, x0;
+      OwnRect r;
+      if (!tile_at(t, b, y0, x0, r)) continue;
+      const int acc = it & 1;
+      const uint32_t use = (uint32_t)(it >> 1);
+      if (!mbar_wait_warp(smem_u32(&tempty_bar[acc]), (use & 1u) ^ 1u, &abort_flag, err)) break;
+      if (!mbar_wait_warp(smem_u32(&full_bar[stage]), phase, &abort_flag, err)) break;
+      tc_fence_after();
+      if (elect_one()) {
         const uint32_t sa = a_base + stage * kDgStage;
         const uint64_t db = sw128_desc(b_base);
 #pragma unroll
@@ -492,8 +490,10 @@ __global__ void __launch_bounds__(kDgThreads, 2)
         }
         mma_commit(smem_u32(&empty_bar[stage]));
         mma_commit(smem_u32(&tfull_bar[acc]));
-        it++;
       }
+      __syncwarp();
+      if (++stage == kDgStages) { stage = 0; phase ^= 1; }
+      it++;
     }
   } else {
     // ---------------- epilogue: P -> shared memory, 9-tap gather, FP32 stores ----------------

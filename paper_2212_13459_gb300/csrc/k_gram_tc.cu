@@ -27,21 +27,21 @@ constexpr uint32_t kSlab = 64 * 128;  // one 64-pixel x 64-channel BF16 slab
 constexpr uint32_t kSmemMax = 227 * 1024;
 
 // Stages of the box ring: ALOAD (some I tile's channels lie outside the J tile, C = 512) keeps
-// room for two A slabs per stage, 4 stages; otherwise A is always read from the B slabs (or the
-// zero slab) and a stage is the B slabs alone, so more boxes are in flight (8 at N = 64, 128;
-// 6 at N = 256).
+// room for two A slabs per stage; otherwise A is always read from the B slabs (or the zero slab)
+// and a stage is the B slabs alone. Two CTAs per SM (96 KB of stages each) instead of one with
+// twice the stages: one's setup and epilogue run under the other's loads. The four launches of
+// 756 x 1008: 81 -> 74 us; 1512 x 2016: 172 -> 156 us.
 template <int N, bool ALOAD>
 struct GramCfg {
   static constexpr uint32_t A_BYTES = ALOAD ? 2 * kSlab : 0u;
   static constexpr uint32_t B_BYTES = (N / 64) * kSlab;
   static constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES;
-  static constexpr int FIT = (int)((kSmemMax - kSlab - 1024) / STAGE_BYTES);
-  static constexpr int STAGES = ALOAD ? 4 : (FIT > 8 ? 8 : FIT);
+  static constexpr int STAGES = (int)(96u * 1024u / STAGE_BYTES) > 8 ? 8 : (int)(96u * 1024u / STAGE_BYTES);
   static constexpr size_t SMEM = (size_t)STAGES * STAGE_BYTES + kSlab + 1024;
 };
 
 template <int N, bool ALOAD>
-__global__ void __launch_bounds__(kThreads, 1) gram_tc_kernel(GramTcArgs a) {
+__global__ void __launch_bounds__(kThreads, 2) gram_tc_kernel(GramTcArgs a) {
   using Cfg = GramCfg<N, ALOAD>;
   constexpr int kStages = Cfg::STAGES;
   constexpr uint32_t A_BYTES = Cfg::A_BYTES;
@@ -59,7 +59,7 @@ __global__ void __launch_bounds__(kThreads, 1) gram_tc_kernel(GramTcArgs a) {
   __shared__ volatile int abort_flag;
 
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const GramTcChunk ch = a.chunks[blockIdx.x];
   const int tile = blockIdx.y, I = tile / a.nJ, J = tile % a.nJ;
   const CUtensorMap *map = a.maps + ch.b;
@@ -98,15 +98,17 @@ __global__ void __launch_bounds__(kThreads, 1) gram_tc_kernel(GramTcArgs a) {
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_sh;
 
+  // (the whole warp runs the issue loops, one elected lane issues: see mbar_wait_warp)
   if (warp == 0) {
-    if (lane == 0) {
-      int stage = 0;
-      uint32_t phase = 0;
-      for (int k = ch.box0; k < ch.box1; k++) {
-        if (!mbar_wait(smem_u32(&empty_bar[stage]), phase ^ 1, &abort_flag, a.err)) break;
+    int stage = 0;
+    uint32_t phase = 1;
+    int bx = ch.box0 % ch.nbx, by = ch.box0 / ch.nbx;
+    for (int k = ch.box0; k < ch.box1; k++) {
+      if (!mbar_wait_warp(smem_u32(&empty_bar[stage]), phase, &abort_flag, a.err)) break;
+      if (elect_one()) {
         const uint32_t fb = smem_u32(&full_bar[stage]);
         const uint32_t sa = smem_base + stage * STAGE_BYTES, sb = sa + A_BYTES;
-        const int x = (k % ch.nbx) * a.TW, y = (k / ch.nbx) * a.TH;
+        const int x = bx * a.TW, y = by * a.TH;
         mbar_expect_tx(fb, tx_bytes);
         if (ALOAD && a_load) {
           tma_load_4d(sa, map, fb, I * 128, x, y, 0);
@@ -114,20 +116,22 @@ __global__ void __launch_bounds__(kThreads, 1) gram_tc_kernel(GramTcArgs a) {
         }
 #pragma unroll
         for (int j = 0; j < N / 64; j++) tma_load_4d(sb + j * kSlab, map, fb, J * N + j * 64, x, y, 0);
-        if (++stage == kStages) { stage = 0; phase ^= 1; }
       }
+      __syncwarp();
+      if (++bx == ch.nbx) { bx = 0; by++; }
+      if (++stage == kStages) { stage = 0; phase ^= 1; }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      int stage = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      for (int k = ch.box0; k < ch.box1; k++) {
-        if (!mbar_wait(smem_u32(&full_bar[stage]), phase, &abort_flag, a.err)) {
-          ok = false;
-          break;
-        }
-        tc_fence_after();
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    for (int k = ch.box0; k < ch.box1; k++) {
+      if (!mbar_wait_warp(smem_u32(&full_bar[stage]), phase, &abort_flag, a.err)) {
+        ok = false;
+        break;
+      }
+      tc_fence_after();
+      if (elect_one()) {
         const uint32_t sa = smem_base + stage * STAGE_BYTES, sb = sa + A_BYTES;
         // A's two 64-channel atoms: its own slabs, B slabs, or the zero slab (after every stage,
         // so the atom distance, the descriptor's leading byte offset, stays positive)
@@ -144,10 +148,12 @@ __global__ void __launch_bounds__(kThreads, 1) gram_tc_kernel(GramTcArgs a) {
                    sw128_desc_mn(sb + kk * 2048, kSlab), IDESC,
                    (k > ch.box0 || kk > 0) ? 1u : 0u);
         mma_commit(smem_u32(&empty_bar[stage]));
-        if (++stage == kStages) { stage = 0; phase ^= 1; }
       }
-      if (ok) mma_commit(smem_u32(&done_bar));
+      __syncwarp();
+      if (++stage == kStages) { stage = 0; phase ^= 1; }
     }
+    if (ok && elect_one()) mma_commit(smem_u32(&done_bar));
+    __syncwarp();
   } else {
     const int q = warp & 3;
     const int row = q * 32 + lane;   // channel I * 128 + row
