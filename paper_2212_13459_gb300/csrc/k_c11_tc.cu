@@ -50,6 +50,7 @@ __global__ void __launch_bounds__(256) conv11_stage_kernel(const float *__restri
                                                            int B, int Hb, int Wb,
                                                            uint4 *__restrict__ xs,
                                                            unsigned *__restrict__ err) {
+  pdl_begin();
   bool bad = false;
   const int npix = B * Hb * Wb;
   const size_t plane = (size_t)H * W;
@@ -203,6 +204,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_sh;
+  pdl_begin();
 
   // (the whole warp runs the issue loops, one elected lane issues: see mbar_wait_warp)
   if (warp == 0) {
@@ -437,6 +439,7 @@ __global__ void __launch_bounds__(kDgThreads, 2)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_sh;
+  pdl_begin();
 
   // tile t -> block b, patch origin (y0, x0) in block-local level-0 coordinates; tiles past the
   // block's owned rectangle are skipped identically by every role
@@ -586,9 +589,9 @@ cudaError_t launch_conv11_fwd_tc(const float *img, int H, int W, const float *w1
   if (npix <= 0) return cudaSuccess;
   if (reinterpret_cast<uintptr_t>(stage_buf) % 16) return cudaErrorInvalidValue;
   const int sgrid = (int)std::min<long long>((npix + 255) / 256, 32LL * tc_num_sms());
-  conv11_stage_kernel<<<sgrid, 256, 0, s>>>(img, H, W, geom, B, Hb, Wb,
-                                            reinterpret_cast<uint4 *>(stage_buf),
-                                            check_finite ? err : nullptr);
+  cudaError_t le = launch_pdl(npix * 28e-6 / 5 <= kEarlyUs, conv11_stage_kernel, sgrid, 256, 0, s, img, H, W, geom, B, Hb, Wb,
+                              reinterpret_cast<uint4 *>(stage_buf), check_finite ? err : nullptr);
+  if (le != cudaSuccess) return le;
   EncodeTiledFn enc = reinterpret_cast<EncodeTiledFn>(tc_encode_tiled_fn());
   if (!enc) return cudaErrorNotSupported;
   CUtensorMap m;
@@ -615,11 +618,10 @@ cudaError_t launch_conv11_fwd_tc(const float *img, int H, int W, const float *w1
   // list puts them first), a split that depends on the owned patches alone
   const int grid = gram_part ? 2 * tc_num_sms()
                              : (int)std::min<long long>(ntiles, 2LL * tc_num_sms());
-  conv11_fwd_tc_kernel<<<grid, kFwdThreads, kFwdSmem, s>>>(m, mo, w11, bias, geom, B, Hb, Wb,
-                                                           tiles_x, tiles_y, patches,
-                                                           (int)ntiles, gram_part, err);
+  le = launch_pdl(ntiles * (128 * 144e-6 / 5) <= kEarlyUs, conv11_fwd_tc_kernel, grid, kFwdThreads, kFwdSmem, s, m, mo, w11, bias, geom, B, Hb,
+                  Wb, tiles_x, tiles_y, patches, (int)ntiles, gram_part, err);
   if (gram_runs) *gram_runs = gram_part ? grid : 0;
-  return cudaGetLastError();
+  return le;
 }
 
 cudaError_t launch_conv11_dgrad_tc(const __nv_bfloat16 *g, const float *w11,
@@ -650,9 +652,8 @@ cudaError_t launch_conv11_dgrad_tc(const __nv_bfloat16 *g, const float *w11,
   const int tiles_y = (max_inner_h + kDgOutH - 1) / kDgOutH;
   const long long ntiles = (long long)B * tiles_x * tiles_y;
   const int grid = (int)std::min<long long>(ntiles, 2LL * tc_num_sms());
-  conv11_dgrad_tc_kernel<<<grid, kDgThreads, kDgSmem, s>>>(m, w11, geom, inner, B, tiles_x,
-                                                           tiles_y, grad, H, W, err);
-  return cudaGetLastError();
+  return launch_pdl(ntiles * (192 * 140e-6 / 5) <= kEarlyUs, conv11_dgrad_tc_kernel, grid, kDgThreads, kDgSmem, s, m, w11, geom, inner, B, tiles_x,
+                    tiles_y, grad, H, W, err);
 }
 
 }  // namespace nst

@@ -97,6 +97,7 @@ __global__ void __launch_bounds__(kThreads, 2) gram_tc_kernel(GramTcArgs a) {
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_sh;
+  pdl_begin();
 
   // (the whole warp runs the issue loops, one elected lane issues: see mbar_wait_warp)
   if (warp == 0) {
@@ -214,6 +215,7 @@ __global__ void __launch_bounds__(kRedWarps * 32) gram_tc_reduce_kernel(GramRedu
   const int sub = warp % L.split, grp = warp / L.split;
   const int e = (((int)blockIdx.x - L.cta0) * (kRedWarps / L.split) + grp) * 128 + lane * 4;
   const bool live = e < L.C * L.C;
+  pdl_begin();
   float s[4] = {0.f, 0.f, 0.f, 0.f}, c[4] = {0.f, 0.f, 0.f, 0.f};
   if (live) {
     const int i = e / L.C, j = e % L.C;
@@ -268,8 +270,7 @@ cudaError_t launch_n(const GramTcArgs &a, int nruns, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  gram_tc_kernel<N, ALOAD><<<dim3(nruns, a.nI * a.nJ), kThreads, smem, s>>>(a);
-  return cudaGetLastError();
+  return launch_pdl(true, gram_tc_kernel<N, ALOAD>, dim3(nruns, a.nI * a.nJ), kThreads, smem, s, a);
 }
 
 // whether some (I, J) tile reads A slabs of its own: an I-tile slab below C that lies outside
@@ -345,8 +346,7 @@ cudaError_t launch_gram_tc_reduce(GramReduceArgs a, cudaStream_t s) {
     ctas += (L.C * L.C + per - 1) / per;
   }
   if (ctas <= 0) return cudaSuccess;
-  gram_tc_reduce_kernel<<<ctas, kRedWarps * 32, 0, s>>>(a);
-  return cudaGetLastError();
+  return launch_pdl(true, gram_tc_reduce_kernel, ctas, kRedWarps * 32, 0, s, a);
 }
 
 }  // namespace nst

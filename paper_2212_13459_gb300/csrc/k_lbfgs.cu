@@ -89,6 +89,7 @@ __global__ void __launch_bounds__(kDotThreads) lbfgs_dots_kernel(
   __shared__ long long sp_off;
   __shared__ Sum red[kDotThreads / 32][4 * G];
   const int grp = blockIdx.x, nb = gridDim.y, cta = blockIdx.y;
+  pdl_begin();
   if (threadIdx.x == 0) {
     const int count = c->count;
     int nj = 0;
@@ -214,8 +215,8 @@ void launch_lbfgs_dots(const float *g, const float *g_prev, const float *S, floa
   const long long need = ((vec ? n / 4 : n) + kDotThreads - 1) / kDotThreads;
   const int nb = (int)(need < 1 ? 1 : need < dot_blocks(m) ? need : dot_blocks(m));
   dim3 grid(first ? 1 : dot_groups(m), nb);
-  lbfgs_dots_kernel<<<grid, kDotThreads, 0, s>>>(g, g_prev, S, Y, stride, n, c, first, vec,
-                                                 partials);
+  launch_pdl(true, lbfgs_dots_kernel, grid, kDotThreads, 0, s, g, g_prev, S, Y, stride, n, c, first, vec,
+             partials);
 }
 
 // The small solve: curvature test, bookkeeping, the two triangular systems and the coefficients
@@ -241,6 +242,7 @@ __global__ void __launch_bounds__(kSolveThreads) lbfgs_solve_kernel(LbfgsCtl *c,
   __shared__ double wpart[kSolveParts][kMaxHistory];
   __shared__ int sl[kMaxHistory], old[kMaxHistory];
   const int tid = threadIdx.x, lane = tid & 31;
+  pdl_begin();
   if (first) {
     if (tid == 0) {
       const double l1 = c->dots[0];
@@ -399,8 +401,7 @@ cudaError_t launch_lbfgs_solve(LbfgsCtl *c, int m, int first, double eps, double
         lbfgs_solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)solve_smem(kMaxHistory));
     if (e != cudaSuccess) return e;
   }
-  lbfgs_solve_kernel<<<1, kSolveThreads, smem, s>>>(c, m, first, eps, SY, YY);
-  return cudaSuccess;
+  return launch_pdl(true, lbfgs_solve_kernel, 1, kSolveThreads, smem, s, c, m, first, eps, SY, YY);
 }
 
 __global__ void __launch_bounds__(256) lbfgs_combine_kernel(
@@ -408,6 +409,7 @@ __global__ void __launch_bounds__(256) lbfgs_combine_kernel(
     float *__restrict__ g_prev, const float *__restrict__ g, long long n,
     const LbfgsCtl *__restrict__ c, int vec) {
   constexpr int U = 8;   // stored pairs whose loads are issued together
+  pdl_begin();
   __shared__ float cS[kMaxHistory], cY[kMaxHistory];
   __shared__ long long off[kMaxHistory];
   __shared__ float cg_sh;
@@ -475,7 +477,7 @@ void launch_lbfgs_combine(float *x, float *S, const float *Y, long long stride, 
                   aligned16(g) && stride % 4 == 0;
   long long b = (n / 4 + 255) / 256;
   const int grid = (int)(b < 152 * 8 ? (b > 0 ? b : 1) : 152 * 8);
-  lbfgs_combine_kernel<<<grid, 256, 0, s>>>(x, S, Y, stride, g_prev, g, n, c, vec);
+  launch_pdl(true, lbfgs_combine_kernel, grid, 256, 0, s, x, S, Y, stride, g_prev, g, n, c, vec);
 }
 
 // ---- bicubic resampling ---------------------------------------------------------------------------

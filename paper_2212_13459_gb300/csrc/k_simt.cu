@@ -613,6 +613,7 @@ __global__ void unpool_idx_kernel(const __nv_bfloat16 *__restrict__ gp,
                                   __nv_bfloat16 *__restrict__ g, int B, int Hp, int Wp, int C,
                                   const BlockGeom *__restrict__ geom, int level_out,
                                   const int4 *__restrict__ rects) {
+  pdl_begin();
   const int C8 = C / 8;
   int4 r = make_int4(0, Hp, 0, Wp);
   long long n = (long long)B * Hp * Wp * C8;
@@ -687,12 +688,11 @@ void launch_unpool_idx(const __nv_bfloat16 *gp, const unsigned char *idx, __nv_b
     const long long per = (long long)max_rect_px * C / 8;
     int nx = (int)std::min<long long>((per + 255) / 256, std::max(1, 152 * 32 / B));
     dim3 grid(nx, B);
-    unpool_idx_kernel<<<grid, 256, 0, s>>>(gp, idx, g, B, Hp, Wp, C, geom, level_out, rects);
+    launch_pdl(per * B * 84e-6 / 5 <= kEarlyUs, unpool_idx_kernel, grid, 256, 0, s, gp, idx, g, B, Hp, Wp, C, geom, level_out, rects);
     return;
   }
-  unpool_idx_kernel<<<ew_grid((long long)B * Hp * Wp * C / 8), 256, 0, s>>>(gp, idx, g, B, Hp, Wp,
-                                                                            C, geom, level_out,
-                                                                            nullptr);
+  launch_pdl(true, unpool_idx_kernel, ew_grid((long long)B * Hp * Wp * C / 8), 256, 0, s, gp, idx, g, B, Hp,
+             Wp, C, geom, level_out, (const int4 *)nullptr);
 }
 template void launch_pool<float>(const float *, float *, int, int, int, int, const BlockGeom *,
                                  int, cudaStream_t);
@@ -851,6 +851,7 @@ __global__ void __launch_bounds__(kFinThreads) style_finalize_kernel(StyleFinali
   const double inv = L.inv_np, rs = L.rs;
   double s = 0.0, g[4], h[4];
   const int e0 = b * kFinPer + tid;
+  pdl_begin();
 #pragma unroll
   for (int k = 0; k < 4; k++) {
     g[k] = L.Gacc[e0 + k * kFinThreads];
@@ -920,7 +921,7 @@ void launch_style_finalize(const StyleFinalizeArgs &a, cudaStream_t s) {
     b.L[l].inv_np = 1.0 / a.L[l].np;   // (two FP64 divisions per thread are half the kernel)
     b.L[l].rs = 4.0 * a.L[l].w / a.L[l].np;
   }
-  style_finalize_kernel<<<n / kFinPer, kFinThreads, 0, s>>>(b);
+  launch_pdl(true, style_finalize_kernel, n / kFinPer, kFinThreads, 0, s, b);
 }
 
 // ---- channel sums over owned pixels, all style layers in one launch -------------------------------
@@ -934,6 +935,7 @@ constexpr int kChansumThreads = 256, kChansumRun = 64;
 template <typename T>
 __global__ void __launch_bounds__(kChansumThreads) chansum_partial_kernel(ChansumArgs a) {
   __shared__ double red[kChansumThreads * 8];   // [lane group][C]
+  pdl_begin();
   int l = 0;
   while (l + 1 < kNStyle && (int)blockIdx.x >= a.L[l + 1].cta0) l++;
   const ChansumLayer L = a.L[l];
@@ -999,6 +1001,7 @@ __global__ void __launch_bounds__(kChansumThreads) chansum_partial_kernel(Chansu
 constexpr int kChansumWarps = 16;
 __global__ void __launch_bounds__(32 * kChansumWarps) chansum_reduce_kernel(ChansumArgs a) {
   __shared__ double red[kChansumWarps][32];
+  pdl_begin();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int l = 0, b = blockIdx.x;
   while (b >= a.L[l].C / 32) b -= a.L[l++].C / 32;
@@ -1040,8 +1043,8 @@ void launch_chansum(ChansumArgs a, cudaStream_t s) {
     rctas += a.L[l].C / 32;
   }
   if (ctas <= 0) return;
-  chansum_partial_kernel<T><<<ctas, kChansumThreads, 0, s>>>(a);
-  chansum_reduce_kernel<<<rctas, 32 * kChansumWarps, 0, s>>>(a);
+  launch_pdl(true, chansum_partial_kernel<T>, ctas, kChansumThreads, 0, s, a);
+  launch_pdl(true, chansum_reduce_kernel, rctas, 32 * kChansumWarps, 0, s, a);
 }
 template void launch_chansum<float>(ChansumArgs, cudaStream_t);
 template void launch_chansum<__nv_bfloat16>(ChansumArgs, cudaStream_t);
@@ -1062,6 +1065,7 @@ __global__ void __launch_bounds__(256) content_loss_kernel(ContentLossArgs a) {
     }
   };
   double s = 0.0;
+  pdl_begin();
   if ((int)blockIdx.x < a.nchunks) {
     const GramChunk ch = a.chunks[blockIdx.x];
     const OwnRect r = a.own[ch.b];
@@ -1115,7 +1119,7 @@ __global__ void __launch_bounds__(256) content_loss_kernel(ContentLossArgs a) {
 
 template <typename T>
 void launch_content_loss(const ContentLossArgs &a, cudaStream_t s) {
-  content_loss_kernel<T><<<a.nchunks > 0 ? a.nchunks : 1, 256, 0, s>>>(a);
+  launch_pdl(true, content_loss_kernel<T>, a.nchunks > 0 ? a.nchunks : 1, 256, 0, s, a);
 }
 template void launch_content_loss<float>(const ContentLossArgs &, cudaStream_t);
 template void launch_content_loss<__nv_bfloat16>(const ContentLossArgs &, cudaStream_t);

@@ -466,6 +466,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_sh;
+  pdl_begin();
   const int kb_total = tg.kb_main + tg.kb2;
 
   if (warp == 0) {
@@ -693,6 +694,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_sh;
+  pdl_begin();
 
   if (warp == 0) {
     if (elect_one()) {
@@ -954,6 +956,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_sh;
+  pdl_begin();
   const int kb_total = tg.kb_main + tg.kb2;
 
   if (warp == 0) {
@@ -1144,6 +1147,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_sh;
+  pdl_begin();
 
   if (warp == 0) {
     // ---------------- TMA producer: one box per tile, one weight tile per tap ----------------
@@ -1357,8 +1361,10 @@ cudaError_t launch_bn(const CUtensorMap &A, const CUtensorMap &B, const CUtensor
     attr_set = true;
   }
   const int grid = std::min(tg.total, g_num_sms);
-  conv_tc_kernel<BN, STAGES><<<grid, kThreads, smem, s>>>(A, B, A2, B2, Bp, B2p, a, tg);
-  return cudaGetLastError();
+  // (us of a 64-deep K-block of one tile, see the costs where the tiles are split)
+  const double us = (BN == 256 ? 0.33 : BN == 128 ? 0.19 : 0.155) * (tg.kb_main + tg.kb2) *
+                    ((tg.total + g_num_sms - 1) / g_num_sms);
+  return launch_pdl(us <= kEarlyUs, conv_tc_kernel<BN, STAGES>, grid, kThreads, smem, s, A, B, A2, B2, Bp, B2p, a, tg);
 }
 
 template <int STAGES>
@@ -1375,8 +1381,8 @@ cudaError_t launch_swap(const CUtensorMap &A, const CUtensorMap &B, const CUtens
     attr_set = true;
   }
   const int grid = std::min(tg.total, g_num_sms);
-  conv_tc_swap_kernel<STAGES><<<grid, kThreads, smem, s>>>(A, B, A2, B2, a, tg);
-  return cudaGetLastError();
+  const double us = 0.4 * (tg.kb_main + tg.kb2) * ((tg.total + g_num_sms - 1) / g_num_sms);
+  return launch_pdl(us <= kEarlyUs, conv_tc_swap_kernel<STAGES>, grid, kThreads, smem, s, A, B, A2, B2, a, tg);
 }
 
 // Output patch of at most `rows` pixels (the tile's M or N) covering n rectangles h[i] x w[i]
@@ -1436,9 +1442,9 @@ cudaError_t launch_halo(const CUtensorMap &A, const CUtensorMap &B, const CUtens
   if (tg.total <= 0) return cudaSuccess;
   int grid = std::min(tg.total * NT, g_num_sms);
   grid = std::max(NT, grid / NT * NT);
-  conv_tc_halo_kernel<BN, KB, P2KB, NT, MASK_SMEM><<<grid, kThreads, smem, s>>>(A, B, A2, B2, a,
-                                                                             tg);
-  return cudaGetLastError();
+  const double us = 1.25 * KB * ((tg.total + g_num_sms - 1) / g_num_sms);
+  return launch_pdl(us <= kEarlyUs, conv_tc_halo_kernel<BN, KB, P2KB, NT, MASK_SMEM>, grid, kThreads, smem, s, A, B,
+                    A2, B2, a, tg);
 }
 
 // 4-D map of an activation with the halo box (64 ch, 10 px, 18 rows, 1)
@@ -1493,8 +1499,8 @@ cudaError_t launch_swap_halo(const ConvArgs &a, cudaStream_t s) {
   tg.total = a.tiles ? a.n_mtiles : a.B * tg.tiles_x * tg.tiles_y;
   if (tg.total <= 0) return cudaSuccess;
   const int grid = std::min(tg.total, g_num_sms);
-  conv_tc_swap_halo_kernel<<<grid, kThreads, kSHSmem, s>>>(mA, mW, a, tg);
-  return cudaGetLastError();
+  const double us = 3.6 * ((tg.total + g_num_sms - 1) / g_num_sms);
+  return launch_pdl(us <= kEarlyUs, conv_tc_swap_halo_kernel, grid, kThreads, kSHSmem, s, mA, mW, a, tg);
 }
 
 // (cin, cout, k2) of the narrow layers -> N slice width and counts; false if not a halo layer
