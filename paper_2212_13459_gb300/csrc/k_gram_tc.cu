@@ -39,9 +39,15 @@ struct GramCfg {
   static constexpr int STAGES = (int)(96u * 1024u / STAGE_BYTES) > 8 ? 8 : (int)(96u * 1024u / STAGE_BYTES);
   static constexpr size_t SMEM = (size_t)STAGES * STAGE_BYTES + kSlab + 1024;
 };
+constexpr int kGramMaxStages = 8;
+constexpr size_t kGramSmem = 96 * 1024 + kSlab + 1024;
+static_assert(GramCfg<64, false>::SMEM <= kGramSmem && GramCfg<128, false>::SMEM <= kGramSmem &&
+              GramCfg<256, false>::SMEM <= kGramSmem && GramCfg<256, true>::SMEM <= kGramSmem &&
+              GramCfg<64, false>::STAGES <= kGramMaxStages, "Gram kernel shared memory");
 
+// One CTA's work: tile `tile` over run `run` of layer a
 template <int N, bool ALOAD>
-__global__ void __launch_bounds__(kThreads, 2) gram_tc_kernel(GramTcArgs a) {
+__device__ __forceinline__ void gram_tc_body(const GramTcArgs &a, int run, int tile) {
   using Cfg = GramCfg<N, ALOAD>;
   constexpr int kStages = Cfg::STAGES;
   constexpr uint32_t A_BYTES = Cfg::A_BYTES;
@@ -54,14 +60,15 @@ __global__ void __launch_bounds__(kThreads, 2) gram_tc_kernel(GramTcArgs a) {
                              ((uint32_t)(N >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
 
   extern __shared__ uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t full_bar[kStages], empty_bar[kStages], done_bar;
+  // (shared by the kernel's variants: declared for the most stages)
+  __shared__ __align__(8) uint64_t full_bar[kGramMaxStages], empty_bar[kGramMaxStages], done_bar;
   __shared__ uint32_t tmem_base_sh;
   __shared__ volatile int abort_flag;
 
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const int warp = warp_index(), lane = threadIdx.x & 31;
-  const GramTcChunk ch = a.chunks[blockIdx.x];
-  const int tile = blockIdx.y, I = tile / a.nJ, J = tile % a.nJ;
+  const GramTcChunk ch = a.chunks[run];
+  const int I = tile / a.nJ, J = tile % a.nJ;
   const CUtensorMap *map = a.maps + ch.b;
   // A slab s (channels I*128 + 64 s ..) is B slab (I*128 + 64 s - J*N) / 64 when it lies inside
   // the J tile, zeros when it lies past C, else loaded
@@ -163,7 +170,7 @@ __global__ void __launch_bounds__(kThreads, 2) gram_tc_kernel(GramTcArgs a) {
     if (lane == 0) ready = mbar_wait(smem_u32(&done_bar), 0, &abort_flag, a.err);
     if (__shfl_sync(0xffffffffu, ready, 0)) {
       tc_fence_after();
-      float *out = a.part + (((size_t)blockIdx.x * a.nI * a.nJ + tile) * 128 + row) * N;
+      float *out = a.part + (((size_t)run * a.nI * a.nJ + tile) * 128 + row) * N;
       const bool live = I * 128 + row < a.C;
 #pragma unroll 1
       for (int c = 0; c < N; c += 32) {
@@ -182,6 +189,26 @@ __global__ void __launch_bounds__(kThreads, 2) gram_tc_kernel(GramTcArgs a) {
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem_base, TMEM_COLS);
+  }
+}
+
+// The Grams of several layers in one launch (they are independent, and alone none fills the chip to
+// its end: 756 x 1008, four launches 74 us, one 59; 64 x 64, 36 us, 10). CTA c of layer l
+// takes run c / tiles, tile c % tiles.
+__global__ void __launch_bounds__(kThreads, 2) gram_tc_kernel(GramTcBatch g) {
+  int l = 0;
+  while (l + 1 < g.n && (int)blockIdx.x >= g.L[l + 1].cta0) l++;
+  const GramTcArgs &a = g.L[l];
+  const int c = (int)blockIdx.x - a.cta0, tiles = a.nI * a.nJ;
+  const int run = c / tiles, tile = c % tiles;
+  switch (a.N) {
+    case 64: gram_tc_body<64, false>(a, run, tile); break;
+    case 128: gram_tc_body<128, false>(a, run, tile); break;
+    default:
+      if (a.aload)
+        gram_tc_body<256, true>(a, run, tile);
+      else
+        gram_tc_body<256, false>(a, run, tile);
   }
 }
 
@@ -259,20 +286,6 @@ __global__ void __launch_bounds__(kRedWarps * 32) gram_tc_reduce_kernel(GramRedu
   }
 }
 
-template <int N, bool ALOAD>
-cudaError_t launch_n(const GramTcArgs &a, int nruns, cudaStream_t s) {
-  constexpr size_t smem = GramCfg<N, ALOAD>::SMEM;
-  static_assert(smem <= kSmemMax, "Gram kernel shared memory");
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(gram_tc_kernel<N, ALOAD>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
-  return launch_pdl(true, gram_tc_kernel<N, ALOAD>, dim3(nruns, a.nI * a.nJ), kThreads, smem, s, a);
-}
-
 // whether some (I, J) tile reads A slabs of its own: an I-tile slab below C that lies outside
 // the J tile (the same test the kernel makes per tile)
 bool gram_needs_aload(const GramTcArgs &a) {
@@ -324,15 +337,26 @@ cudaError_t encode_gram_map(CUtensorMap *m, const void *base, int C, int own_w, 
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-cudaError_t launch_gram_tc(const GramTcArgs &a, int nruns, cudaStream_t s) {
-  if (nruns <= 0) return cudaSuccess;
-  const bool aload = gram_needs_aload(a);
-  switch (a.N) {
-    case 64: return aload ? launch_n<64, true>(a, nruns, s) : launch_n<64, false>(a, nruns, s);
-    case 128: return aload ? launch_n<128, true>(a, nruns, s) : launch_n<128, false>(a, nruns, s);
-    case 256: return aload ? launch_n<256, true>(a, nruns, s) : launch_n<256, false>(a, nruns, s);
-    default: return cudaErrorInvalidValue;
+cudaError_t launch_gram_tc(GramTcBatch g, cudaStream_t s) {
+  int ctas = 0;
+  for (int l = 0; l < g.n; l++) {
+    GramTcArgs &a = g.L[l];
+    if (a.N != 64 && a.N != 128 && a.N != 256) return cudaErrorInvalidValue;
+    a.aload = gram_needs_aload(a) ? 1 : 0;
+    if (a.aload && a.N != 256) return cudaErrorInvalidValue;
+    a.cta0 = ctas;
+    ctas += a.nruns * a.nI * a.nJ;
   }
+  if (ctas <= 0) return cudaSuccess;
+  constexpr size_t smem = kGramSmem;
+  static bool attr = false;
+  if (!attr) {
+    cudaError_t e = cudaFuncSetAttribute(gram_tc_kernel,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    attr = true;
+  }
+  return launch_pdl(true, gram_tc_kernel, ctas, kThreads, smem, s, g);
 }
 
 cudaError_t launch_gram_tc_reduce(GramReduceArgs a, cudaStream_t s) {

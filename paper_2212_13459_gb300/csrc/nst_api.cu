@@ -841,6 +841,7 @@ nst_status gram_batch(nst_ctx *ctx, PassPlan &p, const Batch &bt, const Workspac
     GramReduceArgs red{};
     red.n = kNStyle;
     red.overwrite = first ? 1 : 0;
+    GramTcBatch gb{};
     float *part = ctx->d_gpart;
     for (int si = 0; si < kNStyle; si++) {
       GramReduceLayer &L = red.L[si];
@@ -854,7 +855,7 @@ nst_status gram_batch(nst_ctx *ctx, PassPlan &p, const Batch &bt, const Workspac
         L.nI = L.nJ = 1;
         continue;
       }
-      GramTcArgs a{};
+      GramTcArgs &a = gb.L[gb.n++];
       a.maps = p.d_maps + (size_t)si * nt + bt.t0;
       a.chunks = p.d_tcchunks + bt.tc_off[si];
       a.C = L.C;
@@ -869,12 +870,12 @@ nst_status gram_batch(nst_ctx *ctx, PassPlan &p, const Batch &bt, const Workspac
       L.nI = a.nI;
       L.nJ = a.nJ;
       part += (size_t)L.nruns * a.nI * a.nJ * 128 * a.N;
-      ctx->launches++;
-      cudaError_t e = launch_gram_tc(a, bt.tc_runs[si], s);
-      if (e != cudaSuccess) return cuda_fail(ctx, e, "tensor-core Gram launch");
+      a.nruns = bt.tc_runs[si];
     }
-    ctx->launches++;
-    cudaError_t e = launch_gram_tc_reduce(red, s);
+    ctx->launches += 2;
+    cudaError_t e = launch_gram_tc(gb, s);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "tensor-core Gram launch");
+    e = launch_gram_tc_reduce(red, s);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "Gram reduction launch");
     return NST_OK;
   }

@@ -173,12 +173,18 @@ struct GramTcArgs {
   int C, N, nI, nJ, TH, TW;   // channels, J-tile width, tile counts, box shape (TH * TW = 64)
   float *part;                // [runs][nI * nJ][128][N] FP32 partial tiles
   unsigned *err;
+  int nruns;
+  int cta0, aload;            // set by the launcher
+};
+struct GramTcBatch {
+  GramTcArgs L[kNStyle];
+  int n;
 };
 void gram_tc_shape(int C, int *N, int *nI, int *nJ);
 void gram_tc_patch(int own_h, int own_w, int *TH, int *TW);
 cudaError_t encode_gram_map(CUtensorMap *m, const void *base, int C, int own_w, int own_h,
                             long long row_stride_px, int TH, int TW);
-cudaError_t launch_gram_tc(const GramTcArgs &a, int nruns, cudaStream_t s);
+cudaError_t launch_gram_tc(GramTcBatch g, cudaStream_t s);
 // Gacc[i][j] (+)= the sum over nruns FP32 partial tiles (run r at part + r * nI * nJ * 128 * N,
 // tile (I, J) of 128 x N floats) of n layers, fixed order
 struct GramReduceLayer {
