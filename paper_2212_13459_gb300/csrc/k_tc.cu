@@ -428,7 +428,9 @@ __device__ __forceinline__ void tile_of(const TcGeom &tg, int t, int &mt, int &n
   n0 = (t % tg.n_tiles) * BN + part * nn;
 }
 
-template <int BN, int STAGES>
+// KPS: K-blocks per pipeline stage (two for the narrow tiles, whose MMAs are shorter than a
+// stage's bookkeeping)
+template <int BN, int STAGES, int KPS>
 __global__ void __launch_bounds__(kThreads, 1)
     conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                    const __grid_constant__ CUtensorMap tmA2,
@@ -437,7 +439,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                    const __grid_constant__ CUtensorMap tmB2p, const ConvArgs a, const TcGeom tg) {
   constexpr uint32_t A_BYTES = 128 * kBK * 2;
   constexpr uint32_t B_BYTES = BN * kBK * 2;
-  constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES;
+  constexpr uint32_t KB_BYTES = A_BYTES + B_BYTES, STAGE_BYTES = KPS * KB_BYTES;
   constexpr uint32_t TMEM_COLS = 2 * BN;
 
   extern __shared__ uint8_t smem_raw[];
@@ -481,26 +483,32 @@ __global__ void __launch_bounds__(kThreads, 1)
       const uint32_t tx = (uint32_t)(tg.TH * tg.TW + nn) * (kBK * 2);
       const CUtensorMap *wB = nn == BN ? &tmB : &tmBp, *wB2 = nn == BN ? &tmB2 : &tmB2p;
       KWalk w;
-      for (int kb = 0; kb < kb_total; kb++) {
+      for (int kb = 0; kb < kb_total; kb += KPS) {
         if (!mbar_wait_warp(smem_u32(&empty_bar[stage]), phase, &abort_flag, a.err)) {
           ok = false;
           break;
         }
         if (elect_one()) {
           const uint32_t fb = smem_u32(&full_bar[stage]);
-          const uint32_t sa = smem_base + stage * STAGE_BYTES, sb = sa + A_BYTES;
-          mbar_expect_tx(fb, tx);
-          if (kb < tg.kb_main) {
-            tma_load_4d(sa, &tmA, fb, w.c, x0 + w.dx, y0 + w.dy, b);
-            tma_load_2d(sb, wB, fb, w.k, n0);
-          } else {
-            const int c = (kb - tg.kb_main) * kBK;
-            tma_load_4d(sa, &tmA2, fb, c, x0, y0, b);
-            tma_load_2d(sb, wB2, fb, c, n0);
+          mbar_expect_tx(fb, KPS > 1 && kb + KPS > kb_total ? tx * (kb_total - kb) : tx * KPS);
+          KWalk v = w;
+#pragma unroll
+          for (int j = 0; j < KPS; j++) {
+            const uint32_t sa = smem_base + stage * STAGE_BYTES + j * KB_BYTES, sb = sa + A_BYTES;
+            if (kb + j < tg.kb_main) {
+              tma_load_4d(sa, &tmA, fb, v.c, x0 + v.dx, y0 + v.dy, b);
+              tma_load_2d(sb, wB, fb, v.k, n0);
+            } else if (KPS == 1 || kb + j < kb_total) {
+              const int c = (kb + j - tg.kb_main) * kBK;
+              tma_load_4d(sa, &tmA2, fb, c, x0, y0, b);
+              tma_load_2d(sb, wB2, fb, c, n0);
+            }
+            if (j + 1 < KPS) v.next(a.cin);
           }
         }
         __syncwarp();
-        w.next(a.cin);
+#pragma unroll
+        for (int j = 0; j < KPS; j++) w.next(a.cin);
         if (++stage == STAGES) { stage = 0; phase ^= 1; }
       }
     }
@@ -519,7 +527,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       int mt, n0, nn;
       tile_of<BN>(tg, t, mt, n0, nn);
       const uint32_t idesc = make_idesc(nn);
-      for (int kb = 0; kb < kb_total; kb++) {
+      for (int kb = 0; kb < kb_total; kb += KPS) {
         if (!mbar_wait_warp(smem_u32(&full_bar[stage]), phase, &abort_flag, a.err)) {
           ok = false;
           break;
@@ -527,12 +535,17 @@ __global__ void __launch_bounds__(kThreads, 1)
         tc_fence_after();
         if (elect_one()) {
           // descriptors: the first stage's plus a multiple of the stage size (16-byte units)
-          const uint64_t da = da0 + (uint64_t)(stage * (int)(STAGE_BYTES >> 4));
-          const uint64_t db = da + (A_BYTES >> 4);
 #pragma unroll
-          for (int k = 0; k < kBK / 16; k++)
-            mma_bf16(d, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), idesc,
-                     (kb > 0 || k > 0) ? 1u : 0u);
+          for (int j = 0; j < KPS; j++) {
+            if (j > 0 && kb + j >= kb_total) break;
+            const uint64_t da =
+                da0 + (uint64_t)(stage * (int)(STAGE_BYTES >> 4) + j * (int)(KB_BYTES >> 4));
+            const uint64_t db = da + (A_BYTES >> 4);
+#pragma unroll
+            for (int k = 0; k < kBK / 16; k++)
+              mma_bf16(d, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), idesc,
+                       (kb > 0 || j > 0 || k > 0) ? 1u : 0u);
+          }
           mma_commit(smem_u32(&empty_bar[stage]));
         }
         __syncwarp();
@@ -1347,15 +1360,15 @@ cudaError_t encode_wt(CUtensorMap *m, const void *ptr, int N, int K, int BN) {
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-template <int BN, int STAGES>
+template <int BN, int STAGES, int KPS>
 cudaError_t launch_bn(const CUtensorMap &A, const CUtensorMap &B, const CUtensorMap &A2,
                       const CUtensorMap &B2, const CUtensorMap &Bp, const CUtensorMap &B2p,
                       const ConvArgs &a, const TcGeom &tg, cudaStream_t s) {
-  constexpr size_t smem = (size_t)STAGES * (128 * kBK * 2 + BN * kBK * 2) + 8 * kTileT + 1024;
+  constexpr size_t smem = (size_t)STAGES * KPS * (128 * kBK * 2 + BN * kBK * 2) + 8 * kTileT + 1024;
   static_assert(smem <= 227 * 1024, "tcgen05 convolution shared memory");
   static bool attr_set = false;
   if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(conv_tc_kernel<BN, STAGES>,
+    cudaError_t e = cudaFuncSetAttribute(conv_tc_kernel<BN, STAGES, KPS>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     attr_set = true;
@@ -1364,7 +1377,7 @@ cudaError_t launch_bn(const CUtensorMap &A, const CUtensorMap &B, const CUtensor
   // (us of a 64-deep K-block of one tile, see the costs where the tiles are split)
   const double us = (BN == 256 ? 0.33 : BN == 128 ? 0.19 : 0.155) * (tg.kb_main + tg.kb2) *
                     ((tg.total + g_num_sms - 1) / g_num_sms);
-  return launch_pdl(us <= kEarlyUs, conv_tc_kernel<BN, STAGES>, grid, kThreads, smem, s, A, B, A2, B2, Bp, B2p, a, tg);
+  return launch_pdl(us <= kEarlyUs, conv_tc_kernel<BN, STAGES, KPS>, grid, kThreads, smem, s, A, B, A2, B2, Bp, B2p, a, tg);
 }
 
 template <int STAGES>
@@ -1589,6 +1602,15 @@ void conv_tc_patch_rule(int cin, int cout, int taps, int k2, bool pool, int *row
   }
 }
 
+bool conv_tc_main128(long long m256, long long m128) {
+  // a wave of 128-pixel tiles on the main kernel takes about 0.6 of a wave of 256-pixel tiles on
+  // the pixels-as-N kernel: 128 -> 128 channels at 4 x 32 x 32 16.4 -> 11.8 us (16 and 32 tiles),
+  // 256 -> 128 at 189 x 252 31.5 -> 28.8 us (2 and 3 waves); at 378 x 504, 128 -> 128, 42 and 50 us
+  // (5 and 10 waves)
+  const long long sms = tc_num_sms();
+  return sms > 0 && 6 * ((m128 + sms - 1) / sms) < 10 * ((m256 + sms - 1) / sms);
+}
+
 void conv_tc_pick_patch(const int *h, const int *w, int n, int rows, int fixed_th, int fixed_tw,
                         bool pool, int *TH, int *TW) {
   if (fixed_th) {
@@ -1610,8 +1632,18 @@ cudaError_t launch_conv_tc(const ConvArgs &a, cudaStream_t s) {
     if (a.tiles && (a.TH != kHaloTH || a.TW != kHaloTW)) return cudaErrorInvalidValue;
     return launch_conv_tc_halo(a, hBN, hKB, hP2, hNT, s);
   }
-  // 128 output channels: pixels as the MMA's N (256 wide) instead of channels (128 wide)
-  const bool swap = a.cout == kSwapBN;
+  // 128 output channels: pixels as the MMA's N (256 wide) instead of channels (128 wide), but for
+  // small launches (see conv_tc_main128)
+  bool swap = a.cout == kSwapBN && a.rows != 128;
+  if (swap && !a.tiles) {
+    int th, tw;
+    auto count = [&](int rows) {
+      pick_patch_rows(a.Hb, a.Wb, rows, th, tw, a.pool_out != nullptr);
+      return (long long)a.B * ((a.Hb + th - 1) / th) * ((a.Wb + tw - 1) / tw);
+    };
+    const long long m256 = count(kSwapBP);
+    swap = !conv_tc_main128(m256, count(128));
+  }
   int BN = swap ? kSwapBN : (a.cout >= 256 ? 256 : a.cout);
   const int rows = swap ? kSwapBP : 128;
   TcGeom tg;
@@ -1634,6 +1666,12 @@ cudaError_t launch_conv_tc(const ConvArgs &a, cudaStream_t s) {
   if (tg.total <= 0) return cudaSuccess;
   tg.full = tg.total;
   tg.split = 1;
+  if (BN == 128 && !swap && 2 * tg.total <= g_num_sms) {
+    // below half a wave: 64-channel tiles
+    BN = 64;
+    tg.n_tiles = a.cout / BN;
+    tg.total = tg.full = m_tiles * tg.n_tiles;
+  }
   if (BN == 256) {
     // The last, partly filled wave of 256-channel tiles runs as 128- or 64-channel parts (the
     // same sums in the same order) where that ends earlier. Time of a tile: 256 : 128 : 64
@@ -1685,9 +1723,9 @@ cudaError_t launch_conv_tc(const ConvArgs &a, cudaStream_t s) {
   }
   if (swap) return launch_swap<4>(mA, mB, mA2, mB2, a, tg, s);
   switch (BN) {
-    case 64: return launch_bn<64, 8>(mA, mB, mA2, mB2, mBp, mB2p, a, tg, s);
-    case 128: return launch_bn<128, 6>(mA, mB, mA2, mB2, mBp, mB2p, a, tg, s);
-    case 256: return launch_bn<256, 4>(mA, mB, mA2, mB2, mBp, mB2p, a, tg, s);
+    case 64: return launch_bn<64, 4, 2>(mA, mB, mA2, mB2, mBp, mB2p, a, tg, s);
+    case 128: return launch_bn<128, 3, 2>(mA, mB, mA2, mB2, mBp, mB2p, a, tg, s);
+    case 256: return launch_bn<256, 4, 1>(mA, mB, mA2, mB2, mBp, mB2p, a, tg, s);
     default: return cudaErrorInvalidValue;
   }
 }

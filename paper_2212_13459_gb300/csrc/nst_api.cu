@@ -111,6 +111,7 @@ constexpr int kOwnContent = 5, kOwnInner = 6;
 // table, TH x TW patches.
 struct PatchList {
   int off, n, TH, TW;
+  int rows = 0;   // ConvArgs::rows
 };
 // The passes whose convolutions are restricted to what the owned pixels need (see needed_axis):
 // Step-1 statistics (also the style targets), the content target, the Step-2 forward.
@@ -521,7 +522,7 @@ nst_status build_plan(nst_ctx *ctx, int H, int W, int margin, PassPlan **out) {
   std::vector<int4> patches;
   auto add_list = [&](const Batch &bt, int level, int cin, int cout, int taps, int k2, bool pool,
                       auto pick) -> PatchList {
-    PatchList pl{(int)patches.size(), 0, 0, 0};
+    PatchList pl{(int)patches.size(), 0, 0, 0, 0};
     std::vector<Iv> ry(bt.B), rx(bt.B);
     std::vector<int> hs(bt.B), wsz(bt.B);
     for (int j = 0; j < bt.B; j++) {
@@ -550,7 +551,20 @@ nst_status build_plan(nst_ctx *ctx, int H, int W, int margin, PassPlan **out) {
     }
     int rows, fth, ftw;
     conv_tc_patch_rule(cin, cout, taps, k2, pool, &rows, &fth, &ftw);
-    conv_tc_pick_patch(hs.data(), wsz.data(), bt.B, rows, fth, ftw, pool, &pl.TH, &pl.TW);
+    auto tiles = [&](int r) {
+      conv_tc_pick_patch(hs.data(), wsz.data(), bt.B, r, fth, ftw, pool, &pl.TH, &pl.TW);
+      long long m = 0;
+      for (int j = 0; j < bt.B; j++)
+        m += (long long)((hs[j] + pl.TH - 1) / pl.TH) * ((wsz[j] + pl.TW - 1) / pl.TW);
+      return m;
+    };
+    const long long m = tiles(rows);
+    if (cout == 128 && rows == 256 && !fth) {
+      if (conv_tc_main128(m, tiles(128)))
+        pl.rows = 128;
+      else
+        tiles(256);
+    }
     for (int j = 0; j < bt.B; j++)
       for (int y = ry[j].a; y < ry[j].b; y += pl.TH)
         for (int x = rx[j].a; x < rx[j].b; x += pl.TW) patches.push_back(make_int4(j, y, x, 0));
@@ -561,7 +575,7 @@ nst_status build_plan(nst_ctx *ctx, int H, int W, int margin, PassPlan **out) {
     for (int k = 0; k < kFwdKinds; k++) {
       // conv1_1 (its own kernel, 16 x 8 patches)
       PatchList &c11 = bt.fwd[k][0];
-      c11 = PatchList{(int)patches.size(), 0, 16, 8};
+      c11 = PatchList{(int)patches.size(), 0, 16, 8, 0};
       // Passes that take the Grams (Step 1, the style targets, the resident pass): the patch
       // grid sits on multiples of 16 x 8 px of the block buffer, as do the owned rectangle's
       // edges (block bounds and margins are multiples of 16 px; at the image edge the owned
@@ -617,7 +631,7 @@ nst_status build_plan(nst_ctx *ctx, int H, int W, int margin, PassPlan **out) {
       if (!kPoolAfter[l]) continue;
       const int lv = kLevel[l] + 1;
       PatchList &pl = bt.unpool[l];
-      pl = PatchList{(int)patches.size(), bt.B, 0, 0};
+      pl = PatchList{(int)patches.size(), bt.B, 0, 0, 0};
       for (int j = 0; j < bt.B; j++) {
         const Tile &t = p.tiles[bt.t0 + j];
         const Iv ry = local_rect(ny[bt.t0 + j].D[l + 1], t.ey0 >> lv, (t.ey1 - t.ey0) >> lv,
@@ -707,6 +721,7 @@ void use_patches(ConvArgs &a, const PassPlan &p, const PatchList &pl) {
   a.n_mtiles = pl.n;
   a.TH = pl.TH;
   a.TW = pl.TW;
+  a.rows = pl.rows;
 }
 
 nst_status run_conv(nst_ctx *ctx, ConvArgs a, cudaStream_t s) {

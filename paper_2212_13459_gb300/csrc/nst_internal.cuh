@@ -121,6 +121,7 @@ struct ConvArgs {
   // CUDA-core engine: runs of TH pixels of rectangles (see launch_conv_simt), TW = the CTA tile
   const int4 *tiles;
   int n_mtiles, TH, TW;
+  int rows;   // tensor-core engine, 128 output channels: 128 = the patches are for the main kernel
 };
 
 }  // namespace nst

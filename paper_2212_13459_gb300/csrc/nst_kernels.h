@@ -131,6 +131,9 @@ cudaError_t launch_conv_tc(const ConvArgs &a, cudaStream_t s);
 // pixels (128; 256 for the pixels-as-N kernel of 128-channel outputs). pool: fused pooling.
 void conv_tc_patch_rule(int cin, int cout, int taps, int k2, bool pool, int *rows, int *fixed_th,
                         int *fixed_tw);
+// Whether a launch with 128 output channels and the 256-row rule, m256 patches of 256 pixels or m128
+// of 128, is quicker on the main kernel (128 rows, ConvArgs::rows = 128).
+bool conv_tc_main128(long long m256, long long m128);
 // The patch shape within that rule that covers n rectangles h[i] x w[i] with the fewest
 // patches (with fused pooling TW is 8 or 16 and TH * TW = rows).
 void conv_tc_pick_patch(const int *h, const int *w, int n, int rows, int fixed_th, int fixed_tw,
