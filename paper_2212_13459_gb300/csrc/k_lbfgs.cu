@@ -47,6 +47,9 @@ int lbfgs_partials_count(int m) { return 4 * (m + 1) * dot_blocks(m); }
 // 2.29 M elements: 594 -> 345 us (5.4 TB/s); 10 pairs of 36.6 M: 634 us (5.8 TB/s).
 struct Sum {   // s + c: the sum with the rounding errors of its additions (Knuth's TwoSum)
   float s, c;
+  __device__ __forceinline__ double value() const {   // (c says nothing beside an infinite s)
+    return fabsf(s) <= FLT_MAX ? (double)s + (double)c : (double)s;
+  }
   __device__ __forceinline__ void add(float x) {
     const float t = s + x, z = t - s;
     c += (s - (t - z)) + (x - z);
@@ -58,6 +61,11 @@ struct Sum {   // s + c: the sum with the rounding errors of its additions (Knut
   }
 };
 
+// The chunks are added scaled by 2^-32 (exact): a sum of any number of them stays within FP32's
+// range where each does.
+constexpr float kDotDown = 0x1p-32f;
+constexpr double kDotUp = 0x1p32;
+
 template <int G>
 struct DotAcc {
   Sum acc[4 * G];
@@ -68,7 +76,7 @@ struct DotAcc {
   }
   __device__ __forceinline__ void flush() {
 #pragma unroll
-    for (int d = 0; d < 4 * G; d++) acc[d].add(part[d]), part[d] = 0.f;
+    for (int d = 0; d < 4 * G; d++) acc[d].add(part[d] * kDotDown), part[d] = 0.f;
   }
   __device__ __forceinline__ void add(int j, float sv, float wv, float gv, float yv) {
     part[4 * j] = fmaf(sv, gv, part[4 * j]);
@@ -184,7 +192,7 @@ __global__ void __launch_bounds__(kDotThreads) lbfgs_dots_kernel(
   if (threadIdx.x < 4 * nj) {   // the warps in index order
     Sum v = red[0][threadIdx.x];
     for (int w = 1; w < kDotThreads / 32; w++) v.merge(red[w][threadIdx.x].s, red[w][threadIdx.x].c);
-    partials[(size_t)(grp * G * 4 + threadIdx.x) * nb + cta] = (double)v.s + (double)v.c;
+    partials[(size_t)(grp * G * 4 + threadIdx.x) * nb + cta] = v.value() * kDotUp;
     __threadfence();
   }
   __syncthreads();
