@@ -903,7 +903,8 @@ nst_status gram_batch(nst_ctx *ctx, PassPlan &p, const Batch &bt, const Workspac
     launch_gram_partial<T>((const T *)ws.act[l], p.Hb >> lv, p.Wb >> lv, kCout[l],
                            p.d_own + (size_t)si * nt + bt.t0, p.d_chunks + bt.chunk_off[si],
                            bt.nchunks[si], ctx->d_gpart, s);
-    launch_gram_reduce(ctx->d_gpart, bt.nchunks[si], kCout[l], ctx->d_gacc + gram_offset(si), s);
+    launch_gram_reduce(ctx->d_gpart, bt.nchunks[si], kCout[l], ctx->d_gacc + gram_offset(si),
+                       false, s);
   }
   return NST_OK;
 }
@@ -1564,13 +1565,12 @@ nst_status nst_gram(int dtype, const void *V, long long npix, int C, double *G, 
   const int nb = C / 64, npairs = nb * (nb + 1) / 2;
   float *part = nullptr;
   CK(cudaMallocAsync((void **)&part, (size_t)nchunks * npairs * 4096 * sizeof(float), s));
-  CK(cudaMemsetAsync(G, 0, sizeof(double) * C * C, s));
   if (dtype == NST_PREC_BF16)
     launch_gram_partial_flat<__nv_bfloat16>((const __nv_bfloat16 *)V, npix, C, chunk_len, nchunks,
                                             part, s);
   else
     launch_gram_partial_flat<float>((const float *)V, npix, C, chunk_len, nchunks, part, s);
-  launch_gram_reduce(part, nchunks, C, G, s);
+  launch_gram_reduce(part, nchunks, C, G, true, s);
   CK(cudaFreeAsync(part, s));
   CK(cudaGetLastError());
   return NST_OK;

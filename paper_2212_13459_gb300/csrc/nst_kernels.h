@@ -81,7 +81,8 @@ void launch_gram_partial(const T *V, int Hb, int Wb, int C, const OwnRect *own,
 template <typename T>
 void launch_gram_partial_flat(const T *V, long long npix, int C, long long chunk_len, int nchunks,
                               float *part, cudaStream_t s);
-void launch_gram_reduce(const float *part, int nchunks, int C, double *Gacc, cudaStream_t s);
+void launch_gram_reduce(const float *part, int nchunks, int C, double *Gacc, bool overwrite,
+                        cudaStream_t s);
 void launch_style_finalize(const StyleFinalizeArgs &a, cudaStream_t s);
 // channel sums of the style layers' owned pixels: S[j] += sum over the chunks of V[p][j]
 struct ChansumLayer {

@@ -113,15 +113,13 @@ extern "C" nst_status nst_gram_noalloc(int dtype, const void *V, long long npix,
   e = scratch_for_current_device(&part, why);
   if (e != cudaSuccess) return cuda_fail(e, why);
   cudaStream_t s = (cudaStream_t)stream;
-  // the partial kernel overwrites every block it uses; only the output accumulates
-  e = cudaMemsetAsync(G, 0, sizeof(double) * C * C, s);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
+  // the kernels overwrite every partial block they use and the whole output
   if (dtype == NST_PREC_BF16)
     nst::launch_gram_partial_flat<__nv_bfloat16>((const __nv_bfloat16 *)V, npix, C, chunk,
                                                  nchunks, part, s);
   else
     nst::launch_gram_partial_flat<float>((const float *)V, npix, C, chunk, nchunks, part, s);
-  nst::launch_gram_reduce(part, nchunks, C, G, s);
+  nst::launch_gram_reduce(part, nchunks, C, G, true, s);
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
   return NST_OK;
