@@ -45,7 +45,7 @@ __device__ __forceinline__ uint32_t sw128_chunk(int r, int c) {
 // xs[b][y][x] = (hi_0, hi_1, hi_2, lo_0, lo_1, lo_2, 0, 0) inside the block's valid extent, zero
 // elsewhere (the block is a standalone image with zero padding). err (optional): a non-finite
 // image value is latched there (every image pixel is some block's).
-__global__ void __launch_bounds__(256) conv11_stage_kernel(const float *__restrict__ img, int H,
+__global__ void __launch_bounds__(256) conv11_stage_kernel(const float *img, int H,
                                                            int W, const BlockGeom *__restrict__ geom,
                                                            int B, int Hb, int Wb,
                                                            uint4 *__restrict__ xs,
@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(256) conv11_stage_kernel(const float *__restri
       float hi[3], lo[3];
 #pragma unroll
       for (int ci = 0; ci < 3; ci++) {
-        const float v = __ldg(img + ci * plane + off);
+        const float v = img[ci * plane + off];
         bad |= !isfinite(v);
         hi[ci] = __bfloat162float(__float2bfloat16_rn(v));
         lo[ci] = v - hi[ci];   // exact in FP32; rounded to BF16 by the packing below

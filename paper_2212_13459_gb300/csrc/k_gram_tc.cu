@@ -253,7 +253,7 @@ __global__ void __launch_bounds__(kRedWarps * 32) gram_tc_reduce_kernel(GramRedu
 #pragma unroll
       for (int u = 0; u < 8; u++)
         if (r0 + L.split * u < L.nruns)
-          v[u] = __ldg(reinterpret_cast<const float4 *>(L.part + (size_t)(r0 + L.split * u) * stride + off));
+          v[u] = *reinterpret_cast<const float4 *>(L.part + (size_t)(r0 + L.split * u) * stride + off);
 #pragma unroll
       for (int u = 0; u < 8; u++)
         if (r0 + L.split * u < L.nruns) {

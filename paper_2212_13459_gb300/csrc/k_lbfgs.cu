@@ -87,8 +87,8 @@ struct DotAcc {
 };
 
 __global__ void __launch_bounds__(kDotThreads) lbfgs_dots_kernel(
-    const float *__restrict__ g, const float *__restrict__ g_prev, const float *__restrict__ S,
-    float *__restrict__ Y, long long stride, long long n, LbfgsCtl *c, int first, int vec,
+    const float *g, const float *g_prev, const float *S, float *Y, long long stride, long long n,
+    LbfgsCtl *c, int first, int vec,
     double *partials) {
   constexpr int G = kLbGroup;
   static_assert(4 * G == 16, "the warp reduce-scatter below takes 16 dots");
@@ -130,7 +130,6 @@ __global__ void __launch_bounds__(kDotThreads) lbfgs_dots_kernel(
     } else {
       const float4 gp = reinterpret_cast<const float4 *>(g_prev)[v];
       const float4 yv = make_float4(gv.x - gp.x, gv.y - gp.y, gv.z - gp.z, gv.w - gp.w);
-      if (own_y) reinterpret_cast<float4 *>(ynew)[v] = yv;
       float4 sv[G], wv[G];
 #pragma unroll
       for (int j = 0; j < G; j++) {
@@ -139,6 +138,7 @@ __global__ void __launch_bounds__(kDotThreads) lbfgs_dots_kernel(
           wv[j] = (own_y && j == 0) ? yv : reinterpret_cast<const float4 *>(Y + off[j])[v];
         }
       }
+      if (own_y) reinterpret_cast<float4 *>(ynew)[v] = yv;   // (after the loads are issued)
 #pragma unroll
       for (int j = 0; j < G; j++) {
         if (j < nj) {
@@ -413,9 +413,8 @@ cudaError_t launch_lbfgs_solve(LbfgsCtl *c, int m, int first, double eps, double
 }
 
 __global__ void __launch_bounds__(256) lbfgs_combine_kernel(
-    float *__restrict__ x, float *__restrict__ S, const float *__restrict__ Y, long long stride,
-    float *__restrict__ g_prev, const float *__restrict__ g, long long n,
-    const LbfgsCtl *__restrict__ c, int vec) {
+    float *x, float *S, const float *Y, long long stride, float *g_prev, const float *g, long long n,
+    const LbfgsCtl *c, int vec) {
   constexpr int U = 8;   // stored pairs whose loads are issued together
   pdl_begin();
   __shared__ float cS[kMaxHistory], cY[kMaxHistory];
@@ -442,6 +441,7 @@ __global__ void __launch_bounds__(256) lbfgs_combine_kernel(
   const long long n4 = vec ? n / 4 : 0;
   for (long long v = t0; v < n4; v += tstride) {
     const float4 gv = reinterpret_cast<const float4 *>(g)[v];
+    float4 xv = reinterpret_cast<float4 *>(x)[v];
     float4 d = make_float4(cg * gv.x, cg * gv.y, cg * gv.z, cg * gv.w);
     for (int j0 = 0; j0 < k; j0 += U) {
       float4 sv[U], yv[U];
@@ -464,7 +464,6 @@ __global__ void __launch_bounds__(256) lbfgs_combine_kernel(
       }
     }
     reinterpret_cast<float4 *>(snew)[v] = d;
-    float4 xv = reinterpret_cast<float4 *>(x)[v];
     xv.x += d.x; xv.y += d.y; xv.z += d.z; xv.w += d.w;
     reinterpret_cast<float4 *>(x)[v] = xv;
     reinterpret_cast<float4 *>(g_prev)[v] = gv;

@@ -610,9 +610,8 @@ __global__ void unpool_kernel(const T *__restrict__ gp, const T *__restrict__ ac
 // rects (optional): per block, the pooled rectangle {y0, y1, x0, x1} to route (the rest of the
 // block's full-resolution gradient is left as it is); grid (n, B), row b = block b. Without
 // rects: every pooled position of the buffer, grid-stride over all blocks.
-__global__ void unpool_idx_kernel(const __nv_bfloat16 *__restrict__ gp,
-                                  const unsigned char *__restrict__ idx,
-                                  __nv_bfloat16 *__restrict__ g, int B, int Hp, int Wp, int C,
+__global__ void unpool_idx_kernel(const __nv_bfloat16 *gp, const unsigned char *idx,
+                                  __nv_bfloat16 *g, int B, int Hp, int Wp, int C,
                                   const BlockGeom *__restrict__ geom, int level_out,
                                   const int4 *__restrict__ rects) {
   pdl_begin();

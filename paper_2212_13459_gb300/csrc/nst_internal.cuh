@@ -21,7 +21,9 @@ namespace nst {
 // before its first access to memory that another kernel of the stream writes or reads (weights,
 // patch lists and block geometry are written once, synchronously, and may be read before). It
 // waits until the predecessor has completed with its writes visible, so completion stays
-// transitive along the stream, and then lets the successor's CTAs start.
+// transitive along the stream, and then lets the successor's CTAs start. What the stream writes is
+// read through plain pointers there, not const __restrict__ ones or __ldg: those loads are taken
+// to be of memory that does not change while the kernel runs, and may be moved ahead of the wait.
 __device__ __forceinline__ void pdl_begin() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
