@@ -20,6 +20,7 @@ struct nst_lbfgs {
   double *SY = nullptr, *YY = nullptr;   // [m+1][m+1] s_a . y_b and y_a . y_b by slot
   double *partials = nullptr;
   LbfgsCtl *ctl = nullptr;
+  void *mem = nullptr;               // the one device allocation that holds all of the above
 };
 
 namespace {
@@ -42,34 +43,42 @@ nst_status nst_lbfgs_create_ex(nst_lbfgs **out, long long n, int m, int flags) {
   st->stride = (n + 63) / 64 * 64;
   const size_t slots = (size_t)(m + 1);
   const size_t hist = slots * st->stride * sizeof(float);
-  bool ok = true;
-  if (flags & NST_LBFGS_HOST_HISTORY) {
+  // One device allocation (six took most of a small run's time). Nothing but the control block
+  // needs a value: a slot, a kept gradient and an entry of S^T Y or Y^T Y are written before they
+  // are read.
+  const bool host = (flags & NST_LBFGS_HOST_HISTORY) != 0;
+  size_t bytes = 0;
+  auto take = [&](size_t n_bytes) {
+    const size_t at = bytes;
+    bytes += (n_bytes + 255) / 256 * 256;
+    return at;
+  };
+  const size_t o_ctl = take(sizeof(LbfgsCtl)), o_sy = take(slots * slots * sizeof(double)),
+               o_yy = take(slots * slots * sizeof(double)),
+               o_part = take(lbfgs_partials_count(m) * sizeof(double)),
+               o_g = take(n * sizeof(float)), o_s = take(host ? 0 : hist), o_y = take(host ? 0 : hist);
+  bool ok = cudaMalloc(&st->mem, bytes) == cudaSuccess;
+  if (ok) {
+    char *p = static_cast<char *>(st->mem);
+    st->ctl = reinterpret_cast<LbfgsCtl *>(p + o_ctl);
+    st->SY = reinterpret_cast<double *>(p + o_sy);
+    st->YY = reinterpret_cast<double *>(p + o_yy);
+    st->partials = reinterpret_cast<double *>(p + o_part);
+    st->g_prev = reinterpret_cast<float *>(p + o_g);
+    st->S = reinterpret_cast<float *>(p + o_s);
+    st->Y = reinterpret_cast<float *>(p + o_y);
+  }
+  if (ok && host)
     ok = cudaHostAlloc(&st->S_host, hist, cudaHostAllocMapped | cudaHostAllocPortable) ==
              cudaSuccess &&
          cudaHostAlloc(&st->Y_host, hist, cudaHostAllocMapped | cudaHostAllocPortable) ==
              cudaSuccess &&
          cudaHostGetDevicePointer(&st->S, st->S_host, 0) == cudaSuccess &&
          cudaHostGetDevicePointer(&st->Y, st->Y_host, 0) == cudaSuccess;
-    if (ok) {
-      std::memset(st->S_host, 0, hist);
-      std::memset(st->Y_host, 0, hist);
-    }
-  } else {
-    ok = cudaMalloc(&st->S, hist) == cudaSuccess && cudaMalloc(&st->Y, hist) == cudaSuccess;
-    if (ok) ok = cudaMemset(st->S, 0, hist) == cudaSuccess && cudaMemset(st->Y, 0, hist) == cudaSuccess;
-  }
-  ok = ok &&
-            cudaMalloc(&st->g_prev, n * sizeof(float)) == cudaSuccess &&
-            cudaMalloc(&st->SY, slots * slots * sizeof(double)) == cudaSuccess &&
-            cudaMalloc(&st->YY, slots * slots * sizeof(double)) == cudaSuccess &&
-            cudaMalloc(&st->partials, lbfgs_partials_count(m) * sizeof(double)) == cudaSuccess &&
-            cudaMalloc(&st->ctl, sizeof(LbfgsCtl)) == cudaSuccess;
   if (!ok) {
     nst_lbfgs_destroy(st);
     return NST_ERR_OOM;
   }
-  cudaMemset(st->SY, 0, slots * slots * sizeof(double));
-  cudaMemset(st->YY, 0, slots * slots * sizeof(double));
   LbfgsCtl c;
   std::memset(&c, 0, sizeof(c));
   c.gamma = 1.0;
@@ -88,15 +97,9 @@ nst_status nst_lbfgs_create_ex(nst_lbfgs **out, long long n, int m, int flags) {
 nst_status nst_lbfgs_destroy(nst_lbfgs *st) {
   if (!st) return NST_OK;
   cudaDeviceSynchronize();
-  if (st->S_host) {
-    cudaFreeHost(st->S_host);
-    cudaFreeHost(st->Y_host);
-  } else {
-    cudaFree(st->S);
-    cudaFree(st->Y);
-  }
-  cudaFree(st->g_prev);
-  cudaFree(st->SY); cudaFree(st->YY); cudaFree(st->partials); cudaFree(st->ctl);
+  if (st->S_host) cudaFreeHost(st->S_host);
+  if (st->Y_host) cudaFreeHost(st->Y_host);
+  cudaFree(st->mem);
   delete st;
   return NST_OK;
 }
