@@ -84,7 +84,11 @@ __global__ void __launch_bounds__(256) conv11_stage_kernel(const float *img, int
 // 160-byte steps (SBO) and the two taps of one K = 16 instruction are two core matrices of the
 // same box whose distance is the instruction's LBO. Five instructions per tile: taps (0,1),
 // (2,3), (4,5), (6,7), (8, -) with zero weights in the last one's second half.
-constexpr int kFwdThreads = 192;   // warp 0 TMA, warp 1 MMA + TMEM, warps 2-5 epilogue
+// warp 0 TMA, warp 1 MMA + TMEM, warps 2-9 epilogue (two per TMEM lane quarter, 32 channels each:
+// with four, 16 per SM draining 64 channels each, the epilogue set the pace; 32.4 M pixels 860 ->
+// 826 us)
+constexpr int kFwdEpi = 256;
+constexpr int kFwdThreads = 64 + kFwdEpi;
 constexpr int kFwdStages = 6;
 constexpr int kFwdTH = 16, kFwdTW = 8, kFwdBoxH = kFwdTH + 2, kFwdBoxW = kFwdTW + 2;
 constexpr uint32_t kFwdBoxBytes = kFwdBoxH * kFwdBoxW * 16;   // 2,880
@@ -162,7 +166,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2)
     }
     for (int i = 0; i < 2; i++) {
       mbar_init(smem_u32(&tfull_bar[i]), 1);
-      mbar_init(smem_u32(&tempty_bar[i]), 128);
+      mbar_init(smem_u32(&tempty_bar[i]), kFwdEpi);
     }
     for (int i = 0; i < kFwdOutBufs; i++) mbar_init(smem_u32(&gram_bar[i]), 1);
     mbar_init(smem_u32(&gram_done), 1);
@@ -249,12 +253,12 @@ __global__ void __launch_bounds__(kFwdThreads, 2)
     }
   } else {
     // ---------------- epilogue: bias, ReLU, valid-extent mask, BF16 tile -> TMA store ----------------
-    // Each thread writes its pixel's 128-byte row into a 128-byte-swizzled staging tile (chunk c
-    // of row r at c ^ (r & 7): conflict-free), and one thread stores the 16 x 8 x 64 tile with
+    // Each thread writes half of its pixel's 128-byte row into a 128-byte-swizzled staging tile
+    // (chunk c of row r at c ^ (r & 7): conflict-free), and one thread stores the 16 x 8 x 64 tile with
     // one TMA copy (full-line writes; rows / columns past the buffer are clipped). Four staging
     // tiles rotate (several stores in flight); a tile is rewritten only after its store has
     // finished reading it.
-    const int q = warp & 3;
+    const int q = warp & 3, half = (warp - 2) >> 2;   // lane quarter, channels 32 half ..
     const int row = q * 32 + lane;   // patch pixel (row / 8, row % 8)
     const int et = threadIdx.x - 64;
     // thread et = 0 issues the stores, et = 32 (the next warp) the fused Gram MMAs; per staging
@@ -267,7 +271,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2)
       const int acc = it & 1;
       const uint32_t use = (uint32_t)(it >> 1);
       const int ob = it % kFwdOutBufs;
-      // one thread waits (bounded) and broadcasts, so all 128 threads leave the loop together;
+      // one thread waits (bounded) and broadcasts, so all epilogue threads leave the loop together;
       // the same barrier tells everyone that staging tile ob is free again (its store has read
       // it, see below, and so have the Gram MMAs of its last tile)
       if (et == 0) epi_ok = mbar_wait_sleep(smem_u32(&tfull_bar[acc]), use & 1u, &abort_flag, err);
@@ -279,14 +283,12 @@ __global__ void __launch_bounds__(kFwdThreads, 2)
           gpend &= ~(1u << ob);
         }
       }
-      named_bar_sync(1, 128);
+      named_bar_sync(1, kFwdEpi);
       if (!gram_ok) break;
       if (!epi_ok) break;
       tc_fence_after();
-      float v[64];
-      const uint32_t tb = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * 64);
-      tmem_ld32(tb, v);
-      tmem_ld32(tb + 32, v + 32);
+      float v[32];
+      tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * 64 + half * 32), v);
       tc_fence_before();
       mbar_arrive(smem_u32(&tempty_bar[acc]));
       int b, oy, ox;
@@ -296,19 +298,20 @@ __global__ void __launch_bounds__(kFwdThreads, 2)
       const bool valid = y < g.eh && x < g.ew;
       uint8_t *orow = smem_gen + o_off + (size_t)ob * kFwdOut + (size_t)row * 128;
 #pragma unroll
-      for (int c = 0; c < 8; c++) {
+      for (int cc = 0; cc < 4; cc++) {
+        const int c = half * 4 + cc;   // 16-byte chunk (8 channels) of the pixel's row
         const float4 b0 = *reinterpret_cast<const float4 *>(bias_sh + c * 8);
         const float4 b1 = *reinterpret_cast<const float4 *>(bias_sh + c * 8 + 4);
         const float bb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
         float r[8];
 #pragma unroll
-        for (int j = 0; j < 8; j++) r[j] = valid ? fmaxf(v[c * 8 + j] + bb[j], 0.f) : 0.f;
+        for (int j = 0; j < 8; j++) r[j] = valid ? fmaxf(v[cc * 8 + j] + bb[j], 0.f) : 0.f;
         *reinterpret_cast<uint4 *>(orow + ((c ^ (row & 7)) << 4)) =
             make_uint4(pack_bf16x2(r[0], r[1]), pack_bf16x2(r[2], r[3]),
                        pack_bf16x2(r[4], r[5]), pack_bf16x2(r[6], r[7]));
       }
       fence_proxy_async_smem();
-      named_bar_sync(1, 128);
+      named_bar_sync(1, kFwdEpi);
       const uint32_t tile = smem_base + o_off + (uint32_t)ob * kFwdOut;
       if (et == 0) {
         tma_store_4d(&tmO, tile, 0, ox, oy, b);
@@ -346,22 +349,20 @@ __global__ void __launch_bounds__(kFwdThreads, 2)
         gram_fin = ok;
         gram_any = gfirst ? 0 : 1;
       }
-      named_bar_sync(1, 128);
+      named_bar_sync(1, kFwdEpi);
       tc_fence_after();
       if (q < 2) {   // rows = channels 0..63 (TMEM lanes 64..127 hold the zero rows' products)
-        float v[64];
+        float v[32];
         if (gram_any && gram_fin) {
-          const uint32_t tg = tmem_base + ((uint32_t)(q * 32) << 16) + 128u;
-          tmem_ld32(tg, v);
-          tmem_ld32(tg + 32, v + 32);
+          tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + 128u + (uint32_t)(half * 32), v);
         } else {
 #pragma unroll
-          for (int j = 0; j < 64; j++) v[j] = 0.f;
+          for (int j = 0; j < 32; j++) v[j] = 0.f;
         }
         float4 *dst = reinterpret_cast<float4 *>(gram_part + (size_t)blockIdx.x * kFwdGramRun +
-                                                 (size_t)row * 64);
+                                                 (size_t)row * 64 + half * 32);
 #pragma unroll
-        for (int j = 0; j < 16; j++)
+        for (int j = 0; j < 8; j++)
           dst[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
       }
     }

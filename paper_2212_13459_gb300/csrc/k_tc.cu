@@ -1324,7 +1324,12 @@ __global__ void __launch_bounds__(kThreads, 1)
           const int j = k * 8 + (lane >> 2);
           float r[8];
           swap_tile_read8(tsm, j, cg, r);
-          const EpiPx px = epi_px(a, g, tg, b, oy, ox, c + j);
+          EpiPx px;   // (epi_px for a patch 8 wide)
+          px.y = oy + (c + j) / kSHTW;
+          px.x = ox + (c + j) % kSHTW;
+          px.in = px.y < a.Hb && px.x < a.Wb;
+          px.valid = px.y < (g.eh >> a.level) && px.x < (g.ew >> a.level);
+          px.o = (((size_t)b * a.Hb + px.y) * a.Wb + px.x) * a.cout;
           // (also input gradients of this shape: their mask is read here)
           uint4 mk = make_uint4(0u, 0u, 0u, 0u);
           if (!hoist && a.mask) mk = load_mask8(a, px, n + cg * 8);
