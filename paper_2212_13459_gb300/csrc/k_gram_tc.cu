@@ -192,15 +192,22 @@ __device__ __forceinline__ void gram_tc_body(const GramTcArgs &a, int run, int t
   }
 }
 
+// whether tile I * nJ + J holds elements on or above the diagonal
+__host__ __device__ inline bool gram_tile_needed(int tile, int nJ, int N) {
+  return (tile / nJ) * 128 < (tile % nJ + 1) * N;
+}
+
 // The Grams of several layers in one launch (they are independent, and alone none fills the chip to
 // its end: 756 x 1008, four launches 74 us, one 59; 64 x 64, 36 us, 10). CTA c of layer l
-// takes run c / tiles, tile c % tiles.
+// takes run c / tiles, the (c % tiles)-th of the tiles that meet the diagonal or lie above it (for
+// C = 512 six of the eight).
 __global__ void __launch_bounds__(kThreads, 2) gram_tc_kernel(GramTcBatch g) {
   int l = 0;
   while (l + 1 < g.n && (int)blockIdx.x >= g.L[l + 1].cta0) l++;
   const GramTcArgs &a = g.L[l];
-  const int c = (int)blockIdx.x - a.cta0, tiles = a.nI * a.nJ;
-  const int run = c / tiles, tile = c % tiles;
+  const int c = (int)blockIdx.x - a.cta0, run = c / a.tiles;
+  int left = c % a.tiles, tile = 0;
+  while (!gram_tile_needed(tile, a.nJ, a.N) || left-- > 0) tile++;
   switch (a.N) {
     case 64: gram_tc_body<64, false>(a, run, tile); break;
     case 128: gram_tc_body<128, false>(a, run, tile); break;
@@ -231,7 +238,7 @@ __device__ __forceinline__ void two_sum_add(float &s, float &c, float x) {
 // whose pairs are added in warp order (deterministic). Each element's pair becomes FP64 once.
 // Bound: the read of the partials from L2. One launch per layer, with 64-bit index divisions and
 // two barriers per 128 elements, took 58 us (64 x 64 pixels) to 83 us (756 x 1008) per evaluation;
-// this takes 13 and 60 us (cold, under the profiler; 125 MB of partials at 756 x 1008).
+// this takes 11 and 51 us (cold, under the profiler).
 constexpr int kRedWarps = 16;
 __global__ void __launch_bounds__(kRedWarps * 32) gram_tc_reduce_kernel(GramReduceArgs a) {
   __shared__ float2 red[kRedWarps][128];
@@ -241,7 +248,9 @@ __global__ void __launch_bounds__(kRedWarps * 32) gram_tc_reduce_kernel(GramRedu
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int sub = warp % L.split, grp = warp / L.split;
   const int e = (((int)blockIdx.x - L.cta0) * (kRedWarps / L.split) + grp) * 128 + lane * 4;
-  const bool live = e < L.C * L.C;
+  // G is symmetric, bit for bit (the same products in the same order), and the finaliser reads the
+  // 32 x 32 tiles on and above the diagonal only
+  const bool live = e < L.C * L.C && e % L.C >= (e / L.C & ~31);
   pdl_begin();
   float s[4] = {0.f, 0.f, 0.f, 0.f}, c[4] = {0.f, 0.f, 0.f, 0.f};
   if (live) {
@@ -345,7 +354,9 @@ cudaError_t launch_gram_tc(GramTcBatch g, cudaStream_t s) {
     a.aload = gram_needs_aload(a) ? 1 : 0;
     if (a.aload && a.N != 256) return cudaErrorInvalidValue;
     a.cta0 = ctas;
-    ctas += a.nruns * a.nI * a.nJ;
+    a.tiles = 0;
+    for (int t = 0; t < a.nI * a.nJ; t++) a.tiles += gram_tile_needed(t, a.nJ, a.N) ? 1 : 0;
+    ctas += a.nruns * a.tiles;
   }
   if (ctas <= 0) return cudaSuccess;
   constexpr size_t smem = kGramSmem;

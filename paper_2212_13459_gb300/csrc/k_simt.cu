@@ -955,40 +955,52 @@ void launch_gram_reduce(const float *part, int nchunks, int C, double *Gacc, boo
 }
 
 // ---- style finalisation: G = Gacc / np, E_L = w ||G - Ghat||^2, R = (4 w / np)(G - Ghat) -------------
-// One launch over the elements of all layers. The thread of a diagonal element also forms the
-// channel's mean / std terms of Eq. 5 from the channel sum and G_jj: beta_j (added to R_jj),
-// alpha_j (epilogue offset), its share of the moment loss, and the moments themselves when
-// requested. The CTAs' loss partials are added per layer, in CTA order, by the last CTA to finish.
-// Bound: FP64 (about seven operations per element at two per SM and clock) and latency; four
-// elements per thread are loaded together. Three launches with 16 elements in turn per thread and
-// 64-bit divisions took 36 us; this takes 16.
-constexpr int kFinThreads = 256, kFinPer = 4 * kFinThreads;   // elements per CTA
-static_assert(kFinalizeCtas * kFinPer >= 64 * 64 + 128 * 128 + 256 * 256 + 2 * 512 * 512 &&
-              4096 % kFinPer == 0, "every CTA lies in one layer");
+// One launch over the 32 x 32 tiles on and above the diagonals of all layers; G, Ghat and R are
+// symmetric, and a tile above the diagonal also writes its mirror image (through shared memory).
+// The thread of a diagonal element also forms the channel's mean / std terms of Eq. 5 from the
+// channel sum and G_jj: beta_j (added to R_jj), alpha_j (epilogue offset), its share of the moment
+// loss, and the moments themselves when requested. The CTAs' loss partials are added per layer, in
+// CTA order, by the last CTA to finish.
+// Bound: FP64 (about six operations per element at two per SM and clock) and latency; four
+// elements per thread are loaded together. Three launches over all elements, 16 in turn per thread,
+// with 64-bit divisions, took 36 us; one launch over all elements 16.5; this 15.
+constexpr int kFinThreads = 256;
+__host__ __device__ inline int fin_tiles(int C) { return C / 32 * (C / 32 + 1) / 2; }
 __global__ void __launch_bounds__(kFinThreads) style_finalize_kernel(StyleFinalizeArgs a) {
   __shared__ double red[kFinThreads];
+  __shared__ double tg[32][33];
+  __shared__ float tr[32][33];
   __shared__ int last_sh;
   const int tid = threadIdx.x;
   int l = 0, b = blockIdx.x;
-  while (b >= a.L[l].C * a.L[l].C / kFinPer) b -= a.L[l].C * a.L[l].C / kFinPer, l++;
+  while (b >= fin_tiles(a.L[l].C)) b -= fin_tiles(a.L[l++].C);
   const StyleLayerArgs L = a.L[l];
-  const double inv = L.inv_np, rs = L.rs;
-  double s = 0.0, g[4], h[4];
-  const int e0 = b * kFinPer + tid;
+  int ti = 0;   // tile (ti, tj), ti <= tj
+  for (int n = L.C / 32; b >= n - ti; ti++) b -= n - ti;
+  const int tj = ti + b;
+  const double inv = L.inv_np, rs = L.rs, we = ti == tj ? L.w : 2.0 * L.w;
+  const int j = tj * 32 + (tid & 31), i0 = ti * 32 + (tid >> 5);   // rows i0, i0 + 8, ...
   pdl_begin();
+  double s = 0.0, g[4], h[4];
 #pragma unroll
   for (int k = 0; k < 4; k++) {
-    g[k] = L.Gacc[e0 + k * kFinThreads];
-    h[k] = L.Ghat ? L.Ghat[e0 + k * kFinThreads] : 0.0;
+    const int e = (i0 + 8 * k) * L.C + j;
+    g[k] = L.Gacc[e];
+    h[k] = L.Ghat ? L.Ghat[e] : 0.0;
   }
+  auto put = [&](int e, double G, float r) {
+    L.Gout[e] = G;
+    if (a.r_is_bf16)
+      reinterpret_cast<__nv_bfloat16 *>(L.R)[e] = __float2bfloat16_rn(r);
+    else
+      reinterpret_cast<float *>(L.R)[e] = r;
+  };
 #pragma unroll
   for (int k = 0; k < 4; k++) {
-    const int e = e0 + k * kFinThreads;
+    const int i = i0 + 8 * k;
     const double G = g[k] * inv, d = G - h[k];
-    L.Gout[e] = G;
-    s += L.w * d * d;
+    s += we * d * d;
     double r = rs * d;
-    const int i = e / L.C, j = e % L.C;
     if (i == j && L.S) {
       // rounded products (no contraction into an FMA), so the loss pass reproduces the target
       // pass's mean bit for bit when x = v
@@ -1004,13 +1016,20 @@ __global__ void __launch_bounds__(kFinThreads) style_finalize_kernel(StyleFinali
         r += beta;
       }
     }
-    if (a.r_is_bf16)
-      reinterpret_cast<__nv_bfloat16 *>(L.R)[e] = __float2bfloat16_rn((float)r);
-    else
-      reinterpret_cast<float *>(L.R)[e] = (float)r;
+    put(i * L.C + j, G, (float)r);
+    if (ti != tj) {
+      tg[(tid >> 5) + 8 * k][tid & 31] = G;
+      tr[(tid >> 5) + 8 * k][tid & 31] = (float)r;
+    }
   }
   red[tid] = s;
   __syncthreads();
+  if (ti != tj)
+#pragma unroll
+    for (int k = 0; k < 4; k++) {   // element (tj * 32 + row, ti * 32 + column)
+      const int row = (tid >> 5) + 8 * k, col = tid & 31;
+      put((tj * 32 + row) * L.C + ti * 32 + col, tg[col][row], tr[col][row]);
+    }
   for (int k = kFinThreads / 2; k > 0; k >>= 1) {
     if (tid < k) red[tid] += red[tid + k];
     __syncthreads();
@@ -1026,10 +1045,9 @@ __global__ void __launch_bounds__(kFinThreads) style_finalize_kernel(StyleFinali
   if (tid < 32 * kNStyle) {   // a warp per layer: lane q the CTAs q, q + 32, ... in order, a tree
     const int wl = tid >> 5;
     int c0 = 0;
-    for (int q = 0; q < wl; q++) c0 += a.L[q].C * a.L[q].C / kFinPer;
-    const int n = a.L[wl].C * a.L[wl].C / kFinPer;
+    for (int q = 0; q < wl; q++) c0 += fin_tiles(a.L[q].C);
     double t = 0.0;
-    for (int q = tid & 31; q < n; q += 32) t += __ldcg(a.partial + c0 + q);
+    for (int q = tid & 31; q < fin_tiles(a.L[wl].C); q += 32) t += __ldcg(a.partial + c0 + q);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
     if ((tid & 31) == 0) a.Eparts[wl] = t;
@@ -1041,11 +1059,11 @@ void launch_style_finalize(const StyleFinalizeArgs &a, cudaStream_t s) {
   int n = 0;
   StyleFinalizeArgs b = a;
   for (int l = 0; l < kNStyle; l++) {
-    n += a.L[l].C * a.L[l].C;
+    n += fin_tiles(a.L[l].C);
     b.L[l].inv_np = 1.0 / a.L[l].np;   // (two FP64 divisions per thread are half the kernel)
     b.L[l].rs = 4.0 * a.L[l].w / a.L[l].np;
   }
-  launch_pdl(true, style_finalize_kernel, n / kFinPer, kFinThreads, 0, s, b);
+  launch_pdl(true, style_finalize_kernel, n, kFinThreads, 0, s, b);
 }
 
 // ---- channel sums over owned pixels, all style layers in one launch -------------------------------

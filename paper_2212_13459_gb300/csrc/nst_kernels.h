@@ -12,8 +12,8 @@ struct GramChunk {
 };
 
 struct StyleLayerArgs {
-  const double *Gacc;  // sum over owned pixels of V V^T (FP64)
-  const double *Ghat;  // G^L(v), or null: zero
+  const double *Gacc;  // sum over owned pixels of V V^T (FP64; symmetric, see launch_gram_tc_reduce)
+  const double *Ghat;  // G^L(v) (symmetric), or null: zero
   double *Gout;        // G^L(x) = Gacc / np
   void *R;             // (4 w / np)(G - Ghat) + diag(beta), FP32 or BF16
   int C;
@@ -28,7 +28,7 @@ struct StyleLayerArgs {
   float *alpha;
   double *mean_out, *std_out;
 };
-constexpr int kFinalizeCtas = 596;    // 1,024 elements of the five Gram matrices each
+constexpr int kFinalizeCtas = 321;    // 32 x 32 tiles on and above the diagonals of the five Grams
 struct StyleFinalizeArgs {
   StyleLayerArgs L[kNStyle];
   double *Eparts;   // [5]
@@ -178,7 +178,7 @@ struct GramTcArgs {
   float *part;                // [runs][nI * nJ][128][N] FP32 partial tiles
   unsigned *err;
   int nruns;
-  int cta0, aload;            // set by the launcher
+  int cta0, aload, tiles;     // set by the launcher
 };
 struct GramTcBatch {
   GramTcArgs L[kNStyle];
@@ -190,7 +190,8 @@ cudaError_t encode_gram_map(CUtensorMap *m, const void *base, int C, int own_w, 
                             long long row_stride_px, int TH, int TW);
 cudaError_t launch_gram_tc(GramTcBatch g, cudaStream_t s);
 // Gacc[i][j] (+)= the sum over nruns FP32 partial tiles (run r at part + r * nI * nJ * 128 * N,
-// tile (I, J) of 128 x N floats) of n layers, fixed order
+// tile (I, J) of 128 x N floats) of n layers, fixed order, in the 32 x 32 tiles on and above the
+// diagonal (G is symmetric; the style finaliser reads no others)
 struct GramReduceLayer {
   const float *part;
   int nruns, C, N, nI, nJ;
