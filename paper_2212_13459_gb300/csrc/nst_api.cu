@@ -781,6 +781,7 @@ nst_status forward_batch(nst_ctx *ctx, const PassPlan &p, const Batch &bt, const
     use_patches(a, p, bt.fwd[kind][l]);
     a.A = kPoolAfter[l - 1] ? ws.pool[l - 1] : ws.act[l - 1];
     a.Wt = ctx->d_wf[l];
+    a.const_w = 1;
     a.out = ws.act[l];
     a.mode = kEpiForward;
     a.bias = ctx->d_bias[l];
@@ -943,6 +944,7 @@ nst_status backward_batch(nst_ctx *ctx, const PassPlan &p, const Batch &bt, cons
     a.B = bt.B; a.Hb = p.Hb >> lv; a.Wb = p.Wb >> lv;
     a.cin = kCout[l]; a.cout = kCin[l]; a.taps = 9;
     a.A = ws.g[cur]; a.Wt = ctx->d_wd[l];
+    a.const_w = 1;
     a.out = ws.g[1 - cur];
     a.mode = kEpiBackward;
     a.geom = geom;

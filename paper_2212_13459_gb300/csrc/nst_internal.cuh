@@ -100,6 +100,8 @@ struct ConvArgs {
   int cin, cout, taps;  // main phase
   int k2;               // phase-2 depth (0 = none)
   const void *A, *Wt;   // main phase input [B][Hb][Wb][cin], weights [cout][taps][cin]
+  int const_w;          // no kernel of the stream writes Wt (the context's own weights): the
+                        // tensor-core kernels fetch it ahead of pdl_begin()
   const void *A2, *W2;  // phase 2 input [B][Hb][Wb][k2], weights [cout][k2]
   void *out;            // [B][Hb][Wb][cout]
   int mode;
