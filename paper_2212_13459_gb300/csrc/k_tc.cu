@@ -1736,7 +1736,8 @@ cudaError_t launch_conv_tc(const ConvArgs &a, cudaStream_t s) {
     const long long m256 = count(kSwapBP);
     swap = !conv_tc_main128(m256, count(128));
   }
-  int BN = swap ? kSwapBN : (a.cout >= 256 ? 256 : a.cout);
+  // channels per tile: the widest of 256, 128 and 64 that divides cout (192 takes 64, 384 takes 128)
+  int BN = a.cout % 256 == 0 ? 256 : a.cout % 128 == 0 ? 128 : 64;
   const int rows = swap ? kSwapBP : 128;
   TcGeom tg;
   if (a.tiles) {
