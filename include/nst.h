@@ -175,9 +175,10 @@ nst_status nst_tile_plan(int H, int W, int tiles_h, int tiles_w, int margin, int
  * The inverse-BFGS matrix of the m newest pairs (the matrix the two-loop recursion applies),
  * H0 = gamma I with gamma = s^T y / y^T y of the newest pair, pairs with y^T s <= 1e-10 skipped,
  * no line search: step 1 except min(1, 1/||g||_1) on the first iteration. Applied in its compact
- * form (two passes over the stored vectors per step). FP32 vectors, dot products summed in FP64
- * in a fixed order, all on the device (no host round trip). State (history 2 (m + 1) n floats)
- * is owned by the nst_lbfgs object, allocated at create. */
+ * form (two passes over the stored vectors per step). FP32 vectors; dot products: FP32 runs of 16
+ * elements, added in compensated FP32 (48 bits) within a CTA and in FP64 beyond, with the range of
+ * an FP64 sum, in a fixed order, all on the device (no host round trip). State (history
+ * 2 (m + 1) n floats) is owned by the nst_lbfgs object, allocated at create. */
 nst_status nst_lbfgs_create(nst_lbfgs **out, long long n, int m);
 /* As nst_lbfgs_create, with flags. NST_LBFGS_HOST_HISTORY keeps the 2 (m + 1) history vectors in
  * page-locked host memory mapped into the device address space (on a Grace-Blackwell node the

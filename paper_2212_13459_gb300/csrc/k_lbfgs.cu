@@ -37,14 +37,19 @@ int lbfgs_partials_count(int m) { return 4 * (m + 1) * dot_blocks(m); }
 //
 // Bound: HBM (2 (count + 1) + 2 vectors read once). What kept it from there was the FP64 unit,
 // which retires two operations per SM and clock on this GPU: a double add (and a conversion) per
-// 16 elements and dot, and 80 double shuffle-adds per warp at the end. So a thread's FP32 chunks
-// are added in compensated FP32 (Sum): the error of the chunks themselves, about 2^-24 / sqrt(their
-// number), stays seven orders above that of adding them. The warp reduction is a reduce-scatter
+// 16 elements and dot, and 80 double shuffle-adds per warp at the end. So a CTA's FP32 chunks are
+// added in compensated FP32 (Sum, 48 bits): the error of the chunks themselves, about 2^-24 /
+// sqrt(their number), stays orders above that of adding them, and pairs and FP64 sums of the same
+// chunks came out the same doubles for 6,912 to 9.7 M elements. The warp reduction is a reduce-scatter
 // (16 exchanges for 16 dots, not 80), and the last CTA of a group to finish adds the CTAs'
 // partials in FP64 in index order, in parallel over the groups, where the single CTA of the solve
 // spent 15 us on it. CTAs of all groups that read the same elements are neighbours in launch
 // order, so g and g_prev come from L2 for all but one of them. Measured with 100 stored pairs of
-// 2.29 M elements: 594 -> 345 us (5.4 TB/s); 10 pairs of 36.6 M: 634 us (5.8 TB/s).
+// 2.29 M elements: 594 -> 345 us (5.4 TB/s); 10 pairs of 36.6 M: 634 us (5.8 TB/s). The loads in
+// flight are bounded by the registers: an FP64 sum of two of the dots beside the pairs, a test of
+// every chunk's size, or a second pass over the elements after this one each cost 5 to 8 %.
+// A dot that leaves FP32's range within a CTA comes out infinite or NaN, sets c->beyond, and is made
+// again in FP64 by the solve (lbfgs_dots_again).
 struct Sum {   // s + c: the sum with the rounding errors of its additions (Knuth's TwoSum)
   float s, c;
   __device__ __forceinline__ double value() const {   // (c says nothing beside an infinite s)
@@ -61,11 +66,6 @@ struct Sum {   // s + c: the sum with the rounding errors of its additions (Knut
   }
 };
 
-// The chunks are added scaled by 2^-32 (exact): a sum of any number of them stays within FP32's
-// range where each does.
-constexpr float kDotDown = 0x1p-32f;
-constexpr double kDotUp = 0x1p32;
-
 template <int G>
 struct DotAcc {
   Sum acc[4 * G];
@@ -76,7 +76,7 @@ struct DotAcc {
   }
   __device__ __forceinline__ void flush() {
 #pragma unroll
-    for (int d = 0; d < 4 * G; d++) acc[d].add(part[d] * kDotDown), part[d] = 0.f;
+    for (int d = 0; d < 4 * G; d++) acc[d].add(part[d]), part[d] = 0.f;
   }
   __device__ __forceinline__ void add(int j, float sv, float wv, float gv, float yv) {
     part[4 * j] = fmaf(sv, gv, part[4 * j]);
@@ -88,8 +88,7 @@ struct DotAcc {
 
 __global__ void __launch_bounds__(kDotThreads) lbfgs_dots_kernel(
     const float *g, const float *g_prev, const float *S, float *Y, long long stride, long long n,
-    LbfgsCtl *c, int first, int vec,
-    double *partials) {
+    LbfgsCtl *c, int first, int vec, double *partials) {
   constexpr int G = kLbGroup;
   static_assert(4 * G == 16, "the warp reduce-scatter below takes 16 dots");
   __shared__ long long off[G];
@@ -192,7 +191,7 @@ __global__ void __launch_bounds__(kDotThreads) lbfgs_dots_kernel(
   if (threadIdx.x < 4 * nj) {   // the warps in index order
     Sum v = red[0][threadIdx.x];
     for (int w = 1; w < kDotThreads / 32; w++) v.merge(red[w][threadIdx.x].s, red[w][threadIdx.x].c);
-    partials[(size_t)(grp * G * 4 + threadIdx.x) * nb + cta] = v.value() * kDotUp;
+    partials[(size_t)(grp * G * 4 + threadIdx.x) * nb + cta] = v.value();
     __threadfence();
   }
   __syncthreads();
@@ -208,7 +207,10 @@ __global__ void __launch_bounds__(kDotThreads) lbfgs_dots_kernel(
     for (int q = l; q < nb; q += 16) v += __ldcg(partials + (size_t)(grp * G * 4 + d) * nb + q);
 #pragma unroll
   for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if (l == 0 && d < 4 * nj) c->dots[grp * G * 4 + d] = v;
+  if (l == 0 && d < 4 * nj) {
+    c->dots[grp * G * 4 + d] = v;
+    if (!(fabs(v) <= DBL_MAX)) atomicOr(&c->beyond, 1u);
+  }
   if (threadIdx.x == 0) c->arrived[grp] = 0u;
 }
 
@@ -223,8 +225,8 @@ void launch_lbfgs_dots(const float *g, const float *g_prev, const float *S, floa
   const long long need = ((vec ? n / 4 : n) + kDotThreads - 1) / kDotThreads;
   const int nb = (int)(need < 1 ? 1 : need < dot_blocks(m) ? need : dot_blocks(m));
   dim3 grid(first ? 1 : dot_groups(m), nb);
-  launch_pdl(true, lbfgs_dots_kernel, grid, kDotThreads, 0, s, g, g_prev, S, Y, stride, n, c, first, vec,
-             partials);
+  launch_pdl(true, lbfgs_dots_kernel, grid, kDotThreads, 0, s, g, g_prev, S, Y, stride, n, c, first,
+             vec, partials);
 }
 
 // The small solve: curvature test, bookkeeping, the two triangular systems and the coefficients
@@ -237,13 +239,80 @@ void launch_lbfgs_dots(const float *g, const float *g_prev, const float *S, floa
 // global memory took 1,496 us at k = 100 and 58 us at k = 10; this takes 47 and 17 us (all
 // cold, under the profiler).
 constexpr int kSolveThreads = 512;
+constexpr int kSolveCtas = 16;   // (all but one only where the dots are made again)
 constexpr int kSolveParts = kSolveThreads / kMaxHistory;          // threads per row of Y^T Y
 constexpr int kSolveRow = kMaxHistory / kSolveParts;              // its elements each holds
 static size_t solve_smem(int m) { return (size_t)m * (m | 1) * sizeof(double); }
 
-__global__ void __launch_bounds__(kSolveThreads) lbfgs_solve_kernel(LbfgsCtl *c, int m, int first,
-                                                                    double eps, double *SY,
-                                                                    double *YY) {
+// The dots of the fused pass once more, FP32 chunks of 16 elements added in FP64 throughout: for sums
+// beyond FP32's range (gradients from about 1e17 on) and for NaN and infinity, which stay. CTA b of
+// gridDim.x takes elements b kSolveThreads + thread, ...; true in the last CTA to finish, with c->dots
+// set. Y holds y_new in the spare slot (the fused pass wrote it). No inlining: the solve's registers
+// are its own.
+__device__ __noinline__ bool lbfgs_dots_again(LbfgsCtl *c, const float *g, const float *S,
+                                              const float *Y, long long stride, long long n, int first,
+                                              double *partials) {
+  __shared__ double red[kSolveThreads / 32][4];
+  __shared__ int last_sh;
+  const int tid = threadIdx.x, lane = tid & 31, nd = first ? 1 : 4 * (c->count + 1);
+  const float *yn = Y + c->spare * stride;
+  for (int p = 0; 4 * p < nd; p++) {
+    const long long off = (p == 0 ? c->spare : c->order[p - 1]) * stride;
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    float part[4] = {0.f, 0.f, 0.f, 0.f};
+    int chunk = 0;
+    auto flush = [&]() {
+      chunk = 0;
+#pragma unroll
+      for (int q = 0; q < 4; q++) acc[q] += (double)part[q], part[q] = 0.f;
+    };
+    for (long long i = (long long)blockIdx.x * kSolveThreads + tid; i < n;
+         i += (long long)gridDim.x * kSolveThreads) {
+      if (first) {
+        part[0] += fabsf(g[i]);
+      } else {
+        const float sv = S[off + i], yv = Y[off + i];
+        part[0] = fmaf(sv, g[i], part[0]);
+        part[1] = fmaf(yv, g[i], part[1]);
+        part[2] = fmaf(sv, yn[i], part[2]);
+        part[3] = fmaf(yv, yn[i], part[3]);
+      }
+      if (++chunk == 16) flush();
+    }
+    flush();
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
+      if (lane == 0) red[tid >> 5][q] = acc[q];
+    }
+    __syncthreads();
+    if (tid < 4) {
+      double v = 0.0;
+      for (int w = 0; w < kSolveThreads / 32; w++) v += red[w][tid];
+      partials[(size_t)(4 * p + tid) * gridDim.x + blockIdx.x] = v;
+      __threadfence();
+    }
+    __syncthreads();
+  }
+  if (tid == 0) last_sh = atomicAdd(&c->arrived[0], 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last_sh) return false;
+  __threadfence();
+  for (int d = tid; d < nd; d += kSolveThreads) {   // the CTAs in index order
+    double v = 0.0;
+    for (unsigned b = 0; b < gridDim.x; b++) v += __ldcg(partials + (size_t)d * gridDim.x + b);
+    c->dots[d] = v;
+  }
+  if (tid == 0) c->arrived[0] = c->beyond = 0u;
+  __syncthreads();
+  return true;
+}
+
+__global__ void __launch_bounds__(kSolveThreads)
+    lbfgs_solve_kernel(LbfgsCtl *c, int m, int first, double eps, double *SY, double *YY,
+                       const float *g, const float *S, const float *Y, long long stride, long long n,
+                       double *partials) {
   extern __shared__ double Rs[];   // [k][m | 1]: odd row stride, columns without bank conflicts
   __shared__ double sg[kMaxHistory], yg[kMaxHistory], snew[kMaxHistory], ynew[kMaxHistory];
   __shared__ double diag[kMaxHistory], u[kMaxHistory], w[kMaxHistory];
@@ -251,6 +320,11 @@ __global__ void __launch_bounds__(kSolveThreads) lbfgs_solve_kernel(LbfgsCtl *c,
   __shared__ int sl[kMaxHistory], old[kMaxHistory];
   const int tid = threadIdx.x, lane = tid & 31;
   pdl_begin();
+  if (c->beyond) {   // (unchanged until every CTA has read it)
+    if (!lbfgs_dots_again(c, g, S, Y, stride, n, first, partials)) return;
+  } else if (blockIdx.x) {
+    return;
+  }
   if (first) {
     if (tid == 0) {
       const double l1 = c->dots[0];
@@ -402,14 +476,17 @@ __global__ void __launch_bounds__(kSolveThreads) lbfgs_solve_kernel(LbfgsCtl *c,
 }
 
 cudaError_t launch_lbfgs_solve(LbfgsCtl *c, int m, int first, double eps, double *SY, double *YY,
-                               cudaStream_t s) {
+                               const float *g, const float *S, const float *Y, long long stride,
+                               long long n, double *partials, cudaStream_t s) {
   const size_t smem = solve_smem(m);
   if (smem > 32 * 1024) {   // beyond what a launch may ask for without saying so
-    const cudaError_t e = cudaFuncSetAttribute(
-        lbfgs_solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)solve_smem(kMaxHistory));
+    const cudaError_t e =
+        cudaFuncSetAttribute(lbfgs_solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)solve_smem(kMaxHistory));
     if (e != cudaSuccess) return e;
   }
-  return launch_pdl(true, lbfgs_solve_kernel, 1, kSolveThreads, smem, s, c, m, first, eps, SY, YY);
+  return launch_pdl(true, lbfgs_solve_kernel, kSolveCtas, kSolveThreads, smem, s, c, m, first, eps, SY,
+                    YY, g, S, Y, stride, n, partials);
 }
 
 __global__ void __launch_bounds__(256) lbfgs_combine_kernel(

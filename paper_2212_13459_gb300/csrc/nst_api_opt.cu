@@ -113,7 +113,8 @@ nst_status nst_lbfgs_step(nst_lbfgs *st, float *x, const float *g, void *stream)
   launch_lbfgs_dots(g, st->g_prev, st->S, st->Y, st->stride, st->n, st->ctl, st->m, first,
                     st->partials, s);
   // 2. curvature test, history update, S^T Y / Y^T Y update, small solve (one CTA)
-  if (launch_lbfgs_solve(st->ctl, st->m, first, kCurvEps, st->SY, st->YY, s) != cudaSuccess)
+  if (launch_lbfgs_solve(st->ctl, st->m, first, kCurvEps, st->SY, st->YY, g, st->S, st->Y,
+                         st->stride, st->n, st->partials, s) != cudaSuccess)
     return NST_ERR_CUDA;
   // 3. one pass forming s = t d (into the spare slot), x += s, g_prev = g
   launch_lbfgs_combine(x, st->S, st->Y, st->stride, st->g_prev, g, st->n, st->ctl, s);

@@ -22,6 +22,7 @@ struct LbfgsCtl {
   // CTAs of each group have written their partials (zero between launches)
   double dots[4 * (kMaxHistory + kLbGroup)];
   unsigned arrived[kMaxHistory / kLbGroup + 1];
+  unsigned beyond;   // some dot is not finite (set by the fused pass, cleared by the solve)
 };
 
 // the fused pass over the vectors: y = g - g_prev into the spare slot and, per stored pair and
@@ -29,9 +30,11 @@ struct LbfgsCtl {
 void launch_lbfgs_dots(const float *g, const float *g_prev, const float *S, float *Y,
                        long long stride, long long n, LbfgsCtl *c, int m, int first,
                        double *partials, cudaStream_t s);
-// one CTA: curvature test and history bookkeeping, the compact-form solve, coefficients of the step
+// one CTA: curvature test and history bookkeeping, the compact-form solve, coefficients of the step;
+// before that, where a dot is not finite (a sum beyond FP32's range), all dots again in FP64
 cudaError_t launch_lbfgs_solve(LbfgsCtl *c, int m, int first, double eps, double *SY, double *YY,
-                               cudaStream_t s);
+                               const float *g, const float *S, const float *Y, long long stride,
+                               long long n, double *partials, cudaStream_t s);
 // the step: s = t d into the spare slot, x += s, g_prev = g
 void launch_lbfgs_combine(float *x, float *S, const float *Y, long long stride, float *g_prev,
                           const float *g, long long n, const LbfgsCtl *c, cudaStream_t s);
