@@ -124,7 +124,7 @@ __device__ __forceinline__ void epilogue32(const ConvArgs &a, const BlockGeom &g
     const float4 *b4 = reinterpret_cast<const float4 *>(a.bias + n);
 #pragma unroll
     for (int q = 0; q < 8; q++) {
-      const float4 bb = __ldg(b4 + q);
+      const float4 bb = b4[q];
       v[4 * q] = valid ? fmaxf(v[4 * q] + bb.x, 0.f) : 0.f;
       v[4 * q + 1] = valid ? fmaxf(v[4 * q + 1] + bb.y, 0.f) : 0.f;
       v[4 * q + 2] = valid ? fmaxf(v[4 * q + 2] + bb.z, 0.f) : 0.f;
@@ -300,10 +300,11 @@ __device__ __forceinline__ void swap_tile_read8(const uint8_t *tsm, int j, int c
   r[4] = f1.x; r[5] = f1.y; r[6] = f1.z; r[7] = f1.w;
 }
 
-// 8 consecutive FP32 biases (16-byte aligned)
+// 8 consecutive FP32 biases (16-byte aligned). Plain loads, as everywhere here: in a single layer's
+// launch the bias is the caller's, and the kernel before this one may have written it.
 __device__ __forceinline__ void load8_bias(const float *p, float *bb) {
-  const float4 b0 = __ldg(reinterpret_cast<const float4 *>(p));
-  const float4 b1 = __ldg(reinterpret_cast<const float4 *>(p + 4));
+  const float4 b0 = reinterpret_cast<const float4 *>(p)[0];
+  const float4 b1 = reinterpret_cast<const float4 *>(p)[1];
   bb[0] = b0.x; bb[1] = b0.y; bb[2] = b0.z; bb[3] = b0.w;
   bb[4] = b1.x; bb[5] = b1.y; bb[6] = b1.z; bb[7] = b1.w;
 }
@@ -908,8 +909,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (a.pool_out && BN == 64)
 #pragma unroll
       for (int k = 0; k < 4; k++)
-        pbias[k] = __ldg(reinterpret_cast<const float2 *>(a.bias + nt * BN + half * (BN / 2) +
-                                                          8 * k + 2 * (lane & 3)));
+        pbias[k] = *reinterpret_cast<const float2 *>(a.bias + nt * BN + half * (BN / 2) + 8 * k +
+                                                     2 * (lane & 3));
     int it = 0;
     for (int t = m_first; t < m_total; t += m_step, it++) {
       const int acc = it % NACC;
@@ -951,8 +952,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           if constexpr (BN != 64) {
 #pragma unroll
             for (int k = 0; k < 4; k++)
-              pb[k] = __ldg(reinterpret_cast<const float2 *>(a.bias + nt * BN + c + 8 * k +
-                                                             2 * (lane & 3)));
+              pb[k] = *reinterpret_cast<const float2 *>(a.bias + nt * BN + c + 8 * k +
+                                                        2 * (lane & 3));
             bp = pb;
           }
 #pragma unroll
