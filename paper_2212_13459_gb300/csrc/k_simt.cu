@@ -712,35 +712,59 @@ template void launch_unpool<__nv_bfloat16>(const __nv_bfloat16 *, const __nv_bfl
 // With chunks == null, V is one flat [n_flat][C] matrix and CTA c takes pixels
 // [c * chunk_len, min((c + 1) * chunk_len, n_flat)).
 //
-// 64 threads, 8 x 8 elements each (two groups of 4 channels on either side), packed FMAs, 16-pixel
-// slices double-buffered with the next one in flight to registers. Bound as in the CUDA-core
-// convolution: shared-memory reads and FMAs take 16 clocks each per pixel and warp, where 4 x 4
-// elements per thread took 8 : 4. 47,628 pixels x 256 channels: 154 -> 84 us.
-// FP32 features go straight to shared memory (cp.async, three slices): without the staging
-// registers nine CTAs fit an SM instead of six, and the planned 1,216 CTAs run in one wave.
+// 64 threads; slices of 16 pixels, NBUF - 1 of them ahead on their way to shared memory (cp.async, in
+// the features' own type); packed FMAs. BLK = 64: a CTA makes the whole 64 x 64 block, 8 x 8 elements per
+// thread. BLK = 32: a quarter of it, 4 x 4 per thread. Times below: nst_gram, partials and reduction,
+// against 256 threads with 4 x 4 elements each and loads straight into the slice.
+// Many CTAs per SM: bound by FP32 FMAs and shared-memory reads, which take 16 clocks each per
+// pixel and warp at 8 x 8 (8 : 4 at 4 x 4). Pixels x channels: 50,000 x 256 163 -> 89 us in FP32, 153
+// -> 106 in BF16 (128 with BF16 staged in registers as FP32); 150,000 x 320 542 -> 357 and 534 -> 429.
+// Two slices in FP32, three in BF16: the other way round 4 % and 1.5 % slower.
+// Few CTAs: bound by a CTA's own 256 or more pixels, one after the other on the two schedulers its
+// warps sit on; four quarters on four SMs take a quarter each, with more loads in flight. 300 to
+// 5,000 x 64: 23 -> 15 us (whole blocks 25 in FP32, 27 in BF16).
 constexpr int kGramPx = 16;
-__device__ __forceinline__ void cp_async16(void *dst, const void *src, bool live) {
-  // (src is not read when the size is 0: the 16 bytes become zero)
+// 4 elements to shared memory (src is not read where live is false: zeros)
+__device__ __forceinline__ void cp_async4(float *dst, const float *src, bool live) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
                    (unsigned)__cvta_generic_to_shared(dst)),
                "l"(src), "r"(live ? 16 : 0)
                : "memory");
 }
-template <typename T>
+__device__ __forceinline__ void cp_async4(__nv_bfloat16 *dst, const __nv_bfloat16 *src, bool live) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(
+                   (unsigned)__cvta_generic_to_shared(dst)),
+               "l"(src), "r"(live ? 8 : 0)
+               : "memory");
+}
+// 4 elements from shared memory as two pairs of floats
+__device__ __forceinline__ void load4_pairs(const float *p, unsigned long long v[2]) {
+  const ulonglong2 t = *reinterpret_cast<const ulonglong2 *>(p);
+  v[0] = t.x;
+  v[1] = t.y;
+}
+__device__ __forceinline__ void load4_pairs(const __nv_bfloat16 *p, unsigned long long v[2]) {
+  float f[4];
+  load4(p, f);
+  asm("mov.b64 %0, {%1, %2};" : "=l"(v[0]) : "f"(f[0]), "f"(f[1]));
+  asm("mov.b64 %0, {%1, %2};" : "=l"(v[1]) : "f"(f[2]), "f"(f[3]));
+}
+template <typename T, int BLK, int NBUF>
 __global__ void __launch_bounds__(64) gram_partial_kernel(const T *__restrict__ V, int Hb, int Wb,
                                                           int C, const OwnRect *__restrict__ own,
                                                           const GramChunk *__restrict__ chunks,
                                                           float *__restrict__ part,
                                                           long long chunk_len, long long n_flat) {
-  constexpr bool ASYNC = sizeof(T) == 4;
-  constexpr int NBUF = ASYNC ? 3 : 2;
-  __shared__ __align__(16) float Ai[NBUF][kGramPx][64];
-  __shared__ __align__(16) float Aj[NBUF][kGramPx][64];
+  constexpr int NQ = (64 / BLK) * (64 / BLK);   // CTAs per block pair
+  constexpr int E = BLK / 8, GR = E / 4;        // elements per thread and side, in groups of 4
+  __shared__ __align__(16) T Ai[NBUF][kGramPx][BLK];
+  __shared__ __align__(16) T Aj[NBUF][kGramPx][BLK];
   const int nb = C / 64;
   const int npairs = nb * (nb + 1) / 2;
-  int pair = blockIdx.y, I = 0;
-  while (pair >= nb - I) { pair -= nb - I; I++; }
-  const int J = I + pair;
+  const int pair = blockIdx.y / NQ, quarter = blockIdx.y % NQ;
+  int I = 0, J = pair;
+  while (J >= nb - I) { J -= nb - I; I++; }
+  J += I;
   GramChunk ch;
   OwnRect r;
   if (chunks) {
@@ -749,112 +773,72 @@ __global__ void __launch_bounds__(64) gram_partial_kernel(const T *__restrict__ 
   } else {
     const long long p0 = (long long)blockIdx.x * chunk_len;
     const long long p1 = p0 + chunk_len < n_flat ? p0 + chunk_len : n_flat;
-    ch = {0, (int)p0, (int)p1, 0};
+    ch = {0, (int)p0, (int)p1};
     r = {0, 1, 0, (int)n_flat};
   }
-  const int rw = r.x1 - r.x0;
+  const int rw = r.x1 - r.x0, len = ch.p1 - ch.p0;
   const int tid = threadIdx.x;
-  // this thread loads channels 4 lq .. of pixels lp, lp + 4, ... of a slice
-  const int lq = (tid & 15) * 4, lp = tid >> 4;
-  constexpr int L = kGramPx / 4;
-  float vi[L][4], vj[L][4];
-  auto load = [&](int q0) {
+  // the CTA's channels: ci .. ci + BLK - 1 against cj .. cj + BLK - 1
+  const int ri = (NQ == 1 ? 0 : quarter / 2 * 32), rj = (NQ == 1 ? 0 : quarter % 2 * 32);
+  const int ci = I * 64 + ri, cj = J * 64 + rj;
+  const bool same = ci == cj;
+  // this thread loads channels 4 lq .. of pixels lp, lp + 256 / BLK, ... of a slice
+  constexpr int LP = 256 / BLK;
+  const int lq = (tid % (BLK / 4)) * 4, lp = tid / (BLK / 4);
+  auto fetch = [&](int buf, int k0) {   // pixels k0 .. of the chunk: one slice, one commit group
 #pragma unroll
-    for (int u = 0; u < L; u++) {
-      const int q = q0 + lp + 4 * u;
-      if (q < ch.p1) {
-        const int y = q / rw, x = q - y * rw;
-        const T *row = V + (((size_t)ch.b * Hb + r.y0 + y) * Wb + r.x0 + x) * C;
-        load4(row + I * 64 + lq, vi[u]);
-        if (I != J) load4(row + J * 64 + lq, vj[u]);
-      } else {
-#pragma unroll
-        for (int k = 0; k < 4; k++) vi[u][k] = vj[u][k] = 0.f;
-      }
-    }
-  };
-  auto store = [&](int buf) {
-#pragma unroll
-    for (int u = 0; u < L; u++) {
-      store4(&Ai[buf][lp + 4 * u][lq], vi[u]);
-      if (I != J) store4(&Aj[buf][lp + 4 * u][lq], vj[u]);
-    }
-  };
-  auto fetch = [&](int buf, int q0) {   // (ASYNC) one slice, one commit group
-#pragma unroll
-    for (int u = 0; u < L; u++) {
-      const int q = q0 + lp + 4 * u, qq = q < ch.p1 ? q : ch.p0;
-      const int y = qq / rw, x = qq - y * rw;
+    for (int u = 0; u < kGramPx / LP; u++) {
+      const int k = k0 + lp + LP * u, q = ch.p0 + (k < len ? k : 0);
+      const int y = q / rw, x = q - y * rw;
       const T *row = V + (((size_t)ch.b * Hb + r.y0 + y) * Wb + r.x0 + x) * C;
-      cp_async16(&Ai[buf][lp + 4 * u][lq], row + I * 64 + lq, q < ch.p1);
-      if (I != J) cp_async16(&Aj[buf][lp + 4 * u][lq], row + J * 64 + lq, q < ch.p1);
+      cp_async4(&Ai[buf][lp + LP * u][lq], row + ci + lq, k < len);
+      if (!same) cp_async4(&Aj[buf][lp + LP * u][lq], row + cj + lq, k < len);
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
-  // elements (ti, ti + 32 groups) x (tj, tj + 32): a warp covers 32 + 32 rows and 16 + 16 columns
+  // elements (ti + 32 g .. + 3) x (tj + 32 h .. + 3): a warp covers BLK rows and 16 (+ 16) columns
   const int ti = ((tid & 31) >> 2) * 4, tj = (tid >> 5) * 16 + (tid & 3) * 4;
-  unsigned long long acc[8][4];
+  unsigned long long acc[E][E / 2];
 #pragma unroll
-  for (int i = 0; i < 8; i++)
+  for (int i = 0; i < E; i++)
 #pragma unroll
-    for (int j = 0; j < 4; j++) acc[i][j] = 0ull;
-  if constexpr (ASYNC) {
-    fetch(0, ch.p0);
-    fetch(1, ch.p0 + kGramPx);   // (past the end: zeros)
-  } else {
-    load(ch.p0);
-    store(0);
-    if (ch.p0 + kGramPx < ch.p1) load(ch.p0 + kGramPx);
-    __syncthreads();
-  }
+    for (int j = 0; j < E / 2; j++) acc[i][j] = 0ull;
+#pragma unroll
+  for (int i = 0; i < NBUF - 1; i++) fetch(i, i * kGramPx);   // (past the end: zeros)
   int buf = 0;
-  for (int q0 = ch.p0; q0 < ch.p1; q0 += kGramPx) {
-    if constexpr (ASYNC) {
-      // this slice has arrived in every thread's part, and every thread has left the slice before
-      // it, whose buffer the slice after next takes
-      asm volatile("cp.async.wait_group 1;" ::: "memory");
-      __syncthreads();
-      fetch(buf == 0 ? 2 : buf - 1, q0 + 2 * kGramPx);
-    }
-    const float(*Bj)[64] = I != J ? Aj[buf] : Ai[buf];
+  for (int k0 = 0; k0 < len; k0 += kGramPx) {
+    // this slice has arrived in every thread's part, and every thread has left the slice before
+    // it, whose buffer the next slice to fetch takes
+    asm volatile("cp.async.wait_group %0;" ::"n"(NBUF - 2) : "memory");
+    __syncthreads();
+    fetch(buf == 0 ? NBUF - 1 : buf - 1, k0 + (NBUF - 1) * kGramPx);
+    const T(*Bj)[BLK] = same ? Ai[buf] : Aj[buf];
 #pragma unroll
     for (int p = 0; p < kGramPx; p++) {
-      float ar[8];
-      ulonglong2 b0, b1;
-      const float4 a0 = *reinterpret_cast<const float4 *>(&Ai[buf][p][ti]);
-      const float4 a1 = *reinterpret_cast<const float4 *>(&Ai[buf][p][ti + 32]);
-      ar[0] = a0.x; ar[1] = a0.y; ar[2] = a0.z; ar[3] = a0.w;
-      ar[4] = a1.x; ar[5] = a1.y; ar[6] = a1.z; ar[7] = a1.w;
-      b0 = *reinterpret_cast<const ulonglong2 *>(&Bj[p][tj]);
-      b1 = *reinterpret_cast<const ulonglong2 *>(&Bj[p][tj + 32]);
+      float ar[E];
+      unsigned long long br[E / 2];
 #pragma unroll
-      for (int i = 0; i < 8; i++) {
+      for (int g = 0; g < GR; g++) {
+        load4(&Ai[buf][p][ti + 32 * g], ar + 4 * g);
+        load4_pairs(&Bj[p][tj + 32 * g], br + 2 * g);
+      }
+#pragma unroll
+      for (int i = 0; i < E; i++) {
         const unsigned long long ad = dup2(ar[i]);
-        fma2(acc[i][0], ad, b0.x);
-        fma2(acc[i][1], ad, b0.y);
-        fma2(acc[i][2], ad, b1.x);
-        fma2(acc[i][3], ad, b1.y);
-      }
-    }
-    if constexpr (ASYNC) {
-      buf = buf == 2 ? 0 : buf + 1;
-    } else {
-      if (q0 + kGramPx < ch.p1) {
-        store(buf ^ 1);
-        if (q0 + 2 * kGramPx < ch.p1) load(q0 + 2 * kGramPx);
-      }
-      __syncthreads();
-      buf ^= 1;
-    }
-  }
-  if constexpr (ASYNC) asm volatile("cp.async.wait_all;" ::: "memory");
-  float *o = part + ((size_t)blockIdx.x * npairs + blockIdx.y) * 4096;
 #pragma unroll
-  for (int i = 0; i < 8; i++) {
-    const int row = ti + (i >> 2) * 32 + (i & 3);
-    *reinterpret_cast<ulonglong2 *>(o + row * 64 + tj) = make_ulonglong2(acc[i][0], acc[i][1]);
-    *reinterpret_cast<ulonglong2 *>(o + row * 64 + tj + 32) = make_ulonglong2(acc[i][2], acc[i][3]);
+        for (int j = 0; j < E / 2; j++) fma2(acc[i][j], ad, br[j]);
+      }
+    }
+    buf = buf == NBUF - 1 ? 0 : buf + 1;
   }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  float *o = part + ((size_t)blockIdx.x * npairs + pair) * 4096 + ri * 64 + rj;
+#pragma unroll
+  for (int i = 0; i < E; i++)
+#pragma unroll
+    for (int h = 0; h < GR; h++)
+      *reinterpret_cast<ulonglong2 *>(o + (ti + (i >> 2) * 32 + (i & 3)) * 64 + tj + 32 * h) =
+          make_ulonglong2(acc[i][2 * h], acc[i][2 * h + 1]);
 }
 
 // Gacc[C][C] (+)= sum over chunks (fixed order) of the partial blocks, mirrored for I != J. 8 warps
@@ -922,21 +906,32 @@ __global__ void __launch_bounds__(256) gram_reduce_kernel(const float *__restric
   }
 }
 
+// Up to one whole block per SM (152) runs as quarters: at 120 blocks (5,000 pixels x 192) 19.3 against
+// 25.4 us in FP32 and 21.3 against 29.5 in BF16; at 237 (20,000 x 128) 29.8 against 27.4 and 35.5 against 31.5.
+constexpr int kGramQuarters = 152;
+template <typename T>
+static void launch_gram_blocks(const T *V, int Hb, int Wb, int C, const OwnRect *own,
+                               const GramChunk *chunks, int nchunks, float *part,
+                               long long chunk_len, long long n_flat, cudaStream_t s) {
+  const int nb = C / 64, npairs = nb * (nb + 1) / 2;
+  if ((long long)nchunks * npairs <= kGramQuarters)
+    gram_partial_kernel<T, 32, 8><<<dim3(nchunks, 4 * npairs), 64, 0, s>>>(
+        V, Hb, Wb, C, own, chunks, part, chunk_len, n_flat);
+  else
+    gram_partial_kernel<T, 64, sizeof(T) == 4 ? 2 : 3><<<dim3(nchunks, npairs), 64, 0, s>>>(
+        V, Hb, Wb, C, own, chunks, part, chunk_len, n_flat);
+}
+
 template <typename T>
 void launch_gram_partial(const T *V, int Hb, int Wb, int C, const OwnRect *own,
                          const GramChunk *chunks, int nchunks, float *part, cudaStream_t s) {
-  const int nb = C / 64;
-  dim3 grid(nchunks, nb * (nb + 1) / 2);
-  gram_partial_kernel<T><<<grid, 64, 0, s>>>(V, Hb, Wb, C, own, chunks, part, 0, 0);
+  launch_gram_blocks<T>(V, Hb, Wb, C, own, chunks, nchunks, part, 0, 0, s);
 }
 
 template <typename T>
 void launch_gram_partial_flat(const T *V, long long npix, int C, long long chunk_len, int nchunks,
                               float *part, cudaStream_t s) {
-  const int nb = C / 64;
-  dim3 grid(nchunks, nb * (nb + 1) / 2);
-  gram_partial_kernel<T><<<grid, 64, 0, s>>>(V, 1, (int)npix, C, nullptr, nullptr, part,
-                                              chunk_len, npix);
+  launch_gram_blocks<T>(V, 1, (int)npix, C, nullptr, nullptr, nchunks, part, chunk_len, npix, s);
 }
 template void launch_gram_partial_flat<float>(const float *, long long, int, long long, int,
                                               float *, cudaStream_t);
