@@ -717,15 +717,16 @@ void launch_bicubic(const float *x, int C, int h, int w, float *out, int H, int 
 // rows and all channels, the rows' bounds are made once per CTA, and the FP32 row sums are added
 // in compensated FP32 and divided with a remainder step: the quotient is within 2^-46 of the
 // exact one before it is rounded to FP32; with windows of at most 3 x 3 (a factor up to 2) or
-// 5 x 5 their loads are issued together. 19 us with the source in L2.
-__device__ __noinline__ float area_mean64(const float *src, int w, int y0, int y1, int x0, int x1) {
+// 5 x 5 their loads are issued together (area_kernel). 19 us with the source in L2.
+// the mean of ny x nx elements from p on, summed in FP64
+__device__ __noinline__ float area_mean64(const float *p, int w, int ny, int nx) {
   double acc = 0.0;
-  for (int y = y0; y < y1; y++) {
+  for (int y = 0; y < ny; y++, p += w) {
     float row = 0.f;
-    for (int xx = x0; xx < x1; xx++) row += src[(size_t)y * w + xx];
+    for (int k = 0; k < nx; k++) row += p[k];
     acc += (double)row;
   }
-  return (float)(acc / ((double)(y1 - y0) * (double)(x1 - x0)));
+  return (float)(acc / ((double)ny * (double)nx));
 }
 
 // sum / cnt rounded once: q is within 2 ulp, its remainder exact (no contraction into q's product)
@@ -735,12 +736,12 @@ __device__ __forceinline__ float area_divide(const Sum &acc, float cnt, float in
 }
 
 constexpr int kAreaThreads = 128, kAreaRows = 8;
-// NW > 0: no window is larger than NW x NW (the loads of an output's windows in all channels are
-// issued together); 0: any window
+// Three channels, no window larger than NW x NW: the loads of an output's windows in all channels are
+// issued together
 template <int NW>
-__global__ void __launch_bounds__(kAreaThreads) area_kernel(const float *__restrict__ x, int C,
-                                                            int h, int w, float *__restrict__ out,
-                                                            int H, int W, int R) {
+__global__ void __launch_bounds__(kAreaThreads) area_kernel(const float *__restrict__ x, int h,
+                                                            int w, float *__restrict__ out, int H,
+                                                            int W, int R) {
   __shared__ int ya[kAreaRows], yb[kAreaRows];
   const int X = blockIdx.x * kAreaThreads + threadIdx.x;
   for (long long Y0 = (long long)blockIdx.y * R; Y0 < H; Y0 += (long long)gridDim.y * R) {
@@ -758,67 +759,105 @@ __global__ void __launch_bounds__(kAreaThreads) area_kernel(const float *__restr
       const int y0 = ya[r], y1 = yb[r];
       const float cnt = (float)(y1 - y0) * (float)(x1 - x0), inv = 1.f / cnt;
       float *o = out + (size_t)(Y0 + r) * W + X;
-      if constexpr (NW > 0) {   // C = 3
-        float v[3][NW][NW];
+      float v[3][NW][NW];
 #pragma unroll
-        for (int c = 0; c < 3; c++)
+      for (int c = 0; c < 3; c++)
 #pragma unroll
-          for (int j = 0; j < NW; j++)
+        for (int j = 0; j < NW; j++)
 #pragma unroll
-            for (int k = 0; k < NW; k++)
-              v[c][j][k] = y0 + j < y1 && x0 + k < x1
-                               ? __ldg(x + ((size_t)c * h + y0 + j) * w + x0 + k)
-                               : 0.f;
+          for (int k = 0; k < NW; k++)
+            v[c][j][k] = y0 + j < y1 && x0 + k < x1
+                             ? __ldg(x + ((size_t)c * h + y0 + j) * w + x0 + k)
+                             : 0.f;
 #pragma unroll
-        for (int c = 0; c < 3; c++) {
-          Sum acc{0.f, 0.f};
+      for (int c = 0; c < 3; c++) {
+        Sum acc{0.f, 0.f};
 #pragma unroll
-          for (int j = 0; j < NW; j++) {
-            float row = 0.f;
+        for (int j = 0; j < NW; j++) {
+          float row = 0.f;
 #pragma unroll
-            for (int k = 0; k < NW; k++) row += v[c][j][k];
-            acc.add(row);
-          }
-          float m = area_divide(acc, cnt, inv);
-          if (!(fabsf(acc.s) <= FLT_MAX))   // an infinite or overflowing sum
-            m = area_mean64(x + (size_t)c * h * w, w, y0, y1, x0, x1);
-          o[(size_t)c * H * W] = m;
+          for (int k = 0; k < NW; k++) row += v[c][j][k];
+          acc.add(row);
         }
-      } else {
-        for (int c = 0; c < C; c++) {
-          const float *src = x + (size_t)c * h * w;
-          Sum acc{0.f, 0.f};
-          for (int y = y0; y < y1; y++) {
-            const float *p = src + (size_t)y * w;
-            float row = 0.f;
-            for (int xx = x0; xx < x1; xx++) row += __ldg(p + xx);
-            acc.add(row);
-          }
-          float m = area_divide(acc, cnt, inv);
-          // (as above, or a count that FP32 does not hold)
-          if (!(fabsf(acc.s) <= FLT_MAX) || cnt >= 16777216.f)
-            m = area_mean64(src, w, y0, y1, x0, x1);
-          o[(size_t)c * H * W] = m;
-        }
+        float m = area_divide(acc, cnt, inv);
+        if (!(fabsf(acc.s) <= FLT_MAX))   // an infinite or overflowing sum
+          m = area_mean64(x + ((size_t)c * h + y0) * w + x0, w, y1 - y0, x1 - x0);
+        o[(size_t)c * H * W] = m;
       }
     }
   }
 }
 
+// Any window: a thread per output, consecutive outputs of a channel (grid y) in consecutive threads
+// whatever the width. Bound: the chain of loads and adds of a window, so three CTAs of threads in four
+// of what an SM holds (with all of them the registers spill); the rows' bounds are made once per CTA,
+// the columns' without 64-bit divisions where W w fits 32 bits. A thread per output with FP64 sums
+// took 45 us for 3024 x 4032 -> 378 x 504 and 139 for 6048 x 8064 -> 756 x 1008, a thread per three
+// channels and up to eight rows 51 and 214; this 40 and 127.
+constexpr int kAreaAnyThreads = 128;
+__global__ void __launch_bounds__(kAreaAnyThreads, 12) area_any_kernel(const float *__restrict__ x,
+                                                                      int h, int w,
+                                                                      float *__restrict__ out,
+                                                                      int H, int W, int narrow) {
+  __shared__ int ya[kAreaAnyThreads + 1], yb[kAreaAnyThreads + 1];
+  const long long i0 = (long long)blockIdx.x * kAreaAnyThreads, n = (long long)H * W;
+  const int row0 = (int)(i0 / W);
+  const unsigned at = (unsigned)(i0 - (long long)row0 * W) + threadIdx.x, r = at / (unsigned)W;
+  // (rows row0 .. row0 + the last thread's r, at most kAreaAnyThreads + 1)
+  const unsigned rows = (at - threadIdx.x + kAreaAnyThreads - 1) / (unsigned)W + 1;
+  for (unsigned q = threadIdx.x; q < rows; q += kAreaAnyThreads) {
+    const long long Y = row0 + (long long)q;
+    ya[q] = (int)(Y * h / H);
+    yb[q] = (int)(((Y + 1) * h + H - 1) / H);
+  }
+  __syncthreads();
+  if (i0 + threadIdx.x >= n) return;
+  const unsigned X = at - r * W;
+  int x0, x1;
+  if (narrow) {
+    x0 = (int)(X * w / (unsigned)W);
+    x1 = (int)(((X + 1) * w + W - 1) / (unsigned)W);
+  } else {
+    x0 = (int)((long long)X * w / W);
+    x1 = (int)(((long long)(X + 1) * w + W - 1) / W);
+  }
+  const int ny = yb[r] - ya[r], nx = x1 - x0;
+  const float *p = x + ((size_t)blockIdx.y * h + ya[r]) * w + x0;
+  const float cnt = (float)ny * (float)nx;
+  float m;
+  if (cnt < 16777216.f) {
+    Sum acc{0.f, 0.f};
+    for (int y = 0; y < ny; y++, p += w) {
+      float row = 0.f;
+      for (int k = 0; k < nx; k++) row += __ldg(p + k);
+      acc.add(row);
+    }
+    m = area_divide(acc, cnt, 1.f / cnt);
+    if (!(fabsf(acc.s) <= FLT_MAX)) m = area_mean64(p - (size_t)ny * w, w, ny, nx);   // (as above)
+  } else {   // a count that FP32 does not hold
+    m = area_mean64(p, w, ny, nx);
+  }
+  out[(size_t)blockIdx.y * n + i0 + threadIdx.x] = m;
+}
+
 void launch_area(const float *x, int C, int h, int w, float *out, int H, int W, cudaStream_t s) {
+  // a window spans at most ceil(h / H) + 1 rows (ceil(h / H) when H divides h)
+  const int ny = (h + H - 1) / H + (h % H ? 1 : 0), nx = (w + W - 1) / W + (w % W ? 1 : 0);
+  if (C != 3 || ny > 5 || nx > 5) {
+    const int narrow = (long long)(W + 1LL) * w + W < (1LL << 32);
+    const unsigned ctas = (unsigned)(((long long)H * W + kAreaAnyThreads - 1) / kAreaAnyThreads);
+    area_any_kernel<<<dim3(ctas, C), kAreaAnyThreads, 0, s>>>(x, h, w, out, H, W, narrow);
+    return;
+  }
   const int gx = (W + kAreaThreads - 1) / kAreaThreads;
   int R = kAreaRows;   // rows per CTA, fewer where that leaves less than eight CTAs per SM
   while (R > 1 && (long long)gx * ((H + R - 1) / R) < 8 * 152) R /= 2;
   const int gy = (H + R - 1) / R;
   const dim3 grid(gx, gy < 65535 ? gy : 65535);
-  // a window spans at most ceil(h / H) + 1 rows (ceil(h / H) when H divides h)
-  const int ny = (h + H - 1) / H + (h % H ? 1 : 0), nx = (w + W - 1) / W + (w % W ? 1 : 0);
-  if (C == 3 && ny <= 3 && nx <= 3)
-    area_kernel<3><<<grid, kAreaThreads, 0, s>>>(x, C, h, w, out, H, W, R);
-  else if (C == 3 && ny <= 5 && nx <= 5)
-    area_kernel<5><<<grid, kAreaThreads, 0, s>>>(x, C, h, w, out, H, W, R);
+  if (ny <= 3 && nx <= 3)
+    area_kernel<3><<<grid, kAreaThreads, 0, s>>>(x, h, w, out, H, W, R);
   else
-    area_kernel<0><<<grid, kAreaThreads, 0, s>>>(x, C, h, w, out, H, W, R);
+    area_kernel<5><<<grid, kAreaThreads, 0, s>>>(x, h, w, out, H, W, R);
 }
 
 }  // namespace nst
