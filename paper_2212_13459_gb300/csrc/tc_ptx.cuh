@@ -160,13 +160,19 @@ __device__ __forceinline__ void tc_fence_before() {
 __device__ __forceinline__ void tc_fence_after() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
+// Instructions marked .aligned (and bar.sync, which is one) must be executed by all lanes of a warp
+// together: a warp that has come apart, in an epilogue that stores for some of its lanes, say, can
+// hang in them for good. The compiler does not bring it together for an asm statement, so each of
+// the wrappers does.
 __device__ __forceinline__ void tmem_alloc(uint32_t dst_smem, uint32_t ncols) {
+  __syncwarp();
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem),
                "r"(ncols)
                : "memory");
   asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
+  __syncwarp();
   asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols)
                : "memory");
 }
@@ -187,6 +193,7 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
 // 32 consecutive FP32 columns of this warp's 32 TMEM lanes (one row per thread)
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float *v) {
   uint32_t r[32];
+  __syncwarp();
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
       "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
@@ -207,6 +214,7 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float *v) {
 // v[4k] = (t/4, c), v[4k+1] = (t/4, c+1), v[4k+2] = (t/4+8, c), v[4k+3] = (t/4+8, c+1)
 __device__ __forceinline__ void tmem_ld16x256b_x4(uint32_t taddr, float *v) {
   uint32_t r[16];
+  __syncwarp();
   asm volatile(
       "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
       "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
@@ -232,6 +240,7 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
 }
 // barrier over `nthreads` threads (whole warps) on hardware barrier `id` (1..15)
 __device__ __forceinline__ void named_bar_sync(uint32_t id, uint32_t nthreads) {
+  __syncwarp();
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 
