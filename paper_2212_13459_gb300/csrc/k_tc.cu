@@ -680,7 +680,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 
 // ---- halo-reuse variant for the narrow layers ----------------------------------------------------
-// For the 64/128-channel layers the weights of one N slice (<= 160 KB) stay in shared memory for
+// For the layers with 64 output channels the weights (<= 144 KB) stay in shared memory for
 // the life of the CTA, and each 64-channel K-block loads ONE activation box of 18 rows x 10
 // pixels around a 16 x 8 output patch. The nine taps are nine descriptors into that box,
 // shifted by whole 128-byte pixel rows (the patch's 8-pixel rows are 1,280 bytes apart); the
@@ -717,8 +717,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                         const TcGeom tg) {
   using Cfg = HaloCfg<BN, KB, P2KB, NT>;
   constexpr int STAGES = Cfg::STAGES;
-  // four accumulators in TMEM (512 columns at N = 128): the tiles are short, and more tiles in
-  // flight keep the tensor pipe fed while the epilogue drains
+  // four accumulators in TMEM: the tiles are short, and more tiles in flight keep the tensor pipe
+  // fed while the epilogue drains
   constexpr int NACC = 4;
   constexpr uint32_t TMEM_COLS = NACC * BN;
   constexpr uint32_t IDESC = make_idesc(BN);
@@ -903,10 +903,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int q = warp & 3;
     const int half = (warp - 2) >> 2;
     const int row = q * 32 + lane;
-    // pooled forward (BN = 64: one 32-channel chunk per warp): the bias pairs this thread
-    // applies on every tile, loaded once
+    // pooled forward (one 32-channel chunk per warp): the bias pairs this thread applies on
+    // every tile, loaded once
+    static_assert(BN == 64, "one 32-channel chunk per epilogue warp");
     float2 pbias[4] = {};
-    if (a.pool_out && BN == 64)
+    if (a.pool_out)
 #pragma unroll
       for (int k = 0; k < 4; k++)
         pbias[k] = *reinterpret_cast<const float2 *>(a.bias + nt * BN + half * (BN / 2) + 8 * k +
@@ -947,19 +948,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         // pooled forward: two 16-lane reads of the 16x256b layout (pixel-row pairs 4q, 4q + 2)
 #pragma unroll 1
         for (int c = half * (BN / 2); c < (half + 1) * (BN / 2); c += 32) {
-          float2 pb[4];   // (other widths: this chunk's bias pairs)
-          const float2 *bp = pbias;
-          if constexpr (BN != 64) {
-#pragma unroll
-            for (int k = 0; k < 4; k++)
-              pb[k] = *reinterpret_cast<const float2 *>(a.bias + nt * BN + c + 8 * k +
-                                                        2 * (lane & 3));
-            bp = pb;
-          }
 #pragma unroll
           for (int grp = 0; grp < 2; grp++)
             halo_pool16(a, g, b, oy + 4 * q + 2 * grp, ox, nt * BN + c,
-                        tbase + ((uint32_t)(16 * grp) << 16) + (uint32_t)c, bp);
+                        tbase + ((uint32_t)(16 * grp) << 16) + (uint32_t)c, pbias);
         }
       } else {
 #pragma unroll 1
@@ -1620,8 +1612,7 @@ bool halo_shape(const ConvArgs &a, int *BN, int *KB, int *P2KB, int *NT) {
   // N = 64, at 3024 x 4032, although the 144 KB of resident weights leave three stages)
   if (a.cin == 128 && a.cout == 64 && a.k2 == 0) { *BN = 64; *NT = 1; return true; }
   // (conv2_2, 128 -> 128, runs faster on the pixels-as-N kernel with 256-wide MMAs than here
-  // with two 64-wide N slices; conv2_1, 64 -> 128, is faster here: 0.76 against 0.83 ms at
-  // 3024 x 4032, where the pixels-as-N kernel streams a 16 KB weight box with every K-block)
+  // with two 64-wide N slices)
   return false;
 }
 
@@ -1649,7 +1640,6 @@ cudaError_t launch_conv_tc_halo(const ConvArgs &a, int BN, int KB, int P2KB, int
     if (mask_smem) return launch_halo<64, 1, 1, 1, true>(mA, mB, mA2, mB2, a, s);
     return launch_halo<64, 1, 1, 1>(mA, mB, mA2, mB2, a, s);
   }
-  if (BN == 128 && KB == 1 && P2KB == 0 && NT == 1) return launch_halo<128, 1, 0, 1>(mA, mB, mA2, mB2, a, s);
   if (BN == 64 && KB == 2 && P2KB == 0 && NT == 1) return launch_halo<64, 2, 0, 1>(mA, mB, mA2, mB2, a, s);
   return cudaErrorInvalidValue;
 }
