@@ -590,7 +590,9 @@ cudaError_t launch_conv11_fwd_tc(const float *img, int H, int W, const float *w1
   if (npix <= 0) return cudaSuccess;
   if (reinterpret_cast<uintptr_t>(stage_buf) % 16) return cudaErrorInvalidValue;
   const int sgrid = (int)std::min<long long>((npix + 255) / 256, 32LL * tc_num_sms());
-  cudaError_t le = launch_pdl(npix * 28e-6 / 5 <= kEarlyUs, conv11_stage_kernel, sgrid, 256, 0, s, img, H, W, geom, B, Hb, Wb,
+  // (per pixel: 12 bytes of the image in, 16 of the staged pixel out)
+  cudaError_t le = launch_pdl(traffic_us(28.0 * npix) <= kEarlyUs, conv11_stage_kernel, sgrid, 256,
+                              0, s, img, H, W, geom, B, Hb, Wb,
                               reinterpret_cast<uint4 *>(stage_buf), check_finite ? err : nullptr);
   if (le != cudaSuccess) return le;
   EncodeTiledFn enc = reinterpret_cast<EncodeTiledFn>(tc_encode_tiled_fn());
@@ -619,8 +621,10 @@ cudaError_t launch_conv11_fwd_tc(const float *img, int H, int W, const float *w1
   // list puts them first), a split that depends on the owned patches alone
   const int grid = gram_part ? 2 * tc_num_sms()
                              : (int)std::min<long long>(ntiles, 2LL * tc_num_sms());
-  le = launch_pdl(ntiles * (128 * 144e-6 / 5) <= kEarlyUs, conv11_fwd_tc_kernel, grid, kFwdThreads, kFwdSmem, s, m, mo, w11, bias, geom, B, Hb,
-                  Wb, tiles_x, tiles_y, patches, (int)ntiles, gram_part, err);
+  // (128 pixels per tile: 16 bytes of the staged image in, 128 of the activation out)
+  const bool early = traffic_us(128.0 * 144 * ntiles) <= kEarlyUs;
+  le = launch_pdl(early, conv11_fwd_tc_kernel, grid, kFwdThreads, kFwdSmem, s, m, mo, w11, bias,
+                  geom, B, Hb, Wb, tiles_x, tiles_y, patches, (int)ntiles, gram_part, err);
   if (gram_runs) *gram_runs = gram_part ? grid : 0;
   return le;
 }
@@ -653,8 +657,10 @@ cudaError_t launch_conv11_dgrad_tc(const __nv_bfloat16 *g, const float *w11,
   const int tiles_y = (max_inner_h + kDgOutH - 1) / kDgOutH;
   const long long ntiles = (long long)B * tiles_x * tiles_y;
   const int grid = (int)std::min<long long>(ntiles, 2LL * tc_num_sms());
-  return launch_pdl(ntiles * (192 * 140e-6 / 5) <= kEarlyUs, conv11_dgrad_tc_kernel, grid, kDgThreads, kDgSmem, s, m, w11, geom, inner, B, tiles_x,
-                    tiles_y, grad, H, W, err);
+  // (192 box pixels per tile: 128 bytes of the gradient in, 12 out)
+  const bool early = traffic_us(192.0 * 140 * ntiles) <= kEarlyUs;
+  return launch_pdl(early, conv11_dgrad_tc_kernel, grid, kDgThreads, kDgSmem, s, m, w11, geom,
+                    inner, B, tiles_x, tiles_y, grad, H, W, err);
 }
 
 }  // namespace nst

@@ -593,8 +593,8 @@ __device__ __forceinline__ int keys_taps(int i, float s, float *wt) {
 // Here a lane keeps the column weights of its four outputs for all rows and channels, the row
 // weights serve three channels, and the rows are combined once per source column (not once per
 // output and tap) into shared memory, from where every output takes its four columns:
-// 64 us, with the L1 74 % busy. Lane l's outputs are columns l, l + 32, ... of the strip, so loads and stores are
-// whole lines at any alignment. The same operations in the same order per output: the same bits.
+// 64 us, with the L1 74 % busy. Lane l's outputs are columns l, l + 32, ... of the strip, so loads
+// and stores are whole lines at any alignment. The same operations in the same order per output: the same bits.
 // The rows are the CTA's (uniform base addresses, one 32-bit column offset per load).
 constexpr int kBicX = 128, kBicSpan = 136;   // a strip reads at most kBicX + 1 + 3 source columns
 constexpr int kBicWarps = 4;

@@ -689,11 +689,13 @@ void launch_unpool_idx(const __nv_bfloat16 *gp, const unsigned char *idx, __nv_b
     const long long per = (long long)max_rect_px * C / 8;
     int nx = (int)std::min<long long>((per + 255) / 256, std::max(1, 152 * 32 / B));
     dim3 grid(nx, B);
-    launch_pdl(per * B * 84e-6 / 5 <= kEarlyUs, unpool_idx_kernel, grid, 256, 0, s, gp, idx, g, B, Hp, Wp, C, geom, level_out, rects);
+    // (per 8 channels of a pooled pixel: 20 bytes in, 64 out)
+    launch_pdl(traffic_us(84.0 * per * B) <= kEarlyUs, unpool_idx_kernel, grid, 256, 0, s, gp, idx,
+               g, B, Hp, Wp, C, geom, level_out, rects);
     return;
   }
-  launch_pdl(true, unpool_idx_kernel, ew_grid((long long)B * Hp * Wp * C / 8), 256, 0, s, gp, idx, g, B, Hp,
-             Wp, C, geom, level_out, (const int4 *)nullptr);
+  launch_pdl(true, unpool_idx_kernel, ew_grid((long long)B * Hp * Wp * C / 8), 256, 0, s, gp, idx,
+             g, B, Hp, Wp, C, geom, level_out, (const int4 *)nullptr);
 }
 template void launch_pool<float>(const float *, float *, int, int, int, int, const BlockGeom *,
                                  int, cudaStream_t);
@@ -906,8 +908,9 @@ __global__ void __launch_bounds__(256) gram_reduce_kernel(const float *__restric
   }
 }
 
-// Up to one whole block per SM (152) runs as quarters: at 120 blocks (5,000 pixels x 192) 19.3 against
-// 25.4 us in FP32 and 21.3 against 29.5 in BF16; at 237 (20,000 x 128) 29.8 against 27.4 and 35.5 against 31.5.
+// Up to one whole block per SM (152) runs as quarters: at 120 blocks (5,000 pixels x 192) 19.3
+// against 25.4 us in FP32 and 21.3 against 29.5 in BF16; at 237 (20,000 x 128) 29.8 against 27.4 and
+// 35.5 against 31.5.
 constexpr int kGramQuarters = 152;
 template <typename T>
 static void launch_gram_blocks(const T *V, int Hb, int Wb, int C, const OwnRect *own,

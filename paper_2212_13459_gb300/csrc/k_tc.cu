@@ -1460,7 +1460,8 @@ cudaError_t launch_bn(const CUtensorMap &A, const CUtensorMap &B, const CUtensor
   // (us of a 64-deep K-block of one tile, see the costs where the tiles are split)
   const double us = (BN == 256 ? 0.33 : BN == 128 ? 0.19 : 0.155) * (tg.kb_main + tg.kb2) *
                     ((tg.total + g_num_sms - 1) / g_num_sms);
-  return launch_pdl(us <= kEarlyUs, conv_tc_kernel<BN, STAGES, KPS>, grid, kThreads, smem, s, A, B, A2, B2, Bp, B2p, a, tg);
+  return launch_pdl(us <= kEarlyUs, conv_tc_kernel<BN, STAGES, KPS>, grid, kThreads, smem, s, A, B,
+                    A2, B2, Bp, B2p, a, tg);
 }
 
 template <int STAGES>
@@ -1478,7 +1479,8 @@ cudaError_t launch_swap(const CUtensorMap &A, const CUtensorMap &B, const CUtens
   }
   const int grid = std::min(tg.total, g_num_sms);
   const double us = 0.4 * (tg.kb_main + tg.kb2) * ((tg.total + g_num_sms - 1) / g_num_sms);
-  return launch_pdl(us <= kEarlyUs, conv_tc_swap_kernel<STAGES>, grid, kThreads, smem, s, A, B, A2, B2, a, tg);
+  return launch_pdl(us <= kEarlyUs, conv_tc_swap_kernel<STAGES>, grid, kThreads, smem, s, A, B, A2,
+                    B2, a, tg);
 }
 
 // Output patch of at most `rows` pixels (the tile's M or N) covering n rectangles h[i] x w[i]
@@ -1540,8 +1542,8 @@ cudaError_t launch_halo(const CUtensorMap &A, const CUtensorMap &B, const CUtens
   int grid = std::min(tg.total * NT, g_num_sms);
   grid = std::max(NT, grid / NT * NT);
   const double us = 1.25 * KB * ((tg.total + g_num_sms - 1) / g_num_sms);
-  return launch_pdl(us <= kEarlyUs, conv_tc_halo_kernel<BN, KB, P2KB, NT, MASK_SMEM>, grid, kThreads, smem, s, A, B,
-                    A2, B2, a, tg);
+  return launch_pdl(us <= kEarlyUs, conv_tc_halo_kernel<BN, KB, P2KB, NT, MASK_SMEM>, grid,
+                    kThreads, smem, s, A, B, A2, B2, a, tg);
 }
 
 // 4-D map of an activation with the halo box (64 ch, 10 px, 18 rows, 1)
@@ -1598,7 +1600,8 @@ cudaError_t launch_swap_halo(const ConvArgs &a, cudaStream_t s) {
   if (tg.total <= 0) return cudaSuccess;
   const int grid = std::min(tg.total, g_num_sms);
   const double us = 3.6 * ((tg.total + g_num_sms - 1) / g_num_sms);
-  return launch_pdl(us <= kEarlyUs, conv_tc_swap_halo_kernel, grid, kThreads, kSHSmem, s, mA, mW, a, tg);
+  return launch_pdl(us <= kEarlyUs, conv_tc_swap_halo_kernel, grid, kThreads, kSHSmem, s, mA, mW, a,
+                    tg);
 }
 
 // (cin, cout, k2) of the narrow layers -> N slice width and counts; false if not a halo layer

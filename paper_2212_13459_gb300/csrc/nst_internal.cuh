@@ -34,6 +34,8 @@ __device__ __forceinline__ void pdl_begin() {
 // (32.7 -> 33.9 ms; no single kernel accounts for it), so a launch expected to take over kEarlyUs
 // starts normally.
 constexpr double kEarlyUs = 100.0;
+// microseconds of a launch bound by its memory traffic, at 5 TB/s
+inline double traffic_us(double bytes) { return bytes / 5e6; }
 template <typename... P, typename... A>
 inline cudaError_t launch_pdl(bool early, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
                               cudaStream_t s, A &&...args) {
