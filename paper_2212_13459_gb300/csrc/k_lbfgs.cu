@@ -239,7 +239,9 @@ void launch_lbfgs_dots(const float *g, const float *g_prev, const float *S, floa
 // global memory took 1,496 us at k = 100 and 58 us at k = 10; this takes 47 and 17 us (all
 // cold, under the profiler).
 constexpr int kSolveThreads = 512;
-constexpr int kSolveCtas = 16;   // (all but one only where the dots are made again)
+// All but one only where the dots are made again; 16 take 0.5 us longer where they are not (1,000
+// elements, 10 pairs: 32.0 -> 33.0 us a step, 31.9 with 4)
+constexpr int kSolveCtas = 4;
 constexpr int kSolveParts = kSolveThreads / kMaxHistory;          // threads per row of Y^T Y
 constexpr int kSolveRow = kMaxHistory / kSolveParts;              // its elements each holds
 static size_t solve_smem(int m) { return (size_t)m * (m | 1) * sizeof(double); }
@@ -320,8 +322,16 @@ __global__ void __launch_bounds__(kSolveThreads)
   __shared__ int sl[kMaxHistory], old[kMaxHistory];
   const int tid = threadIdx.x, lane = tid & 31;
   pdl_begin();
-  if (c->beyond) {   // (unchanged until every CTA has read it)
+  // (one round of loads; c->beyond is unchanged until every CTA has read it, and the CTAs that leave
+  // at once use nothing else of this)
+  const unsigned beyond = c->beyond;
+  const int count0 = c->count, sp = c->spare, ld = m + 1;
+  const int slot = tid < kMaxHistory ? c->order[tid] : 0;   // newest first
+  double ys = c->dots[2], yy = c->dots[3];
+  if (beyond) {
     if (!lbfgs_dots_again(c, g, S, Y, stride, n, first, partials)) return;
+    ys = c->dots[2];
+    yy = c->dots[3];
   } else if (blockIdx.x) {
     return;
   }
@@ -333,14 +343,12 @@ __global__ void __launch_bounds__(kSolveThreads)
     }
     return;
   }
-  const int count0 = c->count, sp = c->spare, ld = m + 1;
-  const double ys = c->dots[2], yy = c->dots[3];
   // the candidate becomes the newest pair (dropping the oldest of m) or is left out
   const bool take = ys > eps;
   const int keep = take ? (count0 < m ? count0 : m - 1) : count0;   // older pairs kept
   const int k = keep + (take ? 1 : 0);
   const double gamma = take ? ys / yy : (k > 0 ? c->gamma : 1.0);
-  if (tid < kMaxHistory) old[tid] = c->order[tid];   // newest first
+  if (tid < kMaxHistory) old[tid] = slot;
   __syncthreads();
   if (tid < k) {
     // pair tid (oldest first): its position in the fused pass, its slot, its four dots
