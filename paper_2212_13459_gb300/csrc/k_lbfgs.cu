@@ -726,15 +726,14 @@ void launch_bicubic(const float *x, int C, int h, int w, float *out, int H, int 
 // in compensated FP32 and divided with a remainder step: the quotient is within 2^-46 of the
 // exact one before it is rounded to FP32; with windows of at most 3 x 3 (a factor up to 2) or
 // 5 x 5 their loads are issued together (area_kernel). 19 us with the source in L2.
-// the mean of ny x nx elements from p on, summed in FP64
-__device__ __noinline__ float area_mean64(const float *p, int w, int ny, int nx) {
+__device__ __noinline__ float area_mean64(const float *src, int w, int y0, int y1, int x0, int x1) {
   double acc = 0.0;
-  for (int y = 0; y < ny; y++, p += w) {
+  for (int y = y0; y < y1; y++) {
     float row = 0.f;
-    for (int k = 0; k < nx; k++) row += p[k];
+    for (int xx = x0; xx < x1; xx++) row += src[(size_t)y * w + xx];
     acc += (double)row;
   }
-  return (float)(acc / ((double)ny * (double)nx));
+  return (float)(acc / ((double)(y1 - y0) * (double)(x1 - x0)));
 }
 
 // sum / cnt rounded once: q is within 2 ulp, its remainder exact (no contraction into q's product)
@@ -789,7 +788,7 @@ __global__ void __launch_bounds__(kAreaThreads) area_kernel(const float *__restr
         }
         float m = area_divide(acc, cnt, inv);
         if (!(fabsf(acc.s) <= FLT_MAX))   // an infinite or overflowing sum
-          m = area_mean64(x + ((size_t)c * h + y0) * w + x0, w, y1 - y0, x1 - x0);
+          m = area_mean64(x + (size_t)c * h * w, w, y0, y1, x0, x1);
         o[(size_t)c * H * W] = m;
       }
     }
@@ -841,9 +840,10 @@ __global__ void __launch_bounds__(kAreaAnyThreads, 12) area_any_kernel(const flo
       acc.add(row);
     }
     m = area_divide(acc, cnt, 1.f / cnt);
-    if (!(fabsf(acc.s) <= FLT_MAX)) m = area_mean64(p - (size_t)ny * w, w, ny, nx);   // (as above)
+    if (!(fabsf(acc.s) <= FLT_MAX))   // (as above)
+      m = area_mean64(p - (size_t)ny * w, w, 0, ny, 0, nx);
   } else {   // a count that FP32 does not hold
-    m = area_mean64(p, w, ny, nx);
+    m = area_mean64(p, w, 0, ny, 0, nx);
   }
   out[(size_t)blockIdx.y * n + i0 + threadIdx.x] = m;
 }
