@@ -225,9 +225,9 @@ nst_status nst_conv3x3(int dtype, int engine, int B, int H, int W, int cin, int 
 /* ---- single-layer Gram statistics (unit-test entry of the Gram engine) ------------------------
  * G = sum_p V_p V_p^T over the npix rows of V ([npix][C], row-major, NHWC features of one layer),
  * the un-normalised Gram matrix of Eq. 4 (divide by n_p for G^L). FP32 partial sums over pixel
- * chunks, reduced in FP64 in a fixed order (deterministic). dtype: NST_PREC_FP32 or
- * NST_PREC_BF16 elements; C a multiple of 64, 64 <= C <= 512; 1 <= npix < 2^31. G_dev: C*C
- * doubles in device memory, overwritten. Scratch for the partial sums (at most 1,216 blocks of
+ * chunks, reduced in a fixed order (deterministic) in compensated FP32 (48 bits; in FP64 where a
+ * sum leaves FP32's range). dtype: NST_PREC_FP32 or NST_PREC_BF16 elements; C a multiple of 64,
+ * 64 <= C <= 512; 1 <= npix < 2^31. G_dev: C*C doubles in device memory, overwritten. Scratch for the partial sums (at most 1,216 blocks of
  * 64 x 64 floats, 19 MiB) is allocated stream-ordered and released on `stream`. Bad arguments
  * (including C outside 64..512 or not a multiple of 64) give NST_ERR_INVALID_ARG. */
 nst_status nst_gram(int dtype, const void *V_dev, long long npix, int C, double *G_dev,
