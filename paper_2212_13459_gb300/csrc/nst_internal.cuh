@@ -18,8 +18,9 @@ namespace nst {
 // The kernels of an evaluation and of an L-BFGS step are launched so that a kernel's CTAs may
 // start, and set up barriers, tensor memory and shared memory, while its predecessor in the stream
 // is finishing. Rule for every kernel launched with launch_pdl: each thread calls pdl_begin()
-// before its first access to memory that another kernel of the stream writes or reads (weights,
-// patch lists and block geometry are written once, synchronously, and may be read before). It
+// before its first access to memory that another kernel of the stream writes or reads (a context's
+// weights, patch lists and block geometry are written once, synchronously, and may be read before;
+// a single layer's weights, bias and geometry are the caller's and may not). It
 // waits until the predecessor has completed with its writes visible, so completion stays
 // transitive along the stream, and then lets the successor's CTAs start. What the stream writes is
 // read through plain pointers there, not const __restrict__ ones or __ldg: those loads are taken
